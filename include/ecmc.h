@@ -74,7 +74,9 @@ extern "C" {
 /* Candidate geometry: ECMC_PREC_FP64 = every candidate tested in FP64;
  * ECMC_PREC_FP32_GEOM (default) = candidates screened in FP32 cell-relative
  * coordinates with rigorous error bounds, the contact decided in FP64.  Both
- * give bit-identical trajectories. */
+ * give bit-identical trajectories.  Axis chains in cells small enough for
+ * shared memory find a disk's few candidates once per colour phase and test
+ * them in FP64 under either value. */
 #define ECMC_PARAM_PRECISION 3
 /* Replica number: second word of the Philox key (seed, replica); an integer
  * in [0, 9e15], so that the double passed to set_param holds it exactly. */
@@ -97,12 +99,12 @@ extern "C" {
 #define ECMC_PARAM_WARPS_PER_BLOCK 11
 /* 1 = capture each sweep in a CUDA graph and replay it (default 1). */
 #define ECMC_PARAM_USE_GRAPH 12
-/* Where the chain kernel keeps the cell frames: 0 = shared memory, 1 = FP32
- * screening data in shared memory and FP64 coordinates in global memory,
- * 2 = global memory (cells too large for shared memory), -1 = automatic
- * (default).  The persistent sweep kernel uses 0 or 1 (automatic: 0; with 1
- * its FP64 coordinates live in a per-warp scratch area).  Changes only the
- * speed, never the result. */
+/* Where the chain kernel keeps the cell frames: 0 = shared memory, 1 = part of
+ * them in global memory (axis chains: the disks' candidate lists, in a
+ * per-warp scratch area; isotropic chains, per-phase launches: the FP64
+ * coordinates), 2 = global memory (cells too large for shared memory), -1 =
+ * automatic (default).  The persistent sweep kernel uses 0 or 1.  Changes only
+ * the speed, never the result. */
 #define ECMC_PARAM_FRAME_MODE 13
 /* 1 = replay the legs of a chain that rattles between two reflectors
  * (frozen disks or walls) once its position after a reflection repeats bit
@@ -125,7 +127,8 @@ extern "C" {
  * that faults nothing; default 0). */
 #define ECMC_PARAM_WAIT_TEST 17
 /* Read-only: kernel launches per sweep of the current configuration (5 with
- * the persistent kernel, 12 with per-phase launches). */
+ * the persistent kernel; with per-phase launches 8 for axis chains whose cells
+ * fit in shared memory, which build their frames themselves, and 12 else). */
 #define ECMC_PARAM_KERNELS_PER_SWEEP 18
 /* Start lists (Sec. 3.4 step 5): ECMC_LIST_WITH_REPL (default), every start
  * disk drawn independently among the members (the paper's correct rule);
@@ -172,7 +175,7 @@ typedef struct {
   int64_t lifts;       /* contacts with an active disk (budget passed on)       */
   int64_t frozen_hits; /* contacts with a frozen disk (chain reflected)         */
   int64_t wall_hits;   /* reflections at a cell wall (not counted as events)    */
-  int64_t fp64_evals;  /* candidates evaluated in FP64 (FP32_GEOM screening)    */
+  int64_t fp64_evals;  /* candidates evaluated in FP64                          */
   double sum_b;        /* sum over contacts of the separation along d           */
   double sum_disp;     /* sum over chains of the displacement budget ell        */
   int64_t replayed_legs; /* reflection legs (frozen disk or wall) of a chain that

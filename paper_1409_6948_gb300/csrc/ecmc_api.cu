@@ -66,6 +66,8 @@ struct ecmc_ctx {
   int persist_param = 1; // 1 = one persistent launch per sweep when the frames fit
   int persistent = 0;    // in use
   int fused_blocks = 0;  // grid of the persistent sweep kernel
+  int axis = 0;          // axis chains through their static candidates (ecmc_axis.cuh)
+  AxisShape axis_shape;
   double wait_ms = 5000.0;
   int n_sm = 0;
   std::vector<int2> chunks;
@@ -204,27 +206,138 @@ int choose_tpc(ecmc_ctx* h, int fmode) {
   return 32;
 }
 
+// Shared memory of the axis-chain kernel with tpc lanes per cell: the usual
+// sizes cover the mean numbers of members and objects plus a few standard
+// deviations of a dilute gas (dense fluids vary less); cells beyond them are
+// worked on alone.
+AxisShape axis_shape_for(ecmc_ctx* h, int tpc) {
+  AxisShape s;
+  std::memset(&s, 0, sizeof(s));
+  s.cpw = 32 / tpc;
+  double co = 0.0, mp = 0.0;
+  for (const Geom& g : h->geo) {
+    s.nbin = g.nbin > s.nbin ? g.nbin : s.nbin;
+    s.co_h = g.cap_obj > s.co_h ? g.cap_obj : s.co_h;
+    const double rho = (double)g.N / (g.L * g.L);
+    const double mo = rho * (g.w + 2.0 * g.sigma) * (g.h + 2.0 * g.sigma);
+    const double mm = s.cpw * rho * g.w * g.h;
+    co = std::fmax(co, mo + 2.5 * std::sqrt(mo) + 2.0);
+    mp = std::fmax(mp, mm + 3.0 * std::sqrt(mm) + 2.0);
+  }
+  s.mp_h = h->b.cap;
+  s.co_s = co < s.co_h ? (int)co + 1 : s.co_h;
+  s.mp_s = mp < (double)s.cpw * s.mp_h ? (int)mp + 1 : s.cpw * s.mp_h;
+  if (s.cpw == 1) {
+    s.co_s = s.co_h;
+    s.mp_s = s.mp_h;
+  }
+  return s;
+}
+
+// Lanes per cell of the axis-chain kernel: the fewest, from 8 up, that leave
+// eight warps per SM something to do in a colour phase.  Measured on GB300, us
+// per sweep with 8 / 16 / 32 lanes: 697 / 810 / 1101 at N = 2^20, 240^2 cells;
+// 342 / 270 / 298 at N = 2^18, 120^2 cells; 960 / 558 / 310 at N = 2^16, 32^2
+// cells.  Fewer lanes lost everywhere (780 with 4 at N = 2^20).
+int choose_axis_tpc(ecmc_ctx* h) {
+  if (h->tpc_param) return h->tpc_param;
+  for (int t = 8; t < 32; t *= 2)
+    if ((int64_t)h->b.A_total * t / 32 >= 8 * h->n_sm &&
+        axis_smem(axis_shape_for(h, t), 0) <= 28 * 1024)
+      return t;
+  return 32;
+}
+
+constexpr size_t kSmemLimit = 232448;  // opt-in shared memory per block on sm_103
+
+// Frame placement of the per-phase kernels: whole frames in shared memory when
+// every group of the phase fits at once, else only the light part (FP64 in
+// global memory); frames too large for shared memory are used in place in
+// global memory.
+int auto_fmode(ecmc_ctx* h) {
+  if (h->fmode_param >= 0) return h->fmode_param;
+  const RecLayout l0 = layout_for(h, choose_tpc(h, 0));
+  const size_t groups = (size_t)(h->b.A_total + l0.cpw - 1) / l0.cpw;
+  const size_t one = phase_smem_bytes(l0, 1, 0);
+  return one <= kSmemLimit && groups * one <= (size_t)h->n_sm * kSmemLimit * 9 / 10 ? 0 : 1;
+}
+
+// Room for `need` bytes of frame records or list scratch.
+int need_records(ecmc_ctx* h, size_t need) {
+  if (need <= h->records_cap) return ECMC_OK;
+  cudaFree(h->b.records);
+  h->b.records = nullptr;
+  h->records_cap = 0;
+  CK(cudaMalloc(&h->b.records, need));
+  h->records_cap = need;
+  return ECMC_OK;
+}
+
+// Axis chains: the kernel of ecmc_axis.cuh wherever a cell fits in its shared
+// memory, in one persistent launch per sweep or one launch per phase.  *used
+// says whether it does.
+int axis_layout(ecmc_ctx* h, int* used) {
+  *used = 0;
+  h->axis = 0;
+  if (chain_kind(h->b) == 1 || h->fmode_param == 2) return ECMC_OK;
+  if (h->tpc_param && h->tpc_param != 32 &&
+      phase_smem_bytes(layout_for(h, h->tpc_param), 1, auto_fmode(h)) > kSmemLimit)
+    return ECMC_OK;  // refused by compute_layout: frames too large for so few lanes
+  const int tpc = choose_axis_tpc(h);
+  const AxisShape s = axis_shape_for(h, tpc);
+  if (s.co_h > kAxisMaxObjects) return ECMC_OK;
+  const int n_groups = (h->b.A_total + s.cpw - 1) / s.cpw;
+  // candidate lists in shared memory, unless they leave room for fewer than
+  // four warps per SM, or keep groups of a phase waiting that registers (16
+  // warps per SM) would admit: at N = 2^22, 484^2 cells, 8 lanes, 2608 us per
+  // sweep against 2684; with all groups resident the lists in L1 cost 3-15 %
+  int fm = h->fmode_param;
+  if (fm < 0) {
+    const int w0 = (int)(kSmemLimit / axis_smem(s, 0));
+    const int w1 = (int)(kSmemLimit / axis_smem(s, 1));
+    fm = w0 < 4 || (w0 < 16 && w1 > w0 && n_groups > w0 * h->n_sm) ? 1 : 0;
+  }
+  const size_t sm = axis_smem(s, fm);
+  if (sm > kSmemLimit / 2) return ECMC_OK;
+  int per_sm = 0;
+  if (configure_axis(s, tpc, fm, h->b.reject, &per_sm)) {
+    cudaGetLastError();
+    return ECMC_OK;
+  }
+  const int n_items = 4 * n_groups;
+  h->persistent = h->persist_param;
+  h->fused_blocks = h->persistent ? (per_sm * h->n_sm < n_items ? per_sm * h->n_sm : n_items)
+                                  : n_groups;
+  if (fm == 1) {
+    const int rc = need_records(h, (size_t)h->fused_blocks * axis_scratch(s));
+    if (rc) return rc;
+  }
+  h->axis = 1;
+  h->axis_shape = s;
+  h->tpc = tpc;
+  h->fmode = fm;
+  h->b.fmode = fm;
+  h->warps = 1;
+  *used = 1;
+  return ECMC_OK;
+}
+
 int compute_layout(ecmc_ctx* h) {
   for (Geom& g : h->geo) set_strip_bins(g, h->strip_w);
-  const size_t limit = 232448;  // opt-in shared memory per block on sm_103
+  const size_t limit = kSmemLimit;
   if (h->n_sm == 0) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (h->n_sm <= 0) h->n_sm = 1;
   }
-  // frame placement: whole frames in shared memory when every group of the
-  // phase fits at once, else only the light part (FP64 in global memory);
-  // frames too large for shared memory are used in place in global memory
-  int fmode = h->fmode_param;
-  if (fmode < 0) {
-    const int t0 = choose_tpc(h, 0);
-    const RecLayout l0 = layout_for(h, t0);
-    const size_t groups = (size_t)(h->b.A_total + l0.cpw - 1) / l0.cpw;
-    const size_t total = groups * phase_smem_bytes(l0, 1, 0);
-    fmode = (phase_smem_bytes(l0, 1, 0) <= limit &&
-             total <= (size_t)h->n_sm * limit * 9 / 10) ? 0 : 1;
-  }
+  h->persistent = 0;
+  h->fused_blocks = 0;
+  int used = 0;
+  const int rc_axis = axis_layout(h, &used);
+  if (rc_axis) return rc_axis;
+  if (used) return upload_geometry(h);
+  int fmode = auto_fmode(h);
   h->tpc = choose_tpc(h, fmode);
   h->lay = layout_for(h, h->tpc);
   if (fmode < 2 && phase_smem_bytes(h->lay, 1, fmode) > limit) {
@@ -245,13 +358,8 @@ int compute_layout(ecmc_ctx* h) {
   if (w < 1) w = 1;
   h->warps = w;
   const int n_groups = (h->b.A_total + h->lay.cpw - 1) / h->lay.cpw;
-  const size_t need = (size_t)n_groups * h->lay.bytes;
-  if (need > h->records_cap) {
-    if (h->b.records) cudaFree(h->b.records);
-    h->b.records = nullptr;
-    CK(cudaMalloc(&h->b.records, need));
-    h->records_cap = need;
-  }
+  const int rc_rec = need_records(h, (size_t)n_groups * h->lay.bytes);
+  if (rc_rec) return rc_rec;
   if (h->b.gtouch) cudaFree(h->b.gtouch);
   h->b.gtouch = nullptr;
   if (fmode == 2)
@@ -267,31 +375,17 @@ int compute_layout(ecmc_ctx* h) {
       configure_phase(h->lay, h->tpc, h->warps, fmode))
     return fail(ECMC_ERR_CUDA, "kernel configuration failed: %s",
                 cudaGetErrorString(cudaGetLastError()));
-  // one persistent launch per sweep when a warp's frames, histories and
-  // builder scratch fit in shared memory at least twice per SM
-  h->persistent = 0;
-  h->fused_blocks = 0;
-  // the persistent kernel keeps its frames in shared memory (frame mode 0)
-  // unless mode 1 is asked for: FP64 coordinates in a per-warp scratch area of
-  // global memory, more warps per SM (measured at N = 1M, eta = 0.72: 1.64
-  // against 1.58 * 10^9 events/s); isotropic chains use mode 0
-  const int fm = (h->fmode_param == 1 && chain_kind(h->b) == 0) ? 1 : 0;
-  if (h->persist_param && fmode < 2 && fused_smem_bytes(h->lay, fm) <= limit / 2) {
+  // isotropic chains: one persistent launch per sweep when a warp's frames
+  // and builder scratch fit in shared memory at least twice per SM
+  if (chain_kind(h->b) == 1 && h->persist_param && fmode < 2 &&
+      fused_smem_bytes(h->lay) <= limit / 2) {
     int per_sm = 0;
-    if (configure_fused(h->lay, h->tpc, fm, chain_kind(h->b), &per_sm) == 0) {
+    if (configure_fused(h->lay, h->tpc, &per_sm) == 0) {
       const int n_items = 4 * n_groups;
-      const int grid = per_sm * h->n_sm < n_items ? per_sm * h->n_sm : n_items;
-      const size_t scratch = (size_t)grid * fused_scratch_bytes(h->lay);
-      if (scratch > h->records_cap) {
-        cudaFree(h->b.records);
-        h->b.records = nullptr;
-        CK(cudaMalloc(&h->b.records, scratch));
-        h->records_cap = scratch;
-      }
-      h->fused_blocks = grid;
+      h->fused_blocks = per_sm * h->n_sm < n_items ? per_sm * h->n_sm : n_items;
       h->persistent = 1;
-      h->fmode = fm;
-      h->b.fmode = fm;
+      h->fmode = 0;
+      h->b.fmode = 0;
     } else {
       cudaGetLastError();
     }
@@ -363,8 +457,10 @@ int enqueue_sweep(ecmc_ctx* h) {
   if (h->persistent) {
     {
       Timed tm(h, TC_PHASE);
-      if (launch_fused(h->b, h->lay, h->tpc, h->fused_blocks, h->record_chains, h->precision,
-                       h->stream))
+      if (h->axis ? launch_axis(h->b, h->axis_shape, h->tpc, h->fused_blocks, -1,
+                                h->record_chains, h->stream)
+                  : launch_fused(h->b, h->lay, h->tpc, h->fused_blocks, h->record_chains,
+                                 h->precision, h->stream))
         return fail(ECMC_ERR_CUDA, "sweep kernel launch failed: %s",
                     cudaGetErrorString(cudaGetLastError()));
     }
@@ -376,14 +472,16 @@ int enqueue_sweep(ecmc_ctx* h) {
     return ECMC_OK;
   }
   for (int ci = 0; ci < 4; ++ci) {
-    {
+    if (!h->axis) {
       Timed tm(h, TC_FRAME);
       launch_frame_build(h->b, h->lay, ci, h->stream);
     }
     {
       Timed tm(h, TC_PHASE);
-      if (launch_phase(h->b, h->lay, ci, h->tpc, h->warps, h->record_chains, h->precision,
-                       h->stream))
+      if (h->axis ? launch_axis(h->b, h->axis_shape, h->tpc, h->fused_blocks, ci,
+                                h->record_chains, h->stream)
+                  : launch_phase(h->b, h->lay, ci, h->tpc, h->warps, h->record_chains, h->precision,
+                                 h->stream))
         return fail(ECMC_ERR_CUDA, "chain kernel launch failed: %s",
                     cudaGetErrorString(cudaGetLastError()));
     }
@@ -534,6 +632,7 @@ void free_all(ecmc_ctx* h) {
     cudaFree(h->b.pid[i]);
     cudaFree(h->b.count[i]);
   }
+  cudaFree(h->b.rel);
   cudaFree(h->b.state);
   cudaFree(h->b.cell_stats);
   cudaFree(h->b.totals);
@@ -724,6 +823,7 @@ int create_impl(ecmc_t* out, const ecmc_replica_desc_t* desc, int R) {
       cudaMalloc(&b.cell_stats, sizeof(CellStats) * (size_t)C_total) != cudaSuccess ||
       cudaMalloc(&b.totals, sizeof(RunTotals) * R) != cudaSuccess ||
       cudaMalloc(&b.err, sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&b.rel, sizeof(float2) * slots) != cudaSuccess ||
       cudaMalloc(&b.sched, sizeof(unsigned) * 4) != cudaSuccess ||
       cudaMalloc(&b.done, sizeof(unsigned) * (size_t)C_total) != cudaSuccess ||
       cudaMalloc(&h->d_geo, sizeof(Geom) * R) != cudaSuccess ||
@@ -1090,7 +1190,7 @@ int ecmc_get_param(ecmc_t h, int key, double* v) {
     case ECMC_PARAM_PERSISTENT: *v = h->persistent; break;
     case ECMC_PARAM_WAIT_LIMIT_MS: *v = h->wait_ms; break;
     case ECMC_PARAM_WAIT_TEST: *v = h->b.wait_test; break;
-    case ECMC_PARAM_KERNELS_PER_SWEEP: *v = h->persistent ? 5 : 12; break;
+    case ECMC_PARAM_KERNELS_PER_SWEEP: *v = h->persistent ? 5 : (h->axis ? 8 : 12); break;
     case ECMC_PARAM_CHAINS_IN_FLIGHT:
       *v = h->persistent ? (double)h->fused_blocks * (32 / h->tpc) : 0.0;
       break;

@@ -56,9 +56,11 @@ void launch_sweep_begin(const DevBufs& b, cudaStream_t s) {
 // estimate's error interval [q - eq, q + eq] holds no cell boundary and lies
 // inside (0, cells), its floor is the FP64 result; otherwise (about 2 eq of
 // the disks) the FP64 formula runs.
+// uf receives the FP32 offset from the lattice's corner, wrapped into [0, L).
 __device__ __forceinline__ int cell_1d_screened(double v, double shift, double L, double inv_w,
-                                                int cells, float Lf, float inv_wf, float eq) {
-  float uf = to_float_trunc(v) - to_float_trunc(shift);
+                                                int cells, float Lf, float inv_wf, float eq,
+                                                float& uf) {
+  uf = to_float_trunc(v) - to_float_trunc(shift);
   uf = uf < 0.0f ? uf + Lf : uf;
   const float qf = uf * inv_wf;
   const float lo = qf - eq, hi = qf + eq;
@@ -67,6 +69,16 @@ __device__ __forceinline__ int cell_1d_screened(double v, double shift, double L
     if (ilo == ihi) return ilo;
   }
   return cell_1d(v, shift, L, inv_w, cells);
+}
+
+// The offset u of cell_1d_screened relative to cell c's corner.  With v and
+// the shift within 2^-23 of their FP64 values and six FP32 roundings of
+// numbers up to L + w, it is within 2^-21 (L + w); at the box edge the FP32
+// and the FP64 wrap may differ, hence the wrap of the difference.
+__device__ __forceinline__ float cell_offset(float u, int c, float wf, float Lf) {
+  float d = u - (float)c * wf;
+  d = d > 0.5f * Lf ? d - Lf : d;
+  return d < -0.5f * Lf ? d + Lf : d;
 }
 
 // Append disk (x, y, id) to its bucket in dst.  Called by every lane of the
@@ -78,18 +90,22 @@ __device__ __forceinline__ void bin_one(const Geom* __restrict__ rg,
                                         const SweepState* __restrict__ sts, int rep, bool valid,
                                         double x, double y, int id, double* __restrict__ qx,
                                         double* __restrict__ qy, int* __restrict__ qid,
-                                        int* __restrict__ cnt_dst, int cap, int* err) {
+                                        float2* __restrict__ rel, int* __restrict__ cnt_dst,
+                                        int cap, int* err) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   int cn = -1;
+  float2 off = make_float2(0.0f, 0.0f);
   if (valid) {
     const Geom& g = rg[rep];
     const SweepState& st = sts[rep];
     const int cx = cell_1d_screened(x, st.sx, g.L, g.inv_w, g.cells_x, g.Lf, g.inv_wf,
-                                    g.bin_eq_x);
+                                    g.bin_eq_x, off.x);
     const int cy = cell_1d_screened(y, st.sy, g.L, g.inv_h, g.cells_y, g.Lf, g.inv_hf,
-                                    g.bin_eq_y);
+                                    g.bin_eq_y, off.y);
     cn = g.cell_off + cy * g.cells_x + cx;
+    off.x = cell_offset(off.x, cx, (float)g.w, g.Lf);
+    off.y = cell_offset(off.y, cy, (float)g.h, g.Lf);
   }
   const unsigned grp = __match_any_sync(FULL, cn);
   const int leader = __ffs(grp) - 1;
@@ -106,6 +122,7 @@ __device__ __forceinline__ void bin_one(const Geom* __restrict__ rg,
   qx[o] = x;
   qy[o] = y;
   qid[o] = id;
+  if (rel != nullptr) rel[o] = off;
 }
 
 // Bin every disk of buffer src into the buckets of buffer dst (whose counts
@@ -115,7 +132,8 @@ __global__ void k_bin_bucketed(const Geom* __restrict__ rg, const SweepState* __
                                const double* __restrict__ px, const double* __restrict__ py,
                                const int* __restrict__ pid, const int* __restrict__ cnt_src,
                                double* __restrict__ qx, double* __restrict__ qy,
-                               int* __restrict__ qid, int* __restrict__ cnt_dst, int* err) {
+                               int* __restrict__ qid, float2* __restrict__ rel,
+                               int* __restrict__ cnt_dst, int* err) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool in = i < (int64_t)C_total * cap;  // whole warps reach bin_one
   const int c = in ? (int)(i / cap) : 0;
@@ -123,7 +141,7 @@ __global__ void k_bin_bucketed(const Geom* __restrict__ rg, const SweepState* __
   const bool valid = in && k < min(__ldg(&cnt_src[c]), cap);
   const int r = valid ? cell_rep[c] : 0;
   bin_one(rg, st, r, valid, valid ? px[i] : 0.0, valid ? py[i] : 0.0, valid ? pid[i] : 0, qx,
-          qy, qid, cnt_dst, cap, err);
+          qy, qid, rel, cnt_dst, cap, err);
 }
 
 __device__ __forceinline__ int replica_of_disk(const int64_t* __restrict__ n_off, int R,
@@ -143,12 +161,12 @@ __global__ void k_bin_flat(const Geom* __restrict__ rg, const SweepState* __rest
                            const int64_t* __restrict__ n_off, int R, int64_t N_total, int cap,
                            const double* __restrict__ px, const double* __restrict__ py,
                            double* __restrict__ qx, double* __restrict__ qy, int* __restrict__ qid,
-                           int* __restrict__ cnt_dst, int* err) {
+                           float2* __restrict__ rel, int* __restrict__ cnt_dst, int* err) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = i < N_total;  // whole warps reach bin_one
   const int r = valid ? replica_of_disk(n_off, R, i) : 0;
   bin_one(rg, st, r, valid, valid ? px[i] : 0.0, valid ? py[i] : 0.0,
-          valid ? (int)(i - n_off[r]) : 0, qx, qy, qid, cnt_dst, cap, err);
+          valid ? (int)(i - n_off[r]) : 0, qx, qy, qid, rel, cnt_dst, cap, err);
 }
 
 void launch_bin(const DevBufs& b, int src, int dst, cudaStream_t s) {
@@ -158,14 +176,14 @@ void launch_bin(const DevBufs& b, int src, int dst, cudaStream_t s) {
     const int sb = 1 - dst;
     const int64_t nb = (b.N_total + bs - 1) / bs;
     k_bin_flat<<<(unsigned)nb, bs, 0, s>>>(b.rg, b.state, b.n_off, b.R, b.N_total, b.cap, b.px[sb],
-                                          b.py[sb], b.px[dst], b.py[dst], b.pid[dst],
+                                          b.py[sb], b.px[dst], b.py[dst], b.pid[dst], b.rel,
                                           b.count[dst], b.err);
   } else {
     const int64_t total = (int64_t)b.C_total * b.cap;
     const int64_t nb = (total + bs - 1) / bs;
     k_bin_bucketed<<<(unsigned)nb, bs, 0, s>>>(b.rg, b.state, b.cell_rep, b.C_total, b.cap,
                                               b.px[src], b.py[src], b.pid[src], b.count[src],
-                                              b.px[dst], b.py[dst], b.pid[dst], b.count[dst],
+                                              b.px[dst], b.py[dst], b.pid[dst], b.rel, b.count[dst],
                                               b.err);
   }
 }

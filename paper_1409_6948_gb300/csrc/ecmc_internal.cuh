@@ -165,6 +165,15 @@ inline RecLayout make_layout(int cpw, int nbin, int cap_mem, int cap_obj) {
   return r;
 }
 
+// Sizes of the axis-chain kernel's shared memory (ecmc_axis.cuh): cells per
+// warp, strips across the axis, and the room for objects per frame (co) and
+// members (mp): _s when the warp's cells are worked on together (co_s per
+// cell, mp_s over all of them), _h for one cell at its packing bound alone.
+constexpr int kAxisMaxObjects = 65533;  // candidate indices have 16 bits
+struct AxisShape {
+  int cpw, nbin, co_s, mp_s, co_h, mp_h;
+};
+
 // Device pointers of one handle (and the host-side sizes launches need).
 struct DevBufs {
   double* px[2];
@@ -172,6 +181,8 @@ struct DevBufs {
   int* pid[2];
   int* count[2];
   int cur;  // buffer holding the current positions
+  float2* rel;  // per slot of the current buffer: FP32 position relative to its cell's
+                // corner, within 2^-21 (L + w) (the axis-chain kernel's screen; or NULL)
   SweepState* state;       // [R]
   CellStats* cell_stats;   // [C_total]
   RunTotals* totals;       // [R]
@@ -229,8 +240,7 @@ size_t frame_stage_bytes(const RecLayout& lay);
 int configure_frame_build(const RecLayout& lay);
 int configure_phase(const RecLayout& lay, int tpc, int warps, int fmode);
 int probe_peaks(double* smem_gbs, double* fp64_gflops);
-size_t fused_smem_bytes(const RecLayout& lay, int fm);
-size_t fused_scratch_bytes(const RecLayout& lay);
+size_t fused_smem_bytes(const RecLayout& lay);
 // Chain-loop variant of the kernels: 0 axis chains reflected at walls and
 // frozen disks, 1 isotropic chains, 2 axis chains under the rejecting
 // boundary rule (a compile-time variant, so that the default loop carries
@@ -264,9 +274,16 @@ void set_screen_bounds(Geom& g);
 void set_strip_bins(Geom& g, double strip_w);
 
 inline int chain_kind(const DevBufs& b) { return b.iso ? 1 : (b.reject ? 2 : 0); }
-int configure_fused(const RecLayout& lay, int tpc, int fm, int kind, int* blocks_per_sm);
+int configure_fused(const RecLayout& lay, int tpc, int* blocks_per_sm);
 int launch_fused(const DevBufs& b, const RecLayout& lay, int tpc, int blocks, int records_on,
                  int precision, cudaStream_t s);
+// Axis chains with static candidates (ecmc_axis.cuh); phase < 0: the
+// persistent sweep, else one colour phase.
+size_t axis_smem(const AxisShape& s, int fm);
+size_t axis_scratch(const AxisShape& s);
+int configure_axis(const AxisShape& s, int tpc, int fm, int reject, int* blocks_per_sm);
+int launch_axis(const DevBufs& b, const AxisShape& s, int tpc, int blocks, int phase,
+                int records_on, cudaStream_t st);
 int launch_sqrt_rn(const double* x, double* out, int64_t n, cudaStream_t s);
 void host_sqrt_rn(const double* x, double* out, int64_t n, double rel_error);
 // fmode: 0 = whole frame in shared memory, 1 = FP64 coordinates in global
