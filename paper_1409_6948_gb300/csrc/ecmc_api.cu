@@ -548,7 +548,7 @@ int enqueue_min_dist2(ecmc_ctx* h) {
   std::memcpy(&h->pin_bits[0], &r2, sizeof(r2));
   CK(cudaMemcpyAsync(h->u64_tmp, &h->pin_bits[0], sizeof(unsigned long long),
                      cudaMemcpyHostToDevice, h->stream));
-  for (const Geom& g : h->geo) launch_min_dist(g, h->b, 2.0 * g.sigma, h->u64_tmp, h->stream);
+  launch_min_dist(h->geo.data(), h->b, h->u64_tmp, h->stream);
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(&h->pin_bits[1], h->u64_tmp, sizeof(unsigned long long),
                      cudaMemcpyDeviceToHost, h->stream));
@@ -718,6 +718,7 @@ int setup_geom(const ecmc_replica_desc_t& d, Geom& g, bool lattice_start = true)
   g.inv_w = 1.0 / g.w;
   g.inv_h = 1.0 / g.h;
   set_bin_screen(g);
+  set_min_dist(g);
   g.ell = d.ell;
   g.seed = d.seed;
   g.replica = d.replica;
@@ -1352,9 +1353,10 @@ int ecmc_replica_gr_measure(ecmc_t h, int r) {
   const int R = (int)h->geo.size();
   if (r < -1 || r >= R) return fail(ECMC_ERR_ARG, "replica %d out of range", r);
   const int r0 = r < 0 ? 0 : r, r1 = r < 0 ? R : r + 1;
+  bool have_fixed = false;
   for (int q = r0; q < r1; ++q) {
     launch_gr(h->geo[q], h->b, h->gr_dr, h->gr_nbins, h->gr_counts + (size_t)q * h->gr_nbins,
-              h->stream);
+              &have_fixed, h->stream);
     h->gr_meas[q] += 1;
   }
   CK(cudaGetLastError());
@@ -1371,9 +1373,9 @@ int ecmc_hexatic(ecmc_t h, double rs, double* psi, double* psi_k, int32_t* n_nb,
   }
   const int64_t N = h->b.N_total;
   unsigned long long* bad = h->u64_tmp + 1;
-  CK(cudaMemsetAsync(bad, 0, sizeof(unsigned long long), h->stream));
+  CK(cudaMemsetAsync(bad, 0, 2 * sizeof(unsigned long long), h->stream));
   double2* pk = reinterpret_cast<double2*>(h->xy_tmp);
-  if (launch_hexatic(h->b, rs, pk, h->int_tmp, bad, h->stream))
+  if (launch_hexatic(h->geo.data(), h->b, rs, pk, h->int_tmp, bad, h->stream))
     return fail(ECMC_ERR_CUDA, "hexatic kernel launch failed: %s",
                 cudaGetErrorString(cudaGetLastError()));
   std::vector<double> hk(2 * (size_t)N);

@@ -125,6 +125,10 @@ struct Geom {
   // FP32 within bin_eq_* of the FP64 product; the FP64 formula decides only
   // when that interval touches a cell boundary
   float Lf, inv_wf, inv_hf, bin_eq_x, bin_eq_y;
+  // measurements: 2^32 / L, and the overlap check's scan (set_min_dist)
+  double fix_scale, md_r2;
+  float md_skip;
+  int md_Rx, md_Ry, md_path;
   int boundary;      // 0 reflect at walls and frozen disks, 1 reject the whole chain
   UndoEntry* undo;   // boundary 1: undo logs, undo_stride entries per global cell
   int undo_stride;   // largest bucket capacity of the handle (>= cap_mem)
@@ -216,8 +220,8 @@ struct DevBufs {
 };
 
 // ---- launchers (defined in the .cu files) --------------------------------
-// Every launcher covers all replicas of the handle, except the measurements
-// (min_dist, gr, cells_of), which take the replica's host-side geometry.
+// Every launcher covers all replicas of the handle, except gr and cells_of,
+// which take the replica's host-side geometry.
 void launch_sweep_begin(const DevBufs& b, cudaStream_t s);
 void launch_bin(const DevBufs& b, int src, int dst, cudaStream_t s);
 void launch_frame_build(const DevBufs& b, const RecLayout& lay, int colour_index,
@@ -229,12 +233,12 @@ void launch_sweep_end(const DevBufs& b, cudaStream_t s);
 void launch_gather(const DevBufs& b, double* xy_out, cudaStream_t s);
 void launch_load_flat(const DevBufs& b, const double* xy_dev, cudaStream_t s);
 void launch_cells_of(const Geom& g, const DevBufs& b, int* cell_of_id, cudaStream_t s);
-int launch_hexatic(const DevBufs& b, double rs, double2* psi_k, int* nn,
+int launch_hexatic(const Geom* geo, const DevBufs& b, double rs, double2* psi_k, int* nn,
                    unsigned long long* bad, cudaStream_t s);
-void launch_min_dist(const Geom& g, const DevBufs& b, double rcut, unsigned long long* out,
-                     cudaStream_t s);
+void set_min_dist(Geom& g);
+void launch_min_dist(const Geom* geo, const DevBufs& b, unsigned long long* out, cudaStream_t s);
 void launch_gr(const Geom& g, const DevBufs& b, double dr, int nbins, unsigned long long* counts,
-               cudaStream_t s);
+               bool* have_fixed, cudaStream_t s);
 size_t frame_build_smem(const RecLayout& lay);
 size_t frame_stage_bytes(const RecLayout& lay);
 int configure_frame_build(const RecLayout& lay);

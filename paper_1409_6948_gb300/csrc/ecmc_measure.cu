@@ -147,21 +147,40 @@ __global__ void k_pairs(Geom g, int cap, const double* __restrict__ px,
 // (rcut^2 + Bt) (1 + 2^-19) has no pair within rcut.  The result is the same
 // double, bit for bit, as the minimum of the FP64 formula over all pairs.
 
-// 32-bit fractions of the box side, one uint2 per bucket slot
-__global__ void k_fixed_point(Geom g, int cap, const double* __restrict__ px,
+// 32-bit fractions of the box side, one uint2 per bucket slot, for all
+// replicas of the handle at once.  They go to the position buffer the next
+// binning overwrites.
+__global__ void k_fixed_point(const Geom* __restrict__ rg, const int* __restrict__ cell_rep,
+                              int C_total, int cap, const double* __restrict__ px,
                               const double* __restrict__ py, const int* __restrict__ cnt,
-                              double scale, uint2* __restrict__ fxy) {
-  const int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (li >= (int64_t)g.ncell * cap) return;
-  const int lcell = (int)(li / cap);
-  const int k = (int)(li - (int64_t)lcell * cap);
-  const int c = g.cell_off + lcell;
+                              uint2* __restrict__ fxy) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)C_total * cap) return;
+  const int c = (int)((unsigned)i / (unsigned)cap);
+  const int k = (int)(i - (int64_t)c * cap);
   if (k >= min(cnt[c], cap)) return;
-  const int64_t i = (int64_t)c * cap + k;
+  const double scale = rg[cell_rep[c]].fix_scale;
   // floor, then modulo 2^32: x slightly below 0 or rounded up to 2^32 wraps
   const long long X = __double2ll_rd(px[i] * scale);
   const long long Y = __double2ll_rd(py[i] * scale);
   fxy[i] = make_uint2((unsigned)X, (unsigned)Y);
+}
+
+// Slot indices have 31 bits (create_impl refuses larger handles).
+// Warps per cell: one per 32 disks of the mean cell.
+static unsigned warps_per_cell(int64_t N, int ncell, int cap) {
+  const int64_t y = (N + 32 * (int64_t)ncell - 1) / (32 * (int64_t)ncell);
+  const int64_t most = (cap + 31) / 32;
+  return (unsigned)(y < 1 ? 1 : (y < most ? y : most));
+}
+
+static uint2* launch_fixed_point(const DevBufs& b, cudaStream_t s) {
+  uint2* fxy = reinterpret_cast<uint2*>(b.px[1 - b.cur]);
+  const int bs = 256;
+  const int64_t total = (int64_t)b.C_total * b.cap;
+  k_fixed_point<<<(unsigned)((total + bs - 1) / bs), bs, 0, s>>>(
+      b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], b.count[b.cur], fxy);
+  return fxy;
 }
 
 __device__ __forceinline__ float bt_bound(float x) {
@@ -177,19 +196,27 @@ __device__ __forceinline__ double pair_d2(const double* __restrict__ px,
   return ddx * ddx + ddy * ddy;
 }
 
-// One warp per cell; lane l takes members l, l + 32, ...  HALF: each
-// unordered pair once (own cell with kk > k, then the offsets (ox, 0), ox > 0,
-// and (ox, oy), oy > 0), valid when 2R + 1 <= cells in both directions.
-// Otherwise every neighbour cell of the FP64 scan's enumeration, minus self.
+// A row of gridDim.y warps per cell of all replicas (one launch for a batch:
+// loading 96 replicas took 3.26 ms with two launches each, 1.49 ms now); lane l
+// of warp y takes members 32 y + l, then every 32 gridDim.y-th.  More than one
+// warp where the mean cell holds more than 32 disks: 45 us against 73 with one
+// at N = 65,536 in 32^2 cells.
+// HALF: each unordered pair once (own cell with kk > k, then the offsets (ox,
+// 0), ox > 0, and (ox, oy), oy > 0), valid when 2R + 1 <= cells in both
+// directions.  Otherwise every neighbour cell of the FP64 scan's enumeration,
+// minus self.
 template <bool HALF>
-__global__ void __launch_bounds__(256) k_min_dist_fixed(
-    Geom g, int cap, const double* __restrict__ px, const double* __restrict__ py,
-    const uint2* __restrict__ fxy, const int* __restrict__ cnt, int Rx, int Ry, float t_skip,
-    unsigned long long r2_bits, unsigned long long* __restrict__ out) {
+__device__ __forceinline__ void min_dist_cell(const Geom& g, int lcell, int cap,
+                                              const double* __restrict__ px,
+                                              const double* __restrict__ py,
+                                              const uint2* __restrict__ fxy,
+                                              const int* __restrict__ cnt,
+                                              unsigned long long* __restrict__ out) {
+  const int Rx = g.md_Rx, Ry = g.md_Ry;
+  const float t_skip = g.md_skip;
+  const unsigned long long r2_bits = __double_as_longlong(g.md_r2);
   constexpr unsigned kFull = 0xffffffffu;
   const float kInf = __int_as_float(0x7f800000);
-  const int lcell = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (lcell >= g.ncell) return;  // warp-uniform
   const int lane = threadIdx.x & 31;
   const int c = g.cell_off + lcell;
   const int cx = lcell % g.cells_x, cy = lcell / g.cells_x;
@@ -198,7 +225,7 @@ __global__ void __launch_bounds__(256) k_min_dist_fixed(
   const bool absx = (2 * Rx + 1 >= g.cells_x), absy = (2 * Ry + 1 >= g.cells_y);
   unsigned long long best = r2_bits;
 
-  for (int m0 = 0; m0 < nmem; m0 += 32) {
+  for (int m0 = 32 * blockIdx.y; m0 < nmem; m0 += 32 * gridDim.y) {
     const int k = m0 + lane;
     const bool act = k < nmem;
     const int64_t i = (int64_t)c * cap + (act ? k : 0);
@@ -281,6 +308,17 @@ __global__ void __launch_bounds__(256) k_min_dist_fixed(
   if (lane == 0 && best < r2_bits) atomicMin(out, best);
 }
 
+__global__ void __launch_bounds__(256) k_min_dist_fixed(
+    const Geom* __restrict__ rg, const int* __restrict__ cell_rep, int C_total, int cap,
+    const double* __restrict__ px, const double* __restrict__ py, const uint2* __restrict__ fxy,
+    const int* __restrict__ cnt, unsigned long long* __restrict__ out) {
+  const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (c >= C_total) return;  // warp-uniform
+  const Geom& g = rg[cell_rep[c]];
+  if (g.md_path == 1) min_dist_cell<true>(g, c - g.cell_off, cap, px, py, fxy, cnt, out);
+  else if (g.md_path == 2) min_dist_cell<false>(g, c - g.cell_off, cap, px, py, fxy, cnt, out);
+}
+
 // ---- pair-correlation histogram on fixed-point positions ------------------
 // The counts are the integers of the FP64 scan (k_pairs<true>), found with
 // integer and FP32 work for nearly every pair.  Every pair is screened on its
@@ -298,7 +336,8 @@ __global__ void __launch_bounds__(256) k_min_dist_fixed(
 // qm (host) is twice the sum of these bounds at d = rcut plus the FP32
 // spacing at nbins, so the rounding of q32 -/+ qm is covered as well.
 // D outside [dmin, dmax] puts d certainly below sigma or beyond rcut.
-// One warp per cell, lane l takes members l, l + 32, ...; each unordered pair
+// gridDim.y warps per cell (81 us against 126 with one at N = 65,536 in 32^2
+// cells), lane l takes members l, l + 32, ...; each unordered pair
 // is visited once (own cell kk > k, then the half stencil, valid when 2R + 1
 // <= cells in both directions) and adds 2: the FP64 distance is symmetric, as
 // x_i - x_j rounds to -(x_j - x_i).  Per-warp 32-bit histograms in shared
@@ -324,7 +363,7 @@ __global__ void __launch_bounds__(128) k_gr_fixed(
     const int c = g.cell_off + lcell;
     const int cx = lcell % g.cells_x, cy = lcell / g.cells_x;
     const int nmem = min(cnt[c], cap);
-    for (int m0 = 0; m0 < nmem; m0 += 32) {
+    for (int m0 = 32 * blockIdx.y; m0 < nmem; m0 += 32 * gridDim.y) {
       const int k = m0 + lane;
       const bool act = k < nmem;
       const int i = c * cap + (act ? k : 0);
@@ -375,56 +414,55 @@ __global__ void __launch_bounds__(128) k_gr_fixed(
   }
 }
 
-// The fixed-point scan needs rcut < L / 4 (|dX| < 2^30) and int32 slot
-// indices; other boxes take the FP64 scan.  The fractions go to the
-// position buffer the next binning overwrites.
-void launch_min_dist(const Geom& g, const DevBufs& b, double rcut, unsigned long long* out,
-                     cudaStream_t s) {
-  const int64_t total = (int64_t)g.ncell * b.cap;
-  const int64_t slots_end = (int64_t)(g.cell_off + g.ncell) * b.cap;
-  if (!(rcut < 0.25 * g.L) || slots_end >= ((int64_t)1 << 31)) {
-    const int bs = 128;
-    k_pairs<false><<<(unsigned)((total + bs - 1) / bs), bs, 0, s>>>(
-        g, b.cap, b.px[b.cur], b.py[b.cur], b.count[b.cur], rcut, 0.0, 0, out);
-    return;
-  }
-  const double scale = 4294967296.0 / g.L;
-  uint2* fxy = reinterpret_cast<uint2*>(b.px[1 - b.cur]);
-  {
-    const int bs = 256;
-    k_fixed_point<<<(unsigned)((total + bs - 1) / bs), bs, 0, s>>>(
-        g, b.cap, b.px[b.cur], b.py[b.cur], b.count[b.cur], scale, fxy);
-  }
-  const int Rx = (int)std::ceil(rcut * g.inv_w * (1.0 + 1e-9));
-  const int Ry = (int)std::ceil(rcut * g.inv_h * (1.0 + 1e-9));
-  const double r2 = rcut * rcut;
-  unsigned long long r2_bits = 0;
-  std::memcpy(&r2_bits, &r2, sizeof(r2));
+// Which scan a replica takes (host): the fixed-point scan needs rcut = 2 sigma
+// < L / 4 (|dX| < 2^30); small boxes take the FP64 scan.
+void set_min_dist(Geom& g) {
+  const double rcut = 2.0 * g.sigma;
+  g.fix_scale = 4294967296.0 / g.L;
+  g.md_Rx = (int)std::ceil(rcut * g.inv_w * (1.0 + 1e-9));
+  g.md_Ry = (int)std::ceil(rcut * g.inv_h * (1.0 + 1e-9));
+  g.md_r2 = rcut * rcut;
   // FP32 D above which no pair lies within rcut: (R + Bt(R) + 1)(1 + 2^-19)
   // with R = (rcut 2^32 / L)^2, rounded up
-  const double R = (rcut * scale) * (rcut * scale);
+  const double R = (rcut * g.fix_scale) * (rcut * g.fix_scale);
   const double t_skip_d = (R + 2.9 * std::sqrt(R) + 8.0 + R * std::ldexp(1.0, -40) + 1.0) *
                           (1.0 + std::ldexp(1.0, -19));
-  const float t_skip = std::nextafter((float)t_skip_d, 3.0e38f);
-  const bool half = 2 * Rx + 1 <= g.cells_x && 2 * Ry + 1 <= g.cells_y;
+  g.md_skip = std::nextafter((float)t_skip_d, 3.0e38f);
+  const bool half = 2 * g.md_Rx + 1 <= g.cells_x && 2 * g.md_Ry + 1 <= g.cells_y;
+  g.md_path = !(rcut < 0.25 * g.L) ? 0 : (half ? 1 : 2);
+}
+
+// geo: the R replicas' geometry on the host.
+void launch_min_dist(const Geom* geo, const DevBufs& b, unsigned long long* out, cudaStream_t s) {
+  bool fixed = false;
+  for (int r = 0; r < b.R; ++r) {
+    const Geom& g = geo[r];
+    if (g.md_path) {
+      fixed = true;
+      continue;
+    }
+    const int bs = 128;
+    const int64_t total = (int64_t)g.ncell * b.cap;
+    k_pairs<false><<<(unsigned)((total + bs - 1) / bs), bs, 0, s>>>(
+        g, b.cap, b.px[b.cur], b.py[b.cur], b.count[b.cur], 2.0 * g.sigma, 0.0, 0, out);
+  }
+  if (!fixed) return;
+  const uint2* fxy = launch_fixed_point(b, s);
   const int bs = 256;
-  const unsigned grid = (unsigned)(((int64_t)g.ncell * 32 + bs - 1) / bs);
-  if (half)
-    k_min_dist_fixed<true><<<grid, bs, 0, s>>>(g, b.cap, b.px[b.cur], b.py[b.cur], fxy,
-                                                b.count[b.cur], Rx, Ry, t_skip, r2_bits, out);
-  else
-    k_min_dist_fixed<false><<<grid, bs, 0, s>>>(g, b.cap, b.px[b.cur], b.py[b.cur], fxy,
-                                                 b.count[b.cur], Rx, Ry, t_skip, r2_bits, out);
+  const dim3 grid((unsigned)(((int64_t)b.C_total * 32 + bs - 1) / bs),
+                  warps_per_cell(b.N_total, b.C_total, b.cap));
+  k_min_dist_fixed<<<grid, bs, 0, s>>>(
+      b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], fxy, b.count[b.cur], out);
 }
 
 // The fixed-point histogram needs rcut < L / 4, int32 slot indices, a half
 // stencil (2R + 1 <= cells per side) and at most kGrFixedBins bins; other
-// systems (small boxes) take the FP64 scan.  Like the overlap check, it keeps
-// its fractions in the position buffer the next binning overwrites.
+// systems (small boxes) take the FP64 scan.  *have_fixed: the fractions are in
+// place (the other replicas of one measurement share them).
 constexpr int kGrFixedBins = 2048;
 
 void launch_gr(const Geom& g, const DevBufs& b, double dr, int nbins, unsigned long long* counts,
-               cudaStream_t s) {
+               bool* have_fixed, cudaStream_t s) {
   const int64_t total = (int64_t)g.ncell * b.cap;
   const int64_t slots_end = (int64_t)(g.cell_off + g.ncell) * b.cap;
   const double rcut = g.sigma + dr * nbins;
@@ -438,13 +476,9 @@ void launch_gr(const Geom& g, const DevBufs& b, double dr, int nbins, unsigned l
         g, b.cap, b.px[b.cur], b.py[b.cur], b.count[b.cur], rcut, dr, nbins, counts);
     return;
   }
-  const double scale = 4294967296.0 / g.L;
-  uint2* fxy = reinterpret_cast<uint2*>(b.px[1 - b.cur]);
-  {
-    const int bs = 256;
-    k_fixed_point<<<(unsigned)((total + bs - 1) / bs), bs, 0, s>>>(
-        g, b.cap, b.px[b.cur], b.py[b.cur], b.count[b.cur], scale, fxy);
-  }
+  if (!*have_fixed) launch_fixed_point(b, s);  // once for all replicas measured
+  *have_fixed = true;
+  const uint2* fxy = reinterpret_cast<const uint2*>(b.px[1 - b.cur]);
   const double u = g.L / 4294967296.0;
   const double ed = 1.5;  // |sqrt(D) - d64 / u| in units of u
   const double tmax = rcut / dr + 1.0;
@@ -463,12 +497,13 @@ void launch_gr(const Geom& g, const DevBufs& b, double dr, int nbins, unsigned l
   p.dmin = lo > 0.0 ? (unsigned long long)std::floor(lo * lo) : 0ull;
   const int bs = 128, nw = bs / 32;
   const size_t sm = sizeof(unsigned int) * (size_t)nw * nbins;
-  k_gr_fixed<<<(unsigned)((g.ncell + nw - 1) / nw), bs, sm, s>>>(
+  const dim3 grid((unsigned)((g.ncell + nw - 1) / nw), warps_per_cell(g.N, g.ncell, b.cap));
+  k_gr_fixed<<<grid, bs, sm, s>>>(
       g, b.cap, b.px[b.cur], b.py[b.cur], fxy, b.count[b.cur], Rx, Ry, p, counts);
 }
 
 // Hexatic order parameter (Sec. 2, eq. Psi) with Delaunay next neighbours.
-// One thread per bucket slot: the disks within rs (minimum image) are gathered
+// k_hexatic, one warp per disk: the disks within rs (minimum image) are gathered
 // from the neighbour cells into shared memory and sorted by disk id; disk l is
 // a Delaunay neighbour when the perpendicular bisector of the pair keeps a
 // piece of positive length after every other gathered disk m cuts it with the
@@ -479,100 +514,159 @@ void launch_gr(const Geom& g, const DevBufs& b, double dr, int nbins, unsigned l
 // the concatenated id order.  rs <= 0: 3.5 sigma of each replica.
 constexpr int kHexMaxCand = 64;
 
-__global__ void k_hexatic(const Geom* __restrict__ rg, const int* __restrict__ cell_rep,
-                          int C_total, int cap, const double* __restrict__ px,
-                          const double* __restrict__ py, const int* __restrict__ pid,
-                          const int* __restrict__ cnt, double rs_arg,
-                          double2* __restrict__ psi_out, int* __restrict__ nn_out,
-                          unsigned long long* bad) {
-  extern __shared__ __align__(16) unsigned char hsm[];
-  double2* cand = reinterpret_cast<double2*>(hsm) + (size_t)threadIdx.x * kHexMaxCand;
-  int* cid = reinterpret_cast<int*>(reinterpret_cast<double2*>(hsm) + (size_t)blockDim.x *
-                                                                          kHexMaxCand) +
-             (size_t)threadIdx.x * kHexMaxCand;
-  const int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (li >= (int64_t)C_total * cap) return;
-  const int c = (int)(li / cap);
-  const int k = (int)(li - (int64_t)c * cap);
-  if (k >= min(cnt[c], cap)) return;
+// Which disks are Delaunay neighbours, decided in FP32 with error bounds; only
+// Psi_k itself is evaluated in FP64, over the neighbours in id order, by the
+// expressions of k_hexatic.  What FP32 cannot decide (near-degenerate cells,
+// crystals, dilute spots) is left to k_hexatic, which then runs for those disks
+// only.  k_hexatic spends its time in FP64 divisions, one per pair of the 35
+// disks within 3.5 sigma of a disk: 6.8 ms at N = 65,536 in 32^2 cells with a
+// thread per disk, against 0.28 ms for both kernels now.
+//
+// Candidates: the disks within rc = min(rs, 2.2 L / sqrt(N)) on the fixed-point
+// positions (differences exact but for 1.6 L / 2^32 and three FP32 roundings:
+// hx_d bounds a coordinate difference).  On the bisector d_l / 2 + t perp(d_l)
+// disk m cuts t at b / a, with a = perp(d_l) . d_m and b = (|d_m|^2 - d_l . d_m)
+// / 2 each within hx_e.  tlo and thi are bracketed by b / a -+ (hx_e (1 + |t|)) /
+// (|a| - hx_e) and the rounding of t.  A pair with |a| <= 8 hx_e cuts at |t| >
+// 1000 when |b| > 0.1 sigma^2, which closed cells never reach: it decides
+// nothing if b > 0 and removes l if b < 0.  All cell vertices within rc / 2
+// also mean that no disk beyond rc takes part.  Non-overlapping disks leave at
+// most 58 centres within 3.5 sigma, so the 64-disk limit needs no count.
+// One warp per 32 members of a cell: its lanes scan the same cells, so the
+// loads are broadcast.
+constexpr int kHexList = 32;
+
+__global__ void __launch_bounds__(64) k_hexatic_fixed(
+    const Geom* __restrict__ rg, const int* __restrict__ cell_rep, int C_total, int cap,
+    int chunks, const double* __restrict__ px, const double* __restrict__ py,
+    const int* __restrict__ pid, const uint2* __restrict__ fxy, const int* __restrict__ cnt,
+    double rs_arg, double2* __restrict__ psi_out, int* __restrict__ nn_out,
+    int* __restrict__ undecided, unsigned long long* n_undecided) {
+  extern __shared__ float2 hx_sm[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float2* const cand = hx_sm + warp * kHexList * 32 + lane;  // [entry][lane]
+  int* const cslot = (int*)(hx_sm + (blockDim.x >> 5) * kHexList * 32) + warp * kHexList * 32 +
+                     lane;
+  const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+  const int c = (int)(w / chunks);
+  if (c >= C_total) return;  // warp-uniform
+  const int k = (int)(w - (int64_t)c * chunks) * 32 + lane;
+  const int nmem = min(cnt[c], cap);
+  if (k - lane >= nmem) return;  // warp-uniform
+  const bool act = k < nmem;
   const Geom& g = rg[cell_rep[c]];
   const int lcell = c - g.cell_off;
-  const int64_t i = (int64_t)c * cap + k;
   const int cx = lcell % g.cells_x, cy = lcell / g.cells_x;
-  const double xi = px[i], yi = py[i];
-  const double L = g.L;
+  const int i = c * cap + (act ? k : 0);
   const double rs = rs_arg > 0.0 ? rs_arg : 3.5 * g.sigma;
-  const double rs2 = rs * rs, v2max = 0.25 * rs * rs;
-  const int Rx = (int)ceil(rs * g.inv_w * (1.0 + 1e-9));
-  const int Ry = (int)ceil(rs * g.inv_h * (1.0 + 1e-9));
+  const float unit = (float)(g.L * 0x1p-32);
+  const float sigf = (float)g.sigma;
+  const float rc = fminf((float)rs, 2.2f * (float)(g.L * rsqrt((double)g.N)));
+  const float rc2 = rc * rc;
+  const unsigned reach = (unsigned)fminf(rc / unit + 4.0f, 2147483392.0f);
+  const int Rx = (int)ceilf(rc * (float)g.inv_w * 1.00001f);
+  const int Ry = (int)ceilf(rc * (float)g.inv_h * 1.00001f);
   const NbRange rx = nb_range(Rx, g.cells_x), ry = nb_range(Ry, g.cells_y);
-  const bool absx = (2 * Rx + 1 >= g.cells_x), absy = (2 * Ry + 1 >= g.cells_y);
-  int nc = 0;
-  bool over = false;
+  const bool absx = 2 * Rx + 1 >= g.cells_x, absy = 2 * Ry + 1 >= g.cells_y;
+  const uint2 pi = fxy[i];
+  int n = 0;
   for (int oy = 0; oy < ry.n; ++oy) {
     const int qy = absy ? oy : ((cy + ry.first + oy) % g.cells_y + g.cells_y) % g.cells_y;
     for (int ox = 0; ox < rx.n; ++ox) {
       const int qx = absx ? ox : ((cx + rx.first + ox) % g.cells_x + g.cells_x) % g.cells_x;
       const int q = g.cell_off + qy * g.cells_x + qx;
-      const int nq = min(cnt[q], cap);
-      const int64_t b0 = (int64_t)q * cap;
+      const int nq = min(cnt[q], cap), b0 = q * cap;
+#pragma unroll 4
       for (int kk = 0; kk < nq; ++kk) {
-        const int64_t j = b0 + kk;
-        if (j == i) continue;
-        const double ddx = wrap_half(px[j] - xi, L);
-        const double ddy = wrap_half(py[j] - yi, L);
-        if (!(ddx * ddx + ddy * ddy < rs2)) continue;
-        if (nc == kHexMaxCand) {
-          over = true;
-          continue;
+        const uint2 pj = fxy[b0 + kk];
+        const int dx = (int)(pj.x - pi.x), dy = (int)(pj.y - pi.y);
+        if ((unsigned)dx + reach <= 2u * reach && (unsigned)dy + reach <= 2u * reach &&
+            b0 + kk != i) {
+          const float fx = (float)dx * unit, fy = (float)dy * unit;
+          if (fx * fx + fy * fy < rc2) {
+            if (n < kHexList) {
+              cand[n * 32] = make_float2(fx, fy);
+              cslot[n * 32] = b0 + kk;
+            }
+            ++n;
+          }
         }
-        // insertion by disk id (the order the sums below run in)
-        const int id = pid[j];
-        int pos = nc;
-        while (pos > 0 && cid[pos - 1] > id) {
-          cand[pos] = cand[pos - 1];
-          cid[pos] = cid[pos - 1];
-          --pos;
-        }
-        cand[pos] = make_double2(ddx, ddy);
-        cid[pos] = id;
-        ++nc;
       }
     }
   }
-  double re = 0.0, im = 0.0;
-  int n = 0;
-  bool ok = !over;
-  for (int l = 0; l < nc; ++l) {
-    const double2 dl = cand[l];
-    const double ux = -dl.y, uy = dl.x;
-    const double px0 = 0.5 * dl.x, py0 = 0.5 * dl.y;
-    double tlo = -__longlong_as_double(0x7ff0000000000000ll);
-    double thi = __longlong_as_double(0x7ff0000000000000ll);
-    for (int m = 0; m < nc && tlo < thi; ++m) {
+  const float hx_d = 1.6f * unit + 0x1.8p-23f * rc;
+  const float hx_e = 4.0f * rc * hx_d + 0x1p-21f * rc2;
+  const float vmax2 = (0.25f * rc2 - 4.0f * rc * hx_d) * 0.999f;
+  bool known = act && n <= kHexList;
+  if (n > kHexList) n = kHexList;
+  int nn = 0;  // neighbours: their entries move to the front, sorted by id
+  unsigned nb_mask = 0;
+  for (int l = 0; l < n && known; ++l) {
+    const float2 d = cand[l * 32];
+    const float dd = d.x * d.x + d.y * d.y;
+    float lo0 = -__int_as_float(0x7f800000), lo1 = lo0;  // lower, upper bound of tlo
+    float hi0 = -lo0, hi1 = hi0;
+    bool dead = false;
+    for (int m = 0; m < n; ++m) {
       if (m == l) continue;
-      const double2 dm = cand[m];
-      const double a = ux * dm.x + uy * dm.y;
-      const double b = 0.5 * (dm.x * dm.x + dm.y * dm.y) - (px0 * dm.x + py0 * dm.y);
-      if (a > 0.0) {
-        const double t = b / a;
-        if (t < thi) thi = t;
-      } else if (a < 0.0) {
-        const double t = b / a;
-        if (t > tlo) tlo = t;
-      } else if (b < 0.0) {
-        thi = -__longlong_as_double(0x7ff0000000000000ll);
+      const float2 e = cand[m * 32];
+      const float a = d.x * e.y - d.y * e.x;
+      const float b = 0.5f * (e.x * (e.x - d.x) + e.y * (e.y - d.y));
+      const float aa = fabsf(a);
+      if (aa <= 8.0f * hx_e) {
+        if (b > 0.1f * sigf * sigf) continue;
+        if (b < -0.1f * sigf * sigf) dead = true;
+        else known = false;
+        break;
+      }
+      const float t = __fdividef(b, a);
+      const float dt = __fdividef(hx_e * (1.0f + fabsf(t)), aa - hx_e) + 0x1p-20f * fabsf(t);
+      if (a > 0.0f) {
+        hi0 = fminf(hi0, t - dt);
+        hi1 = fminf(hi1, t + dt);
+      } else {
+        lo0 = fmaxf(lo0, t - dt);
+        lo1 = fmaxf(lo1, t + dt);
+      }
+      if (lo0 > hi1) {
+        dead = true;
+        break;
       }
     }
-    if (!(tlo < thi)) continue;
-    if (isinf(tlo) || isinf(thi)) {
-      ok = false;
-    } else {
-      const double vx0 = px0 + tlo * ux, vy0 = py0 + tlo * uy;
-      const double vx1 = px0 + thi * ux, vy1 = py0 + thi * uy;
-      if (!(vx0 * vx0 + vy0 * vy0 < v2max) || !(vx1 * vx1 + vy1 * vy1 < v2max)) ok = false;
+    if (!known) break;
+    if (dead) continue;
+    // open or long edges are left to the FP64 test, as are those whose length
+    // is within the bounds
+    const float tm = fmaxf(fabsf(lo0), fabsf(hi1));
+    if (!(lo1 < hi0) || !(dd * (0.25f + tm * tm) < vmax2)) {
+      known = false;
+      break;
     }
-    const double zx = dl.x, zy = dl.y;
+    nb_mask |= 1u << l;
+  }
+  if (!act) return;
+  const int64_t id = g.n_off + pid[i];
+  if (!known) {
+    undecided[atomicAdd(n_undecided, 1ull)] = i;
+    return;
+  }
+  // the neighbours in ascending id, Psi_k in FP64
+  double re = 0.0, im = 0.0;
+  const double xi = px[i], yi = py[i], L = g.L;
+  int last = -1;
+  nn = __popc(nb_mask);
+  for (int s = 0; s < nn; ++s) {
+    int best = INT_MAX, slot = 0;
+    for (unsigned r = nb_mask; r; r &= r - 1) {
+      const int sl = cslot[(__ffs((int)r) - 1) * 32];
+      const int idj = pid[sl];
+      if (idj > last && idj < best) {
+        best = idj;
+        slot = sl;
+      }
+    }
+    last = best;
+    const double zx = wrap_half(px[slot] - xi, L), zy = wrap_half(py[slot] - yi, L);
     const double z2x = zx * zx - zy * zy, z2y = 2.0 * zx * zy;
     const double z3x = z2x * zx - z2y * zy, z3y = z2x * zy + z2y * zx;
     const double z6x = z3x * z3x - z3y * z3y, z6y = 2.0 * z3x * z3y;
@@ -580,25 +674,174 @@ __global__ void k_hexatic(const Geom* __restrict__ rg, const int* __restrict__ c
     const double r6 = r2 * r2 * r2;
     re += z6x / r6;
     im += z6y / r6;
-    ++n;
   }
-  if (!ok) atomicAdd(bad, 1ull);
-  const int64_t id = g.n_off + pid[i];
-  psi_out[id] = make_double2(n > 0 ? re / (double)n : 0.0, n > 0 ? im / (double)n : 0.0);
-  nn_out[id] = over ? -1 : n;
+  psi_out[id] = make_double2(nn > 0 ? re / (double)nn : 0.0, nn > 0 ? im / (double)nn : 0.0);
+  nn_out[id] = nn;
 }
 
-size_t hexatic_smem_bytes(int threads) {
-  return (size_t)threads * kHexMaxCand * (sizeof(double2) + sizeof(int));
+// The FP64 decision, a warp per disk.  list: the bucket slots to work on
+// (*n_list of them), or NULL for every slot.
+__global__ void __launch_bounds__(128) k_hexatic(
+    const Geom* __restrict__ rg, const int* __restrict__ cell_rep, int C_total, int cap,
+    const double* __restrict__ px, const double* __restrict__ py, const int* __restrict__ pid,
+    const int* __restrict__ cnt, double rs_arg, double2* __restrict__ psi_out,
+    int* __restrict__ nn_out, const int* __restrict__ list, const unsigned long long* n_list,
+    unsigned long long* bad) {
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ double2 s_raw[4][kHexMaxCand], s_cand[4][kHexMaxCand];
+  __shared__ int s_id[4][kHexMaxCand];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double2* const raw = s_raw[warp];
+  double2* const cand = s_cand[warp];
+  int* const cid = s_id[warp];
+  const int64_t total = list != nullptr ? (int64_t)*n_list : (int64_t)C_total * cap;
+  const int64_t step = (int64_t)gridDim.x * 4;
+  for (int64_t at = (int64_t)blockIdx.x * 4 + warp; at < total; at += step) {
+    const int i = list != nullptr ? list[at] : (int)at;
+    const int c = i / cap, k = i - c * cap;
+    if (k >= min(cnt[c], cap)) continue;  // warp-uniform
+    const Geom& g = rg[cell_rep[c]];
+    const int lcell = c - g.cell_off;
+    const int cx = lcell % g.cells_x, cy = lcell / g.cells_x;
+    const double xi = px[i], yi = py[i];
+    const double L = g.L;
+    const double rs = rs_arg > 0.0 ? rs_arg : 3.5 * g.sigma;
+    const double rs2 = rs * rs, v2max = 0.25 * rs * rs;
+    const int Rx = (int)ceil(rs * g.inv_w * (1.0 + 1e-9));
+    const int Ry = (int)ceil(rs * g.inv_h * (1.0 + 1e-9));
+    const NbRange rx = nb_range(Rx, g.cells_x), ry = nb_range(Ry, g.cells_y);
+    const bool absx = (2 * Rx + 1 >= g.cells_x), absy = (2 * Ry + 1 >= g.cells_y);
+    int nc = 0;
+    __syncwarp();
+    for (int oy = 0; oy < ry.n; ++oy) {
+      const int qy = absy ? oy : ((cy + ry.first + oy) % g.cells_y + g.cells_y) % g.cells_y;
+      for (int ox = 0; ox < rx.n; ++ox) {
+        const int qx = absx ? ox : ((cx + rx.first + ox) % g.cells_x + g.cells_x) % g.cells_x;
+        const int q = g.cell_off + qy * g.cells_x + qx;
+        const int nq = min(cnt[q], cap), b0 = q * cap;
+        for (int k0 = 0; k0 < nq; k0 += 32) {
+          const int j = b0 + k0 + lane;
+          bool in = k0 + lane < nq && j != i;
+          double ddx = 0.0, ddy = 0.0;
+          if (in) {
+            ddx = wrap_half(px[j] - xi, L);
+            ddy = wrap_half(py[j] - yi, L);
+            in = ddx * ddx + ddy * ddy < rs2;
+          }
+          const unsigned got = __ballot_sync(FULL, in);
+          const int pos = nc + __popc(got & ((1u << lane) - 1u));
+          if (in && pos < kHexMaxCand) {
+            raw[pos] = make_double2(ddx, ddy);
+            cid[pos] = pid[j];
+          }
+          nc += __popc(got);
+        }
+      }
+    }
+    const int64_t id = g.n_off + pid[i];
+    if (nc > kHexMaxCand) {
+      if (lane == 0) {
+        atomicAdd(bad, 1ull);
+        psi_out[id] = make_double2(0.0, 0.0);
+        nn_out[id] = -1;
+      }
+      continue;
+    }
+    __syncwarp();
+    // sorted by disk id (the order the sums below run in)
+    for (int l = lane; l < nc; l += 32) {
+      const int idl = cid[l];
+      int r = 0;
+      for (int m = 0; m < nc; ++m) r += cid[m] < idl;
+      cand[r] = raw[l];
+    }
+    __syncwarp();
+    double re = 0.0, im = 0.0;
+    int n = 0;
+    bool ok = true;
+    for (int l0 = 0; l0 < nc; l0 += 32) {
+      const int l = l0 + lane;
+      const double2 dl = cand[l < nc ? l : 0];
+      const double ux = -dl.y, uy = dl.x;
+      const double px0 = 0.5 * dl.x, py0 = 0.5 * dl.y;
+      double tlo = -__longlong_as_double(0x7ff0000000000000ll);
+      double thi = __longlong_as_double(0x7ff0000000000000ll);
+      bool nb = l < nc;
+      for (int m = 0; m < nc && nb; ++m) {
+        if (m == l) continue;
+        const double2 dm = cand[m];
+        const double a = ux * dm.x + uy * dm.y;
+        const double b = 0.5 * (dm.x * dm.x + dm.y * dm.y) - (px0 * dm.x + py0 * dm.y);
+        if (a > 0.0) {
+          const double t = b / a;
+          if (t < thi) thi = t;
+        } else if (a < 0.0) {
+          const double t = b / a;
+          if (t > tlo) tlo = t;
+        } else if (b < 0.0) {
+          thi = -__longlong_as_double(0x7ff0000000000000ll);
+        }
+        nb = tlo < thi;
+      }
+      double tx = 0.0, ty = 0.0;
+      if (nb) {
+        if (isinf(tlo) || isinf(thi)) {
+          ok = false;
+        } else {
+          const double vx0 = px0 + tlo * ux, vy0 = py0 + tlo * uy;
+          const double vx1 = px0 + thi * ux, vy1 = py0 + thi * uy;
+          if (!(vx0 * vx0 + vy0 * vy0 < v2max) || !(vx1 * vx1 + vy1 * vy1 < v2max)) ok = false;
+        }
+        const double zx = dl.x, zy = dl.y;
+        const double z2x = zx * zx - zy * zy, z2y = 2.0 * zx * zy;
+        const double z3x = z2x * zx - z2y * zy, z3y = z2x * zy + z2y * zx;
+        const double z6x = z3x * z3x - z3y * z3y, z6y = 2.0 * z3x * z3y;
+        const double r2 = zx * zx + zy * zy;
+        const double r6 = r2 * r2 * r2;
+        tx = z6x / r6;
+        ty = z6y / r6;
+      }
+      for (unsigned r = __ballot_sync(FULL, nb); r; r &= r - 1) {
+        const int src = __ffs((int)r) - 1;
+        re += __shfl_sync(FULL, tx, src);
+        im += __shfl_sync(FULL, ty, src);
+        ++n;
+      }
+    }
+    ok = __all_sync(FULL, ok);
+    if (lane == 0) {
+      if (!ok) atomicAdd(bad, 1ull);
+      psi_out[id] = make_double2(n > 0 ? re / (double)n : 0.0, n > 0 ? im / (double)n : 0.0);
+      nn_out[id] = n;
+    }
+  }
 }
 
-int launch_hexatic(const DevBufs& b, double rs, double2* psi_k, int* nn,
+// geo: the R replicas' geometry on the host.  bad[0] counts the uncertified
+// disks, bad[1] is scratch; both zero on entry.  The undecided disks are listed
+// in the position buffer the next binning overwrites.
+int launch_hexatic(const Geom* geo, const DevBufs& b, double rs, double2* psi_k, int* nn,
                    unsigned long long* bad, cudaStream_t s) {
-  const int bs = 32;
-  const int64_t total = (int64_t)b.C_total * b.cap;
-  k_hexatic<<<(unsigned)((total + bs - 1) / bs), bs, hexatic_smem_bytes(bs), s>>>(
+  // the FP32 decision needs the packing bound of the 64-disk limit
+  bool fixed = true;
+  int* const list = reinterpret_cast<int*>(b.py[1 - b.cur]);
+  unsigned long long* const n_list = bad + 1;
+  for (int r = 0; r < b.R; ++r) fixed = fixed && !(rs > 3.5 * geo[r].sigma);
+  if (fixed) {
+    const uint2* fxy = launch_fixed_point(b, s);
+    const int wpb = 2, chunks = (b.cap + 31) / 32;
+    const int64_t blocks = ((int64_t)b.C_total * chunks + wpb - 1) / wpb;
+    const size_t sm = (size_t)wpb * kHexList * 32 * (sizeof(float2) + sizeof(int));
+    k_hexatic_fixed<<<(unsigned)blocks, 32 * wpb, sm, s>>>(
+        b.rg, b.cell_rep, b.C_total, b.cap, chunks, b.px[b.cur], b.py[b.cur], b.pid[b.cur], fxy,
+        b.count[b.cur], rs, psi_k, nn, list, n_list);
+  }
+  // enough warps to fill the GPU when every disk is left to it
+  const int64_t most = ((int64_t)b.C_total * b.cap + 3) / 4;
+  const int64_t blocks = most < 152 * 12 ? most : 152 * 12;
+  k_hexatic<<<(unsigned)blocks, 128, 0, s>>>(
       b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], b.pid[b.cur],
-      b.count[b.cur], rs, psi_k, nn, bad);
+      b.count[b.cur], rs, psi_k, nn, fixed ? list : nullptr, n_list, bad);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -215,7 +215,7 @@ extern "C" int ecmc_sweep_noalloc(double* xy, int64_t N, double L, double sigma,
   launch_load_flat(b, xy, s);
   launch_sweep_begin(b, s);
   launch_bin(b, -1, b.cur, s);
-  launch_min_dist(g, b, 2.0 * g.sigma, d_min, s);
+  launch_min_dist(&g, b, d_min, s);
   int err = 0;
   unsigned long long min_bits = 0;
   if (cudaGetLastError() != cudaSuccess ||
