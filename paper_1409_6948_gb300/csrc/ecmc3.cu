@@ -955,6 +955,118 @@ __global__ void k3_min_dist(Geom3 g, const double* __restrict__ px, const double
   if ((threadIdx.x & 31) == 0 && best < r2_bits) atomicMin(out, best);
 }
 
+// The same minimum on fixed-point positions, as in two dimensions
+// (ecmc_measure.cu, k_min_dist_fixed, which derives the method): coordinates as
+// 32-bit fractions of the box side, squared distances D in FP32, one FP64
+// evaluation per lane unless its two smallest D are too close to call, and then
+// the window that holds every candidate.  Three dimensions change the bounds:
+// |D - D*| <= 2 sqrt(3) e sqrt(D) + 9 e^2 with e = 1 + 2^-16, and the FP64
+// formula adds less than 2^-18 sqrt(3 D) + 2^-50 D, below Bt(D) = 4.2 sqrt(D) +
+// 16 + D / 2^40; the FP32 value of D (two roundings per square, two sums) stays
+// within 2^-21 of D.  Pairs are visited once: the own cell with kk > k, then the
+// 13 neighbours of the half stencil, so boxes need four cells per side and
+// rcut < L / 4 (the FP64 scan takes the others).
+//
+// The FP64 scan was bound by the FP64 pipe, 27 x 8 candidates of three wraps
+// each per sphere: 2.1 ms at N = 64^3 in 32^3 cells.  One warp per cell; cells
+// of up to 8 (16) members split the stencil over four (two) groups of lanes.
+__global__ void k3_fixed_point(Geom3 g, double scale, const double* __restrict__ px,
+                               const double* __restrict__ py, const double* __restrict__ pz,
+                               const int* __restrict__ cnt, const int* __restrict__ ids,
+                               uint4* __restrict__ fq) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)g.ncell * g.cap_mem) return;
+  const int c = (int)(i / g.cap_mem);
+  if ((int)(i - (int64_t)c * g.cap_mem) >= min(cnt[c], g.cap_mem)) return;
+  const int id = ids[i];
+  fq[i] = make_uint4((unsigned)__double2ll_rd(px[id] * scale),
+                     (unsigned)__double2ll_rd(py[id] * scale),
+                     (unsigned)__double2ll_rd(pz[id] * scale), (unsigned)id);
+}
+
+__device__ __forceinline__ float bt_bound3(float x) {
+  return 4.2f * sqrtf(x) + 16.0f + x * 0x1p-40f;
+}
+
+__global__ void __launch_bounds__(256) k3_min_dist_fixed(
+    Geom3 g, const double* __restrict__ px, const double* __restrict__ py,
+    const double* __restrict__ pz, const int* __restrict__ cnt, const uint4* __restrict__ fq,
+    float t_skip, unsigned long long r2_bits, unsigned long long* __restrict__ out) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const float kInf = __int_as_float(0x7f800000);
+  const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (c >= g.ncell) return;  // warp-uniform
+  const int lane = threadIdx.x & 31, nc = g.cells;
+  const int cx = c % nc, cy = (c / nc) % nc, cz = c / (nc * nc);
+  const int nmem = min(cnt[c], g.cap_mem);
+  const int gsz = nmem <= 8 ? 8 : (nmem <= 16 ? 16 : 32);
+  unsigned long long best = r2_bits;
+  for (int m0 = 0; m0 < nmem; m0 += gsz) {
+    const int k = m0 + (lane & (gsz - 1));
+    const bool act = k < nmem;
+    const uint4 pi = fq[(int64_t)c * g.cap_mem + (act ? k : 0)];
+    // cells of the half stencil: 0 the own one (kk > k), then offsets 14 .. 26
+    // of the 3x3x3 block
+    auto scan = [&](auto&& visit) {
+      for (int e = lane / gsz; e < 14; e += 32 / gsz) {
+        int q = c;
+        if (e > 0) {
+          const int f = 13 + e;
+          int qx = cx + f % 3 - 1, qy = cy + (f / 3) % 3 - 1, qz = cz + f / 9 - 1;
+          qx = qx < 0 ? qx + nc : (qx >= nc ? qx - nc : qx);
+          qy = qy < 0 ? qy + nc : (qy >= nc ? qy - nc : qy);
+          qz = qz < 0 ? qz + nc : (qz >= nc ? qz - nc : qz);
+          q = (qz * nc + qy) * nc + qx;
+        }
+        const int nq = min(cnt[q], g.cap_mem);
+        const uint4* const f = fq + (int64_t)q * g.cap_mem;
+        const int kmin = e == 0 ? k : -1;
+#pragma unroll 4
+        for (int kk = 0; kk < nq; ++kk) {
+          const uint4 pj = f[kk];
+          const float dx = (float)(int)(pj.x - pi.x), dy = (float)(int)(pj.y - pi.y),
+                      dz = (float)(int)(pj.z - pi.z);
+          const float D = dx * dx + dy * dy + dz * dz;
+          visit(kk > kmin ? D : kInf, (int)pj.w);
+        }
+      }
+    };
+    auto exact = [&](int j) {
+      const int i = (int)pi.w;
+      const double ex = wrap_half(px[j] - px[i], g.L);
+      const double ey = wrap_half(py[j] - py[i], g.L);
+      const double ez = wrap_half(pz[j] - pz[i], g.L);
+      const unsigned long long bits =
+          (unsigned long long)__double_as_longlong(ex * ex + ey * ey + ez * ez);
+      best = bits < best ? bits : best;
+    };
+    float m1 = kInf, m2 = kInf;
+    int j1 = 0;
+    if (act)
+      scan([&](float D, int j) {
+        const bool lt1 = D < m1;
+        m2 = lt1 ? m1 : fminf(m2, D);
+        j1 = lt1 ? j : j1;
+        m1 = lt1 ? D : m1;
+      });
+    if (act && m1 <= t_skip) {
+      if (m2 - m1 > bt_bound3(m1) + bt_bound3(m2) + m2 * 0x1p-20f) {
+        exact(j1);
+      } else {
+        const float win = (m1 + 4.0f * bt_bound3(m1) + 64.0f) * (1.0f + 0x1p-19f);
+        scan([&](float D, int j) {
+          if (D <= win) exact(j);
+        });
+      }
+    }
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    const unsigned long long o2 = __shfl_xor_sync(FULL, best, off);
+    best = o2 < best ? o2 : best;
+  }
+  if (lane == 0 && best < r2_bits) atomicMin(out, best);
+}
+
 }  // namespace ecmc3
 
 // ---- host side ----------------------------------------------------------------
@@ -976,6 +1088,7 @@ struct ecmc3_ctx {
   double* history = nullptr;
   int64_t* hist_len = nullptr;
   unsigned long long* u64 = nullptr;
+  uint4* fq = nullptr;  // fixed-point positions by bucket slot (overlap check)
   int warps = 1;
   int64_t t_host = 0;
   bool valid = false;
@@ -1074,8 +1187,27 @@ int min_dist2_3(ecmc3_ctx* h, double* d2) {
   unsigned long long bits = 0;
   std::memcpy(&bits, &r2, sizeof(r2));
   CK3(cudaMemcpyAsync(h->u64, &bits, sizeof(bits), cudaMemcpyHostToDevice, h->stream));
-  k3_min_dist<<<(unsigned)((g.N + 255) / 256), 256, 0, h->stream>>>(
-      g, h->px, h->py, h->pz, h->cnt, h->ids, h->cell_of, bits, h->u64);
+  const int64_t slots = (int64_t)g.ncell * g.cap_mem;
+  bool fixed = rc < 0.25 * g.L && g.cells >= 4;
+  if (fixed && !h->fq && cudaMalloc(&h->fq, sizeof(uint4) * (size_t)slots) != cudaSuccess) {
+    cudaGetLastError();  // no room: the FP64 scan needs none
+    h->fq = nullptr;
+    fixed = false;
+  }
+  if (fixed) {
+    const double scale = 4294967296.0 / g.L;
+    const double R = (rc * scale) * (rc * scale);
+    const double skip = (R + 4.2 * std::sqrt(R) + 17.0 + R * std::ldexp(1.0, -40)) *
+                        (1.0 + std::ldexp(1.0, -19));
+    k3_fixed_point<<<(unsigned)((slots + 255) / 256), 256, 0, h->stream>>>(
+        g, scale, h->px, h->py, h->pz, h->cnt, h->ids, h->fq);
+    k3_min_dist_fixed<<<(unsigned)(((int64_t)g.ncell * 32 + 255) / 256), 256, 0, h->stream>>>(
+        g, h->px, h->py, h->pz, h->cnt, h->fq, std::nextafter((float)skip, 3.0e38f), bits,
+        h->u64);
+  } else {
+    k3_min_dist<<<(unsigned)((g.N + 255) / 256), 256, 0, h->stream>>>(
+        g, h->px, h->py, h->pz, h->cnt, h->ids, h->cell_of, bits, h->u64);
+  }
   CK3(cudaGetLastError());
   CK3(cudaMemcpyAsync(&bits, h->u64, sizeof(bits), cudaMemcpyDeviceToHost, h->stream));
   const int rc2 = check3(h);
@@ -1128,6 +1260,7 @@ void free3(ecmc3_ctx* h) {
   cudaFree(h->history);
   cudaFree(h->hist_len);
   cudaFree(h->u64);
+  cudaFree(h->fq);
   cudaFree(h->sched);
   cudaFree(h->done);
   if (h->own) cudaStreamDestroy(h->own);
