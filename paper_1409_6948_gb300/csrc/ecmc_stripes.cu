@@ -52,6 +52,7 @@ struct GeomS {
   // sorted-frame kernel: strips of width sw across the axis, nstrip of them
   double sw, inv_sw;
   int nstrip;
+  int near;  // a disk within sigma of a stripe's band lies at most this many stripes away
 };
 
 struct StateS {
@@ -369,6 +370,17 @@ __global__ void __launch_bounds__(kThreads) ks_phase(
 // once its last tested object has b - sigma above min(r, best s); otherwise
 // the next six are tested.  The first hit is the minimum of (s, key) over
 // the warp: the same object, distance and event as the full scan.
+//
+// What bounds it: one warp's serial chain, about 3,350 cycles an event (450
+// instructions; comparisons and square roots on the integer pipes, as each
+// FP64 instruction holds the pipe for some 60 cycles), then the frame, built
+// once per phase by the whole block: 55 us of a phase's 300.  The frame is
+// bound by the scan over all N stripe indices and the scattered fetches of
+// the members' coordinates, so both are done 32 at a time and the sort goes
+// through buckets of a few objects.  N = 2^16, 32 stripes, ell = 8, one chain
+// a stripe, GB300: 607 us a sweep; 1937 with the frame built by ordered
+// compaction of 512 ids at a time, a rank over whole strips (110 objects) and
+// FP64 comparisons.  With no chains' work (ell -> 0): 138 against 1401.
 constexpr int kSortThreads = 512;
 constexpr int kLanesPerStrip = 6;
 
@@ -377,8 +389,11 @@ __device__ __forceinline__ int strip_of_v(const GeomS& g, double v) {
   return q < 0 ? 0 : (q >= g.nstrip ? g.nstrip - 1 : q);
 }
 
+constexpr size_t sorted_object_bytes = sizeof(double) * 2 + sizeof(int) * 2;
+constexpr unsigned long long kMagnitude = 0x7fffffffffffffffull;
+
 __host__ __device__ inline size_t sorted_smem_bytes(int cap_obj, int cap_mem, int nstrip) {
-  return (sizeof(double) * 2 + sizeof(int) * 2) * (size_t)cap_obj + sizeof(int) * (size_t)cap_mem +
+  return sorted_object_bytes * (size_t)cap_obj + sizeof(int) * (size_t)cap_mem +
          sizeof(int) * (size_t)(3 * nstrip + 8) + ((size_t)cap_obj + 16);
 }
 
@@ -389,8 +404,7 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
     double* __restrict__ fU0, int* __restrict__ flist, StripeS* __restrict__ stats,
     int* __restrict__ recs, int* err) {
   extern __shared__ __align__(16) unsigned char ssm[];
-  __shared__ int wcnt[kSortThreads / 32];
-  __shared__ int sm_over, sm_n;
+  __shared__ int sm_over, sm_n, sm_mem;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned FULL = 0xffffffffu;
   const StateS s = *st;
@@ -422,109 +436,233 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
   int* fill = rot + g.nstrip;        // nstrip (build), then rot at the chain start
   unsigned char* sq = (unsigned char*)(fill + g.nstrip);  // strip of every object
 
-  if (tid == 0) sm_over = 0;
-  for (int q = tid; q < g.nstrip; q += kSortThreads) fill[q] = 0;
-  __syncthreads();
-
-  // frame, part 1: the members in ascending id (unsorted, in global scratch)
-  int n = 0;
-  for (int64_t i0 = 0; i0 < g.N; i0 += kSortThreads) {
-    const int64_t i = i0 + tid;
-    const bool mem = i < g.N && stripe_of[i] == k;
-    const unsigned bal = __ballot_sync(FULL, mem);
-    if (lane == 0) wcnt[warp] = __popc(bal);
-    __syncthreads();
-    int before = 0, total = 0;
-    for (int q = 0; q < kSortThreads / 32; ++q) {
-      before += q < warp ? wcnt[q] : 0;
-      total += wcnt[q];
-    }
-    const int slot = n + before + __popc(bal & ((1u << lane) - 1u));
-    __syncthreads();
-    if (mem) {
-      if (slot < g.cap_mem) {
-        gU[slot] = along[i];
-        gV[slot] = wrap_half(across[i] - origin, L);
-        gK[slot] = (long long)i * 3 + 1;
-      } else {
-        sm_over = 1;
-      }
-    }
-    n += total;
+  // buckets of the sort: each strip cut into n_cut parts along the axis; the
+  // counters lie in the member map, which is filled last
+  const int n_cut = g.cap_mem / g.nstrip < 2 ? 1 : min(16, g.cap_mem / g.nstrip);
+  const int n_bucket = n_cut * g.nstrip;
+  int* bucket = n_cut > 1 ? mem_g : fill;
+  const float cut_scale = (float)n_cut / (float)L;
+  // (the coordinate is not negative and the map is monotonic)
+  auto cut_of = [&](double u) {
+    const int c = (int)((float)u * cut_scale);
+    return c < n_cut ? c : n_cut - 1;
+  };
+  if (tid == 0) {
+    sm_over = 0;
+    sm_n = 0;
   }
-  const int n_mem = n;
+  for (int q = tid; q < n_bucket; q += kSortThreads) bucket[q] = 0;
+
+  // frame, part 1: the members in ascending id, and the images across
+  // (-L, 0, +L) of the other disks within sigma of the band (in any order:
+  // the strips are sorted by (U, key) below).  Ids are cut into runs, dealt to
+  // the warps in turn: a first pass counts the members of each run, a second
+  // places them.  An image within sigma of the band belongs to a disk at most
+  // g.near stripes away.  Members and those disks are few in a run or fill it,
+  // by the lattice the ids come from: each warp collects them in a queue, so
+  // that their coordinates are fetched and tested 32 at a time.
+  // The queues use the room of the sorted frame, which is not yet built: as
+  // many warps take part as have a queue there.
+  constexpr int kUnroll = 8;  // loads in flight
+  // (cap_obj < 22, no whole queue: L < 4.2 sigma, and the at most 16 disks
+  // of such a box never fill a quarter of one)
+  const int n_queues = (int)(sorted_object_bytes * (size_t)g.cap_obj / (sizeof(int2) * 64));
+  const int n_scan = max(1, min(kSortThreads / 32, n_queues));
+  const int n_run_max = min(256, g.cap_obj);
+  const int n_vec = (int)((g.N + 32 * kUnroll - 1) / (32 * kUnroll));
+  const int run = (n_vec + n_run_max - 1) / n_run_max * (32 * kUnroll);
+  const int n_run = (int)((g.N + run - 1) / run);
+  if (warp < n_scan)
+    for (int ir = warp; ir < n_run; ir += n_scan) {
+      const int64_t lo = (int64_t)ir * run;
+      const int i_lo = (int)lo, i_hi = (int)min(lo + run, g.N);
+      int c = 0;
+      for (int i0 = i_lo; i0 < i_hi; i0 += 32 * kUnroll) {
+        int so[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+          const int i = i0 + 32 * u + lane;
+          so[u] = i < i_hi ? stripe_of[i] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) c += so[u] == k;
+      }
+      c = __reduce_add_sync(FULL, c);
+      if (lane == 0) gO[ir] = c;
+    }
   __syncthreads();
-  // frame, part 2: images across (-L, 0, +L) of the other disks within sigma
-  // of the band (any order: the strips are sorted by (U, key) below)
-  if (tid == 0) sm_n = n_mem;
+  if (warp == 0) {  // the members before each run
+    int acc = 0;
+    for (int q0 = 0; q0 < n_run; q0 += 32) {
+      const int c = q0 + lane < n_run ? gO[q0 + lane] : 0;
+      int x = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, o);
+        x += lane >= o ? y : 0;
+      }
+      if (q0 + lane < n_run) gO[q0 + lane] = acc + x - c;
+      acc += __shfl_sync(FULL, x, 31);
+    }
+    if (lane == 0) {
+      sm_n = acc;
+      sm_mem = acc;
+      if (acc > g.cap_mem) sm_over = 1;
+    }
+  }
   __syncthreads();
-  for (int64_t i = tid; i < g.N; i += kSortThreads) {
-    if (stripe_of[i] == k) continue;
-    const double v0 = wrap_half(across[i] - origin, L);
-    for (int im = -1; im <= 1; ++im) {
-      const double v = im == 0 ? v0 : (im > 0 ? v0 + L : v0 - L);
-      if (!(v > -sigma && v < g.w + sigma)) continue;
-      const int slot = atomicAdd(&sm_n, 1);
-      if (slot < g.cap_obj) {
-        gU[slot] = along[i];
-        gV[slot] = v;
-        gK[slot] = (long long)i * 3 + (im + 1);
-      } else {
-        sm_over = 1;
+  const int n_mem = sm_mem;
+  if (warp < n_scan) {
+    int2* queue = (int2*)ssm + 64 * warp;
+    int n_queue = 0;
+    const double hL = 0.5 * L, v_hi = g.w + sigma;
+    // |v0| <= L/2: where the band ends before L/2 only the image at 0 counts
+    const int im_max = (g.w + sigma) * (1.0 + 1e-9) < hL ? 0 : 1;
+    auto place = [&](int2 e) {  // e: the id, and a member's slot or -1
+      const int i = e.x;
+      const double u = along[i];
+      const double v0 = ecmc::wrap_half_i(across[i] - origin, L, hL);
+      if (e.y >= 0) {
+        gU[e.y] = u;
+        gV[e.y] = v0;
+        gK[e.y] = (long long)i * 3 + 1;
+        return;
+      }
+#pragma unroll 1
+      for (int im = -im_max; im <= im_max; ++im) {
+        const double v = im == 0 ? v0 : (im > 0 ? v0 + L : v0 - L);
+        if (!(ecmc::dlt(-sigma, v) && ecmc::dlt(v, v_hi))) continue;
+        const int slot = atomicAdd(&sm_n, 1);
+        if (slot < g.cap_obj) {
+          gU[slot] = u;
+          gV[slot] = v;
+          gK[slot] = (long long)i * 3 + (im + 1);
+        } else {
+          sm_over = 1;
+        }
+      }
+    };
+    for (int ir = warp; ir < n_run; ir += n_scan) {
+      const int64_t lo = (int64_t)ir * run;
+      const int i_lo = (int)lo, i_hi = (int)min(lo + run, g.N);
+      int slot0 = gO[ir];
+      for (int i0 = i_lo; i0 < i_hi; i0 += 32 * kUnroll) {
+        int so[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+          const int i = i0 + 32 * u + lane;
+          so[u] = i < i_hi ? stripe_of[i] : -1;
+        }
+#pragma unroll 1
+        for (int u = 0; u < kUnroll; ++u) {
+          const int i = i0 + 32 * u + lane;
+          int si = so[0];
+#pragma unroll
+          for (int q = 1; q < kUnroll; ++q) si = q == u ? so[q] : si;
+          int dk = si > k ? si - k : k - si;
+          dk = dk > g.S - dk ? g.S - dk : dk;
+          const bool take = si >= 0 && dk <= g.near;
+          const unsigned tb = __ballot_sync(FULL, take);
+          if (tb == 0) continue;
+          const unsigned mb = __ballot_sync(FULL, si == k);
+          const unsigned below = (1u << lane) - 1u;
+          const int slot = slot0 + __popc(mb & below);
+          slot0 += __popc(mb);
+          // (a member beyond the bound: the phase is given up below)
+          if (take)
+            queue[n_queue + __popc(tb & below)] =
+                make_int2(i, si == k ? min(slot, g.cap_mem - 1) : -1);
+          n_queue += __popc(tb);
+          __syncwarp();
+          if (n_queue >= 32) {
+            const int2 e = queue[lane], rest = queue[32 + lane];
+            __syncwarp();
+            place(e);
+            n_queue -= 32;
+            if (lane < n_queue) queue[lane] = rest;
+            __syncwarp();
+          }
+        }
       }
     }
+    if (lane < n_queue) place(queue[lane]);
   }
   __syncthreads();
   const bool over = sm_over != 0;
-  n = over ? 0 : sm_n;
+  const int n = over ? 0 : sm_n;
   if (over && tid == 0) atomicCAS(err, kOk, kCapacity);
 
-  // strips: counts, starts, then each object's rank within its strip by
-  // (U, key); the sorted frame goes through global scratch into shared memory
-  for (int o = tid; o < n; o += kSortThreads) atomicAdd(&fill[strip_of_v(g, gV[o])], 1);
-  __syncthreads();
-  if (tid == 0) {
-    int acc = 0;
-    for (int q = 0; q < g.nstrip; ++q) {
-      sstart[q] = acc;
-      acc += fill[q];
-      fill[q] = 0;
-      rot[q] = 0;
-    }
-    sstart[g.nstrip] = acc;
-  }
-  __syncthreads();
+  // strips and their buckets: counts, starts, then each object's rank within
+  // its bucket by (U, key)
   for (int o = tid; o < n; o += kSortThreads) {
     const int q = strip_of_v(g, gV[o]);
-    const int p = sstart[q] + atomicAdd(&fill[q], 1);
+    const int b = q * n_cut + cut_of(gU[o]);
+    gO[o] = b;
+    atomicAdd(&bucket[b], 1);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int acc = 0;
+    for (int b0 = 0; b0 < n_bucket; b0 += 32) {
+      const int b = b0 + lane;
+      const int c = b < n_bucket ? bucket[b] : 0;
+      int x = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, o);
+        x += lane >= o ? y : 0;
+      }
+      if (b < n_bucket) {
+        bucket[b] = acc + x - c;
+        if (b % n_cut == 0) sstart[b / n_cut] = acc + x - c;
+      }
+      acc += __shfl_sync(FULL, x, 31);
+    }
+    if (lane == 0) sstart[g.nstrip] = acc;
+  }
+  for (int q = tid; q < g.nstrip; q += kSortThreads) rot[q] = 0;
+  __syncthreads();
+  // (afterwards a bucket's counter is its end, the start of the next)
+  for (int o = tid; o < n; o += kSortThreads) {
+    const int b = gO[o];
+    const int p = atomicAdd(&bucket[b], 1);
     U[p] = gU[o];
     V[p] = gV[o];
     key[p] = (int)gK[o];
     orig[p] = o;
+    sq[p] = (unsigned char)(b / n_cut);
   }
   __syncthreads();
-  for (int q = 0; q < g.nstrip; ++q) {
-    const int b0 = sstart[q], b1 = sstart[q + 1];
-    for (int p = b0 + tid; p < b1; p += kSortThreads) {
-      const double up = U[p];
-      const int kp = key[p];
-      int r = 0;
-      for (int p2 = b0; p2 < b1; ++p2) r += (U[p2] < up || (U[p2] == up && key[p2] < kp));
-      const int f = b0 + r;
-      gU[f] = up;
-      gV[f] = V[p];
-      gK[f] = kp;
-      gO[f] = orig[p];
+  for (int p = tid; p < n; p += kSortThreads) {
+    const double u = U[p];
+    const int b = sq[p] * n_cut + cut_of(u);
+    const int b0 = b ? bucket[b - 1] : 0, b1 = bucket[b];
+    // coordinates along the axis are not negative: they order as their bits
+    // (the sign of a zero aside)
+    const unsigned long long up = (unsigned long long)__double_as_longlong(u) & kMagnitude;
+    const int kp = key[p];
+    int f = b0;
+    for (int p2 = b0; p2 < b1; ++p2) {
+      const unsigned long long u2 = (unsigned long long)__double_as_longlong(U[p2]) & kMagnitude;
+      f += u2 < up || (u2 == up && key[p2] < kp);
     }
+    gU[f] = u;
+    gV[f] = V[p];
+    gK[f] = kp;
+    gO[f] = orig[p];
   }
   __syncthreads();
   for (int f = tid; f < n; f += kSortThreads) {
-    U[f] = gU[f];
+    const double u = gU[f];
+    const int o = gO[f];
+    U[f] = u;
     V[f] = gV[f];
     key[f] = (int)gK[f];
-    orig[f] = gO[f];
-    sq[f] = (unsigned char)strip_of_v(g, gV[f]);
-    if (gO[f] < n_mem) mem_g[gO[f]] = f;
+    orig[f] = o;
+    if (o < n_mem) {
+      mem_g[o] = f;
+      U0[o] = u;  // where a rejected chain goes back to
+    }
   }
   __syncthreads();
 
@@ -534,6 +672,14 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
     int chains = 0, accepted = 0;
     const int slot = lane / kLanesPerStrip, li = lane - slot * kLanesPerStrip;  // slot 5: idle
     const double INF = __longlong_as_double(0x7ff0000000000000ll);
+    const unsigned gm = ((1u << kLanesPerStrip) - 1u) << (slot * kLanesPerStrip);
+    const float L_eps = (float)L * 1e-15f;
+    // rounds of the 6-ary search that leave nothing of the longest strip
+    int nq_max = 0;
+    for (int q = lane; q < g.nstrip; q += 32) nq_max = max(nq_max, sstart[q + 1] - sstart[q]);
+    nq_max = __reduce_max_sync(FULL, nq_max);
+    int n_round = 0;
+    for (int len = nq_max; len > 0; len /= kLanesPerStrip + 1) ++n_round;
     // shuffled list of distinct members (negative control), as the oracle
     // draws it: entry 0 as drawn, then Fisher-Yates on entries 1..
     if (g.list_mode == 1 && n_mem > 0 && !over && lane == 0) {
@@ -579,10 +725,8 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
       double r = g.ell, chain_b = 0.0;
       long long nev = 0;
       if (lane == 0 && rec) rec[0] = key[m] / 3;
-      if (g.reject) {
-        for (int q = lane; q < n_mem; q += 32) U0[q] = U[mem_g[q]];
+      if (g.reject)
         for (int q = lane; q < g.nstrip; q += 32) fill[q] = rot[q];
-      }
       __syncwarp();
       int done = 0;  // 1 budget used up, 2 rejected, 3 contact cap
       for (long long iter = 0;; ++iter) {
@@ -599,7 +743,7 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
         // 6-ary search over [lo, hi): the predicate is false ... false true ...
         // true (compared as order-preserving integers)
         int lo = 0, hi = nq;
-        while (__any_sync(FULL, hi - lo > 0)) {
+        for (int round = 0; round < n_round; ++round) {
           const int len = hi - lo;
           const int step = (len + kLanesPerStrip) / (kLanesPerStrip + 1);  // >= 1
           const int probe = lo + (li + 1) * step - 1;
@@ -611,19 +755,15 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
             const long long ku = ecmc::dkey(U[b0 + pi]);
             pred = dsg > 0 ? (ku > kUm) : (ku >= kUm);
           }
-          const unsigned bt = __ballot_sync(FULL, act && pred);
-          const unsigned bf = __ballot_sync(FULL, act && !pred);
-          const unsigned gm = ((1u << kLanesPerStrip) - 1u) << (slot * kLanesPerStrip);
-          const unsigned t_g = bt & gm, f_g = bf & gm;
+          // (a probe beyond the interval counts as true)
+          const unsigned f_g = __ballot_sync(FULL, act && !pred) & gm;
           if (sv && len > 0) {
             // the true probes are a suffix of the probes: nf false probes put
             // the answer in [lo + nf step, first true probe] (or above the
-            // last probe); the interval shrinks every round
+            // last probe); len / 7 of the interval is left
             const int nf = __popc(f_g);
-            const int nlo = lo + nf * step;
-            const int nhi = t_g ? lo + (nf + 1) * step - 1 : hi;
-            lo = nlo;
-            hi = nhi < nlo ? nlo : nhi;
+            lo += nf * step;
+            hi = nf < kLanesPerStrip ? min(hi, lo + step - 1) : hi;
           }
         }
         // logical start of the scan: the first object ahead along d
@@ -692,16 +832,19 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
         const float Hf = __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(hf)));
         const float rf = ecmc::to_float_up_nn(r);
         const float limf = rf < Hf ? rf : Hf;
-        const double lim0 = (double)limf;
-        if (!__any_sync(FULL, still_open(0, bl0, lim0))) {
+        // a strip's last tested object out of reach, in FP32 with the roundings
+        // on the far side (if not, the exact test of the loop below decides)
+        const bool far0 = sv && nq > kLanesPerStrip && li == kLanesPerStrip - 1;
+        const float bl32 = ecmc::to_float_trunc(bl0);
+        const bool reach = !(bl32 - limf > g_sigf * 1.00001f + (bl32 + limf) * 1e-6f + L_eps);
+        if (!__any_sync(FULL, far0 && reach)) {
           // every strip is finished after window 0: the first hit is among
           // the candidates whose lower bound reaches min(r, Hf); evaluate
           // those with the oracle's expression
           const bool need = cand && lo_c <= limf;
           const unsigned nb = __ballot_sync(FULL, need);
           if (need) {
-            bs = b_c - sqrt(x_c);
-            if (bs < 0.0) bs = 0.0;
+            bs = ecmc::clamp0(b_c - ecmc::sqrt_rn(x_c));
             bk = key[j_c];
             bj = j_c;
             bb = b_c;
@@ -719,7 +862,7 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
               const int k2 = __shfl_xor_sync(FULL, bk, o);
               const int j2 = __shfl_xor_sync(FULL, bj, o);
               const double b2 = __shfl_xor_sync(FULL, bb, o);
-              if (s2 < bs || (s2 == bs && k2 < bk)) {
+              if (ecmc::lt_nn(s2, bs) || (ecmc::dbits(s2) == ecmc::dbits(bs) && k2 < bk)) {
                 bs = s2;
                 bk = k2;
                 bj = j2;
@@ -790,8 +933,8 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
           done = 3;
           break;
         }
-        if (r <= bs) {  // budget used up: the chain ends
-          const double x = Um + d * r;
+        if (ecmc::le_nn(r, bs)) {  // budget used up: the chain ends
+          const double x = Um + ecmc::flip_if(r, dsg < 0);
           if (lane == 0) {
             U[m] = wrap_along(x, L);
             if (x >= L || x < 0.0) {
@@ -816,10 +959,12 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
         }
         // the move, with the wrap round the periodic axis: bs <= b <= L, so x
         // lies in (-L, 2L), where wrap_along is x - L (exact) or x + L
-        const double x = Um + d * bs;
-        const bool wrapped = (x >= L) || (x < 0.0);
+        const double x = Um + ecmc::flip_if(bs, dsg < 0);
+        const bool below0 = ecmc::dkey(x) < 0, wrapped = below0 || !ecmc::dlt(x, L);
         if (lane == 0) {
-          U[m] = x >= L ? x - L : (x < 0.0 ? x + L : x);
+          double xw = x;
+          if (wrapped) xw = below0 ? x + L : x - L;
+          U[m] = xw;
           if (wrapped) {
             const int nm_ = sstart[qm + 1] - sstart[qm];
             int rr = rot[qm] + (dsg > 0 ? nm_ - 1 : 1);
@@ -840,8 +985,17 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
         }
       }
       if (done == 2) {
-        for (int q = lane; q < n_mem; q += 32) U[mem_g[q]] = U0[q];
+        for (int q0 = lane; q0 < n_mem; q0 += 32 * kUnroll) {
+          double u0[kUnroll];
+#pragma unroll
+          for (int u = 0; u < kUnroll; ++u) u0[u] = q0 + 32 * u < n_mem ? U0[q0 + 32 * u] : 0.0;
+#pragma unroll
+          for (int u = 0; u < kUnroll; ++u)
+            if (q0 + 32 * u < n_mem) U[mem_g[q0 + 32 * u]] = u0[u];
+        }
         for (int q = lane; q < g.nstrip; q += 32) rot[q] = fill[q];
+      } else if (g.reject && c + 1 < g.n_m) {  // the state the next chain starts from
+        for (int q = lane; q < n_mem; q += 32) U0[q] = U[mem_g[q]];
       }
       __syncwarp();
       chains++;
@@ -1112,6 +1266,9 @@ int ecmc_stripes_create(ecmc_stripes_t* out, int64_t N, double L, double sigma, 
   g.sw = 0.5 * sigma * (1.0 + std::ldexp(1.0, -30));
   g.inv_sw = 1.0 / g.sw;
   g.nstrip = (int)std::ceil((w + 2.0 * sigma) / g.sw) + 2;
+  // w > sigma: the next stripe on either side, and one more where rounding of
+  // a stripe's edge (a few ulp of L) could matter
+  g.near = w - sigma > 1e-12 * L ? 1 : 2;
   h->sorted_smem = sorted_smem_bytes(g.cap_obj, g.cap_mem, g.nstrip);
   {
     int dev = 0, optin = 0;
