@@ -7,20 +7,34 @@
 // k3_phase launches -- and k3_end (deterministic sums).  Either way one warp
 // processes one active cell (cell3): it sorts the cell's members by id,
 // gathers the members and every periodic image of the 26 neighbour cells'
-// spheres within sigma of the cell into a shared-memory frame (FP64
-// coordinates and their FP32 roundings), bins the frame across the sweep's
-// axis, and runs the cell's n_m chains.  Each event takes the three rows of
-// bins around the mover, screens their spheres in FP32 with a rigorous
-// margin (a sphere behind the mover or with perpendicular offset >= sigma
-// cannot be hit), tests the survivors in FP64 with the oracle's expressions
-// (no contraction: the library is built with -fmad=false) in one warp-wide
-// pass, and a shuffle reduction picks the first hit by (distance, key).  As
-// in the two-dimensional loop, comparisons of FP64 values and the square
-// root run on the integer pipes (bit-pattern orders, the correctly rounded
-// sqrt_rn): the same results as the FP64 instructions, with the FP64 pipe
-// left the arithmetic.  Positions live in sphere-id order; a cell reads its
-// frozen neighbours' positions, which no warp writes while it runs (later
-// colours wait for it, earlier ones have finished).
+// spheres within sigma of the cell into a shared-memory frame, and runs the
+// cell's n_m chains.
+//
+// Members move along the sweep's axis only, so an object is a candidate for
+// a member's contacts (c^2 < sigma^2 across the axis) for the whole phase or
+// not at all, and the square root in the contact distance is fixed as well.
+// Both are found when a member first becomes active -- an FP32 screen of the
+// frame with a rigorous margin (or of the nine bins across the axis round it,
+// where a frame has more than 4 x 4 of them), then the oracle's FP64
+// expressions (no contraction: the library is built with -fmad=false) -- and
+// kept as a list in shared memory.  An event is then one pass over some 20
+// list entries: b, b - root, and a minimum over the warp.  Lists share a room
+// of fixed size; when it is full they are dropped and found again.
+//
+// What bounds it: 16 to 20 warps a SM (registers, frames of 10 KB) that wait
+// for fixed latencies, shared memory and instruction fetch (1.4 instructions
+// a cycle), and the FP64 pipe, half busy: one warp instruction holds it for
+// 14 cycles of the SM however few lanes take part.  Hence comparisons of FP64
+// values and the square root run on the integer pipes (bit-pattern orders,
+// the correctly rounded sqrt_rn), a replayed leg takes one FP64 addition, and
+// the neighbours' spheres pass an FP32 test of their positions within their
+// cells (rel) before their coordinates are fetched.  N = 64^3, eta = 0.45,
+// 32^3 cells, ell = 2, n_m = 1, GB300: 541 us a sweep, 758 with a search of
+// the bins at every event and FP64 tests of all 26 neighbours; frames alone
+// 297 / 403; 8^3 cells, n_m = 32: 12.3 / 18.7 ms; 16^3 spheres in 4^3 cells:
+// 1.16 / 1.75 ms.  Positions live in sphere-id order; a cell reads its frozen
+// neighbours' positions, which no warp writes while it runs (later colours
+// wait for it, earlier ones have finished).
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -49,7 +63,6 @@ using ecmc::plus_zero;
 using ecmc::sqrt_rn;
 using ecmc::to_float_trunc;
 using ecmc::unit_double;
-using ecmc::wrap_box0;
 using ecmc::wrap_half;
 using ecmc::wrap_half_i;
 
@@ -63,14 +76,14 @@ struct Geom3 {
   int cells, ncell, nact, n_m;
   uint64_t seed, replica;
   int cap_mem, cap_obj;  // bucket slots per cell; frame objects per cell
+  int cap_list;          // entries of the members' candidate lists, together
   int warp_bytes;        // shared memory of one warp's frame
   // FP32 screen: frame coordinates lie in (-sigma, w + sigma) and are
   // truncated to FP32 (integer pipes) with error < 2^-23 M (M >= w + sigma),
   // so FP32 differences (two truncations and one FP32 rounding of at most
-  // 2^-24 2M) are within d = 8 2^-24 M of the FP64 ones; a hit (b > 0,
-  // c^2 < sigma^2) then has b32 > -d and c2_32 < sigma^2 + 4 d sigma +
-  // 2 d^2 + FP32 rounding; the thresholds below are twice those bounds
-  float scr_b;           // pass iff b32 > -scr_b
+  // 2^-24 2M) are within d = 8 2^-24 M of the FP64 ones; c^2 < sigma^2 then
+  // has c2_32 < sigma^2 + 4 d sigma + 2 d^2 + FP32 rounding; the threshold
+  // below is twice that bound
   float scr_c2;          // pass iff c2_32 < scr_c2
   // L >= 2 (w + sigma): a periodic image X0 +- L of a wrapped coordinate
   // X0 in [-L/2, L/2) lies outside (-sigma, w + sigma), so only the
@@ -83,6 +96,10 @@ struct Geom3 {
   // the FP32 rounding of the coordinates the bin index is computed from
   int nbin;
   float inv_hb;          // 1 / bin side
+  int use_bins;          // the search for a member's candidates goes by bins
+  // a neighbour cell's sphere, by its FP32 position in that cell, can lie
+  // within sigma of this cell: above near_lo (cell below), below near_hi
+  float near_lo, near_hi;
   int replay;            // replay periodic rattles (results unchanged)
 };
 
@@ -138,24 +155,30 @@ __global__ void k3_begin(Geom3 g, State3* st, unsigned* sched) {
 __global__ void k3_bin(Geom3 g, const State3* __restrict__ st, const double* __restrict__ px,
                        const double* __restrict__ py, const double* __restrict__ pz,
                        int* __restrict__ cnt, int* __restrict__ ids, int* __restrict__ cell_of,
-                       int* err) {
+                       float4* __restrict__ rel, int* err) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.N) return;
   const State3 s = *st;
-  const int cx = cell_1d(px[i], s.s[0], g.L, g.inv_w, g.cells);
-  const int cy = cell_1d(py[i], s.s[1], g.L, g.inv_w, g.cells);
-  const int cz = cell_1d(pz[i], s.s[2], g.L, g.inv_w, g.cells);
+  const double x = px[i], y = py[i], z = pz[i];
+  const int cx = cell_1d(x, s.s[0], g.L, g.inv_w, g.cells);
+  const int cy = cell_1d(y, s.s[1], g.L, g.inv_w, g.cells);
+  const int cz = cell_1d(z, s.s[2], g.L, g.inv_w, g.cells);
   const int c = (cz * g.cells + cy) * g.cells + cx;
   cell_of[i] = c;
   const int slot = atomicAdd(&cnt[c], 1);
-  if (slot < g.cap_mem) ids[(int64_t)c * g.cap_mem + slot] = (int)i;
-  else atomicCAS(err, kOk, kCapacity);
-}
-
-// (s, key) before (bs, bk) for hit distances s, bs >= +0 (or +inf): the
-// bit patterns compare like the values
-__device__ __forceinline__ bool first_before(double s, long long k, double bs, long long bk) {
-  return lt_nn(s, bs) || (dbits(s) == dbits(bs) && k < bk);
+  if (slot >= g.cap_mem) {
+    atomicCAS(err, kOk, kCapacity);
+    return;
+  }
+  ids[(int64_t)c * g.cap_mem + slot] = (int)i;
+  if (rel != nullptr) {  // the position within the cell, and the id
+    const double hL = 0.5 * g.L;
+    rel[(int64_t)c * g.cap_mem + slot] = make_float4(
+        to_float_trunc(wrap_half_i(x - (s.s[0] + (double)cx * g.w), g.L, hL)),
+        to_float_trunc(wrap_half_i(y - (s.s[1] + (double)cy * g.w), g.L, hL)),
+        to_float_trunc(wrap_half_i(z - (s.s[2] + (double)cz * g.w), g.L, hL)),
+        __int_as_float((int)i));
+  }
 }
 
 // Cold paths of cell3, kept out of line so that the hot loop's code stays
@@ -181,30 +204,15 @@ __device__ __noinline__ unsigned images_mask3(double x0, double x1, double x2, d
   return mask;
 }
 
-// A lane's best candidate: hit distance, b, tie-break key, frame index.
-struct Hit3 {
-  double s, b;
-  long long k;
-  int j;
-};
-
-// The warp's first hit by (s, key) through a shuffle tree, for keys that do
-// not fit 32 bits (N >= 2^32 / 27).
-__device__ __noinline__ Hit3 first_hit_tree(Hit3 h) {
-#pragma unroll 1
-  for (int off = 16; off > 0; off >>= 1) {
-    const double os = __shfl_xor_sync(0xffffffffu, h.s, off);
-    const double ob = __shfl_xor_sync(0xffffffffu, h.b, off);
-    const long long ok2 = __shfl_xor_sync(0xffffffffu, h.k, off);
-    const int oj = __shfl_xor_sync(0xffffffffu, h.j, off);
-    if (first_before(os, ok2, h.s, h.k)) {
-      h.s = os;
-      h.b = ob;
-      h.k = ok2;
-      h.j = oj;
-    }
+// The lane of set `at` (the lanes whose hit distances are equal) with the
+// smallest key.
+__device__ __noinline__ int first_key3(unsigned at, long long key) {
+  int win = __ffs(at) - 1;
+  for (unsigned left = at & (at - 1); left != 0u; left &= left - 1u) {
+    const int l = __ffs(left) - 1;
+    if (__shfl_sync(0xffffffffu, key, l) < __shfl_sync(0xffffffffu, key, win)) win = l;
   }
-  return h;
+  return win;
 }
 
 // The distinct neighbour cells with two cells per side, where the cells at
@@ -224,6 +232,13 @@ __device__ __noinline__ void neighbour_list_small(int* nbl, int cx, int cy, int 
   nbl[26] = n;
 }
 
+// wrap_box0 with the comparisons on the integer pipes
+__device__ __forceinline__ double wrap_box_i(double v, double L) {
+  if (ecmc::dkey(v) < 0) v += L;
+  if (!dlt(v, L)) v -= L;
+  return v;
+}
+
 // Position loads: through L1 in the per-phase kernels (the writers finished
 // in an earlier launch), from L2 in the persistent kernel (the writers may
 // be warps of other SMs in the same launch).
@@ -240,7 +255,8 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
                                       unsigned char* base, double* __restrict__ px,
                                       double* __restrict__ py, double* __restrict__ pz,
                                       const int* __restrict__ cnt, const int* __restrict__ ids,
-                                      Cell3* __restrict__ cs, int* __restrict__ recs, int* err) {
+                                      float4* __restrict__ rel, Cell3* __restrict__ cs,
+                                      int* __restrict__ recs, int* err) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int colour = st.perm[colour_index];
@@ -253,34 +269,38 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
   const double o[3] = {st.s[0] + (double)cx * w, st.s[1] + (double)cy * w,
                        st.s[2] + (double)cz * w};
 
+  // the order of alignment; warp_bytes3 adds up the same sizes
   double* C[3];
   C[0] = reinterpret_cast<double*>(base);
   C[1] = C[0] + g.cap_obj;
   C[2] = C[1] + g.cap_obj;
-  long long* key = reinterpret_cast<long long*>(C[2] + g.cap_obj);
+  double* lroot = C[2] + g.cap_obj;  // candidate lists: sqrt(sigma^2 - c^2) ...
   // the chain's last kHist3 legs: start and end coordinate of the active
   // sphere along the axis, length, contact term bb - bs
-  double* hP = reinterpret_cast<double*>(key + g.cap_obj);
+  double* hP = lroot + g.cap_list;
   double* hE = hP + kHist3;
   double* hS = hE + kHist3;
   double* hT = hS + kHist3;
-  float* F[3];  // FP32 roundings of C, kept current as members move
-  F[0] = reinterpret_cast<float*>(hT + kHist3);
-  F[1] = F[0] + g.cap_obj;
-  F[2] = F[1] + g.cap_obj;
-  int* sid = reinterpret_cast<int*>(F[2] + g.cap_obj);  // members sorted by id
-  int* raw = sid + g.cap_mem;                           // members as bucketed
-  int* nbl = raw + g.cap_mem;                           // 26 neighbour cells + count
+  // FP32 roundings of the two coordinates across the axis (fixed)
+  float2* F = reinterpret_cast<float2*>(hT + kHist3);
+  int* oid = reinterpret_cast<int*>(F + g.cap_obj);     // sphere id of an object
+  int* sid = oid + g.cap_obj;                           // members sorted by id
+  int* lst = sid + g.cap_mem;  // a member's list (start << 16 | length) or -1
+  int* raw = lst;              // before: members as bucketed
+  int* nbl = lst + g.cap_mem;                           // 26 neighbour cells + count
   int* npre = nbl + 28;                                 // their bucket sizes, prefix sums
   int* hM = npre + 28;    // legs: active sphere, direction, kind (0 lift, 1 frozen, 2 wall)
   int* hSg = hM + kHist3;
   int* hK = hSg + kHist3;
-  int* cand = hK + kHist3;                              // FP32 screen survivors
-  int* ord = cand + g.cap_obj;                          // objects sorted by bin
-  const int nb = g.nbin, nb2 = nb * nb;
-  int* bst = ord + g.cap_obj;                           // bin starts, nb2 + 1
+  const int nb = g.nbin, nb2 = g.use_bins ? nb * nb : 0;
+  int* bst = hK + kHist3;                               // bin starts, nb2 + 1
   int* cur = bst + nb2 + 1;                             // scatter cursors, nb2
-  unsigned char* touched = reinterpret_cast<unsigned char*>(cur + nb2);
+  unsigned short* lidx = reinterpret_cast<unsigned short*>(cur + nb2);  // ... and objects
+  unsigned short* ord = lidx + g.cap_list;              // objects sorted by bin
+  // bucket slot of a member; the top bit: it has been active
+  unsigned short* mslot = ord + (g.use_bins ? g.cap_obj : 0);
+  unsigned char* oimg = reinterpret_cast<unsigned char*>(mslot + g.cap_mem);  // image 0..26
+  const int ax = st.axis, axp = ax == 0 ? 1 : 0, axq = ax == 2 ? 1 : 2;
 
   const int nmem = min(cnt[c], g.cap_mem);
   for (int k = lane; k < nmem; k += 32) raw[k] = ids[(int64_t)c * g.cap_mem + k];
@@ -303,6 +323,7 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
   // the neighbours' objects as one list: npre[e] = sum of the bucket sizes
   // of neighbours 0 .. e-1
   const int nnb = nbl[26];
+  const bool screen = g.single_image && rel != nullptr;  // (26 distinct neighbours)
   {
     const int nq = lane < nnb ? min(cnt[nbl[lane]], g.cap_mem) : 0;
     int incl = nq;
@@ -317,36 +338,37 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
   // members in ascending id (the rank of each is the number of smaller
   // ids); the positions are loaded before the rank is counted
   const double hL = 0.5 * L;
-  for (int k = lane; k < nmem; k += 32) {
+  for (int k0 = 0; k0 < nmem; k0 += 32) {
+    const int k = k0 + lane;
+    if (k >= nmem) continue;
     const int v = raw[k];
     const double mx = ldpos<CG>(px + v), my = ldpos<CG>(py + v), mz = ldpos<CG>(pz + v);
     int r = 0;
     for (int j = 0; j < nmem; ++j) r += raw[j] < v ? 1 : 0;
     sid[r] = v;
-    touched[r] = 0;
+    mslot[r] = (unsigned short)k;
     C[0][r] = wrap_half_i(mx - o[0], L, hL);
     C[1][r] = wrap_half_i(my - o[1], L, hL);
     C[2][r] = wrap_half_i(mz - o[2], L, hL);
-    F[0][r] = to_float_trunc(C[0][r]);
-    F[1][r] = to_float_trunc(C[1][r]);
-    F[2][r] = to_float_trunc(C[2][r]);
-    key[r] = (long long)v * 27 + 13;
+    oid[r] = v;
+    oimg[r] = 13;
   }
   __syncwarp();
+  for (int k = lane; k < nmem; k += 32) lst[k] = -1;  // (raw has been read)
   // frozen images, appended in the order (neighbour, bucket slot, image):
   // 32 entries of the neighbours' joint list per round, warp prefix sums
   int nobj = nmem;
   const double lo = -g.sigma, hi = w + g.sigma;
   const int ntot = npre[nnb];
   // the bucket slot of entry t of the joint list (t < ntot)
-  auto slot_of = [&](int t) {
+  auto slot_of = [&](int t) {  // (and the neighbour)
     int el = 0, eh = nnb;  // the neighbour e with npre[e] <= t < npre[e + 1]
     while (eh - el > 1) {
       const int mid = (el + eh) >> 1;
       if (npre[mid] <= t) el = mid;
       else eh = mid;
     }
-    return (int64_t)nbl[el] * g.cap_mem + (t - npre[el]);
+    return make_int2(nbl[el] * g.cap_mem + (t - npre[el]), el);
   };
   // one round: the entries of 32 lanes (valid where in) with their box
   // positions p, appended as frame objects in lane order
@@ -383,88 +405,115 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
         C[0][slot] = kx == 0 ? plus_zero(X0[0]) : X0[0] + (kx > 0 ? L : -L);
         C[1][slot] = ky == 0 ? plus_zero(X0[1]) : X0[1] + (ky > 0 ? L : -L);
         C[2][slot] = kz == 0 ? plus_zero(X0[2]) : X0[2] + (kz > 0 ? L : -L);
-        F[0][slot] = to_float_trunc(C[0][slot]);
-        F[1][slot] = to_float_trunc(C[1][slot]);
-        F[2][slot] = to_float_trunc(C[2][slot]);
-        key[slot] = (long long)id * 27 + img;
+        oid[slot] = id;
+        oimg[slot] = (unsigned char)img;
       }
       ++slot;
     }
     nobj += __shfl_sync(FULL, incl, 31);
   };
-  // two rounds per pass, their loads issued together so that the L2
-  // latencies overlap
-  for (int t0 = 0; t0 < ntot; t0 += 64) {
-    const int ta = t0 + lane, tb = t0 + 32 + lane;
-    const bool ina = ta < ntot, inb = tb < ntot;
-    const int ida = ina ? ids[slot_of(ta)] : 0;
-    const int idb = inb ? ids[slot_of(tb)] : 0;
-    double pa[3] = {0.0, 0.0, 0.0}, pb[3] = {0.0, 0.0, 0.0};
-    if (ina) {
-      pa[0] = ldpos<CG>(px + ida);
-      pa[1] = ldpos<CG>(py + ida);
-      pa[2] = ldpos<CG>(pz + ida);
-    }
-    if (inb) {
-      pb[0] = ldpos<CG>(px + idb);
-      pb[1] = ldpos<CG>(py + idb);
-      pb[2] = ldpos<CG>(pz + idb);
-    }
-    // one copy of the append code for both rounds
+  // Ids of the spheres to append.  With one image a sphere's FP32 position in
+  // its cell (rel) decides for all but a margin whether it comes near this
+  // cell: a neighbour's at offset -1 must lie above near_lo, at +1 below
+  // near_hi.  Of some 200 spheres in the 26 neighbours about 50 are left for
+  // the FP64 test.  Otherwise every sphere is tested.
+  int* const app = reinterpret_cast<int*>(lroot);  // (the lists come later)
+  const int cap_app = 2 * g.cap_list;
+  int n_app = 0;
+  if (screen) {
 #pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      if (h == 1 && t0 + 32 >= ntot) break;
-      const double q[3] = {h ? pb[0] : pa[0], h ? pb[1] : pa[1], h ? pb[2] : pa[2]};
-      append(h ? inb : ina, h ? idb : ida, q);
+    for (int t0 = 0; t0 < ntot; t0 += 64) {
+      bool near[2];
+      int id[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int t = t0 + 32 * h + lane;
+        near[h] = t < ntot;
+        id[h] = 0;
+        if (near[h]) {
+          const int2 q = slot_of(t);
+          const float4 f = __ldcg(rel + q.x);
+          const int e = q.y < 13 ? q.y : q.y + 1;
+          const int ez = e / 9, ey = (e - 9 * ez) / 3, ex = e - 9 * ez - 3 * ey;
+          near[h] = (ex == 1 || (ex == 0 ? f.x > g.near_lo : f.x < g.near_hi)) &&
+                    (ey == 1 || (ey == 0 ? f.y > g.near_lo : f.y < g.near_hi)) &&
+                    (ez == 1 || (ez == 0 ? f.z > g.near_lo : f.z < g.near_hi));
+          id[h] = __float_as_int(f.w);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const unsigned nbm = __ballot_sync(FULL, near[h]);
+        const int at = n_app + __popc(nbm & ((1u << lane) - 1u));
+        if (near[h] && at < cap_app) app[at] = id[h];
+        n_app += __popc(nbm);
+      }
     }
+    __syncwarp();
+  } else {
+    n_app = ntot;
   }
-  const bool ok = nobj <= g.cap_obj;
+#pragma unroll 1
+  for (int t0 = 0; t0 < n_app; t0 += 32) {
+    const int t = t0 + lane;
+    const bool in = t < n_app && (!screen || t < cap_app);
+    const int id = in ? (screen ? app[t] : ids[slot_of(t).x]) : 0;
+    double q[3] = {0.0, 0.0, 0.0};
+    if (in) {
+      q[0] = ldpos<CG>(px + id);
+      q[1] = ldpos<CG>(py + id);
+      q[2] = ldpos<CG>(pz + id);
+    }
+    append(in, id, q);
+  }
+  const bool ok = nobj <= g.cap_obj && !(screen && n_app > cap_app);
   if (!ok && lane == 0) atomicCAS(err, kOk, kCapacity);
   __syncwarp();
 
-  // bins across the sweep's axis (members move only along it, so the bins
-  // hold for the whole phase): counting sort of the objects, q-major
-  const int ax = st.axis, axp = ax == 0 ? 1 : 0, axq = ax == 2 ? 1 : 2;
+  // the coordinates across the sweep's axis, which members move along: these
+  // hold for the whole phase, and so do bins across it (counting sort of the
+  // objects, q-major)
   const float sigf = (float)g.sigma;
   auto bin_of = [&](float v) {
     const int b = (int)((v + sigf) * g.inv_hb);
     return b < 0 ? 0 : (b >= nb ? nb - 1 : b);
   };
   const int nobj_ok = ok ? nobj : 0;
-  for (int i = lane; i <= nb2; i += 32) bst[i] = 0;
-  __syncwarp();
   for (int o2 = lane; o2 < nobj_ok; o2 += 32)
-    atomicAdd(&bst[1 + bin_of(F[axq][o2]) * nb + bin_of(F[axp][o2])], 1);
+    F[o2] = make_float2(to_float_trunc(C[axp][o2]), to_float_trunc(C[axq][o2]));
   __syncwarp();
-  if (nb2 < 32) {
-    // bin starts by a warp scan of the counts (bst[0] = 0)
-    int v = lane <= nb2 ? bst[lane] : 0;
+  if (g.use_bins) {
+    for (int i = lane; i <= nb2; i += 32) bst[i] = 0;
+    __syncwarp();
+    for (int o2 = lane; o2 < nobj_ok; o2 += 32)
+      atomicAdd(&bst[1 + bin_of(F[o2].y) * nb + bin_of(F[o2].x)], 1);
+    __syncwarp();
+    int acc = 0;
+    for (int i0 = 0; i0 <= nb2; i0 += 32) {  // starts (bst[0] = 0)
+      int v = i0 + lane <= nb2 ? bst[i0 + lane] : 0;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int u = __shfl_up_sync(FULL, v, off);
-      if (lane >= off) v += u;
+      for (int off = 1; off < 32; off <<= 1) {
+        const int u = __shfl_up_sync(FULL, v, off);
+        if (lane >= off) v += u;
+      }
+      if (i0 + lane <= nb2) bst[i0 + lane] = acc + v;
+      acc += __shfl_sync(FULL, v, 31);
     }
-    if (lane <= nb2) bst[lane] = v;
-  } else if (lane == 0) {
-    for (int i = 1; i <= nb2; ++i) bst[i] += bst[i - 1];
+    __syncwarp();
+    for (int i = lane; i < nb2; i += 32) cur[i] = bst[i];
+    __syncwarp();
+    for (int o2 = lane; o2 < nobj_ok; o2 += 32)
+      ord[atomicAdd(&cur[bin_of(F[o2].y) * nb + bin_of(F[o2].x)], 1)] = (unsigned short)o2;
+    __syncwarp();
   }
-  __syncwarp();
-  for (int i = lane; i < nb2; i += 32) cur[i] = bst[i];
-  __syncwarp();
-  for (int o2 = lane; o2 < nobj_ok; o2 += 32)
-    ord[atomicAdd(&cur[bin_of(F[axq][o2]) * nb + bin_of(F[axp][o2])], 1)] = o2;
-  __syncwarp();
 
+  auto key_of = [&](int j) { return (long long)oid[j] * 27 + oimg[j]; };
   // the cell's chains
   double* CA = C[ax];
   double* CP = C[axp];
   double* CQ = C[axq];
-  float* FA = F[ax];
-  const float* FP = F[axp];
-  const float* FQ = F[axq];
   const double INF = __longlong_as_double(0x7ff0000000000000ll);
-  // keys id * 27 + image below 2^32 - 1: the reduction below may use 32-bit minima
-  const bool key32 = g.N * 27 < ((int64_t)1 << 32) - 27;
+  int n_list = 0;  // entries of the candidate lists in use
   double sum_b = 0.0;
   int n_ev = 0, n_li = 0, n_fr = 0, n_wa = 0, n_ch = 0, n_rep = 0;
   for (int k = 0; k < g.n_m; ++k) {
@@ -487,7 +536,7 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
     int ch_ev = 0, ch_wa = 0;
     int n_leg = 0;        // legs recorded in the history
     int64_t ch_rep = 0;   // legs of this chain replayed
-    if (lane == 0) touched[m] = 1;
+    if (lane == 0) mslot[m] |= 0x8000;
     ++n_ch;
     for (int64_t iter = 0;; ++iter) {
       if (iter + ch_rep >= ecmc::kMaxEventsPerChain) {
@@ -495,97 +544,112 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
         break;
       }
       __syncwarp();
-      const double P = CA[m], Pp = CP[m], Pq = CQ[m];
-      const float P32 = FA[m], Pp32 = FP[m], Pq32 = FQ[m];
+      const double P = CA[m];
       const double sw = clamp0(sg > 0 ? w - P : P);
-      double bs = INF, bb = 0.0;
-      long long bk = LLONG_MAX;
-      int bj = -1;
-      // candidates: the three rows of bins around the mover, each a
-      // contiguous run of ord[]; FP32 screen, survivors compacted into
-      // cand[] so that the FP64 tests below take one warp-wide pass
-      const int bpm = bin_of(Pp32), bqm = bin_of(Pq32);
-      const int plo = bpm > 0 ? bpm - 1 : 0, phi = bpm < nb - 1 ? bpm + 1 : nb - 1;
-      int rs[3], rl[3];
+      // The candidates of m: objects less than sigma away across the axis,
+      // c^2 < sigma^2.  Neither they nor sqrt(sigma^2 - c^2) change during
+      // the phase, so both are found when m first becomes active.
+      int list = lst[m];
+      if (list < 0) {
+        const double Pp = CP[m], Pq = CQ[m];
+        const float2 f = F[m];
+        int rs[3] = {0, 0, 0}, rl[3] = {nobj, 0, 0};
+        if (g.use_bins) {
+          // the three rows of bins around m, each a contiguous run of ord[]
+          const int bpm = bin_of(f.x), bqm = bin_of(f.y);
+          const int plo = bpm > 0 ? bpm - 1 : 0, phi = bpm < nb - 1 ? bpm + 1 : nb - 1;
 #pragma unroll
-      for (int k3 = 0; k3 < 3; ++k3) {
-        const int row = bqm - 1 + k3;
-        const bool in = row >= 0 && row < nb;
-        rs[k3] = in ? bst[row * nb + plo] : 0;
-        rl[k3] = in ? bst[row * nb + phi + 1] - rs[k3] : 0;
-      }
-      const int n_c = rl[0] + rl[1] + rl[2];
-      int ns = 0;
-      for (int t0 = 0; t0 < n_c; t0 += 32) {
-        const int t = t0 + lane;
-        bool pass = false;
-        int j = -1;
-        if (t < n_c) {
-          j = t < rl[0] ? ord[rs[0] + t]
-                        : (t < rl[0] + rl[1] ? ord[rs[1] + t - rl[0]]
-                                             : ord[rs[2] + t - rl[0] - rl[1]]);
+          for (int k3 = 0; k3 < 3; ++k3) {
+            const int row = bqm - 1 + k3;
+            const bool in = row >= 0 && row < nb;
+            rs[k3] = in ? bst[row * nb + plo] : 0;
+            rl[k3] = in ? bst[row * nb + phi + 1] - rs[k3] : 0;
+          }
         }
-        if (t < n_c && j != m) {
-          const float da32 = FA[j] - P32;
-          const float dp32 = FP[j] - Pp32, dq32 = FQ[j] - Pq32;
-          pass = ((sg > 0 ? da32 : -da32) > -g.scr_b) &&
-                 (dp32 * dp32 + dq32 * dq32 < g.scr_c2);
+        const int n_c = rl[0] + rl[1] + rl[2];
+        int nl = 0;
+#pragma unroll 1
+        for (int t0 = 0; t0 < n_c; t0 += 32) {  // FP32 screen
+          const int t = t0 + lane;
+          bool pass = false;
+          int j = t;
+          if (t < n_c) {
+            if (g.use_bins)
+              j = ord[t < rl[0] ? rs[0] + t
+                                : (t < rl[0] + rl[1] ? rs[1] + t - rl[0]
+                                                     : rs[2] + t - rl[0] - rl[1])];
+            const float2 fj = F[j];
+            const float dp32 = fj.x - f.x, dq32 = fj.y - f.y;
+            pass = j != m && dp32 * dp32 + dq32 * dq32 < g.scr_c2;
+          }
+          const unsigned bal = __ballot_sync(FULL, pass);
+          const int np = __popc(bal);
+          if (n_list + nl + np > g.cap_list) {
+            if (n_list == 0) {  // (a list is shorter than that: cap_list)
+              if (lane == 0) atomicCAS(err, kOk, kCapacity);
+              break;
+            }
+            // no room: drop the lists and start this one over
+            for (int q = lane; q < nmem; q += 32) lst[q] = -1;
+            n_list = 0;
+            nl = 0;
+            t0 = -32;
+            continue;
+          }
+          if (pass)
+            lidx[n_list + nl + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)j;
+          nl += np;
         }
-        const unsigned bal = __ballot_sync(FULL, pass);
-        if (pass) cand[ns + __popc(bal & ((1u << lane) - 1u))] = j;
-        ns += __popc(bal);
+        __syncwarp();
+        for (int t = lane; t < nl; t += 32) {
+          const int j = lidx[n_list + t];
+          const double dp = CP[j] - Pp;
+          const double dq = CQ[j] - Pq;
+          const double c2 = dp * dp + dq * dq;
+          // sigma^2 - c^2 is a positive normal number here (sigma in
+          // [2^-40, 2^40]), as sqrt_rn requires; an object that the screen
+          // let through is never hit: s = b + inf
+          lroot[n_list + t] = lt_nn(c2, g.sig2) ? sqrt_rn(g.sig2 - c2) : -INF;
+        }
+        list = n_list << 16 | nl;
+        if (lane == 0) lst[m] = list;
+        n_list += nl;
+        __syncwarp();
       }
-      __syncwarp();
-      for (int t = lane; t < ns; t += 32) {
-        const int j = cand[t];
-        const double da = CA[j] - P;
-        const double b = flip_if(da, sg < 0);
+      double bs = INF, bb = 0.0;
+      int bj = -1;
+      const int l0 = list >> 16, nl = list & 0xffff;
+      for (int t = lane; t < nl; t += 32) {
+        const int j = lidx[l0 + t];
+        const double b = flip_if(CA[j] - P, sg < 0);
         if (dbits(b) <= 0) continue;  // b > 0
-        const double dp = CP[j] - Pp;
-        const double dq = CQ[j] - Pq;
-        const double c2 = dp * dp + dq * dq;
-        if (!lt_nn(c2, g.sig2)) continue;
-        // sigma^2 - c^2 is a positive normal number here (sigma in
-        // [2^-40, 2^40]), as sqrt_rn requires
-        const double s = clamp0(b - sqrt_rn(g.sig2 - c2));
-        const long long kj = key[j];
-        if (first_before(s, kj, bs, bk)) {
+        const double s = clamp0(b - lroot[l0 + t]);
+        if (lt_nn(s, bs) || (dbits(s) == dbits(bs) && bj >= 0 && key_of(j) < key_of(bj))) {
           bs = s;
           bb = b;
-          bk = kj;
           bj = j;
         }
       }
-      if (key32) {
-        // the first hit by (s, key) with three hardware minima: s >= +0 (or
-        // +inf) orders as its bit pattern, compared high word then low word,
-        // and keys below 2^32 break exact ties; lanes without a candidate
-        // hold (+inf, max key)
+      {
+        // the first hit by (s, key): s >= +0 (or +inf) orders as its bit
+        // pattern, compared high word, then low word; keys break exact ties
         const unsigned long long sb = (unsigned long long)dbits(bs);
         const unsigned hi = (unsigned)(sb >> 32), lo = (unsigned)sb;
         const unsigned mhi = __reduce_min_sync(FULL, hi);
-        const unsigned mlo = __reduce_min_sync(FULL, hi == mhi ? lo : 0xffffffffu);
-        const bool at = hi == mhi && lo == mlo;
-        const unsigned k32 = bk == LLONG_MAX ? 0xffffffffu : (unsigned)bk;
-        const unsigned mk = __reduce_min_sync(FULL, at ? k32 : 0xffffffffu);
-        const int win = __ffs(__ballot_sync(FULL, at && k32 == mk)) - 1;
+        unsigned at = __ballot_sync(FULL, hi == mhi);
+        if (at & (at - 1)) {
+          const unsigned mlo = __reduce_min_sync(FULL, hi == mhi ? lo : 0xffffffffu);
+          at = __ballot_sync(FULL, hi == mhi && lo == mlo);
+          if ((at & (at - 1)) && mhi != 0x7ff00000u) at = 1u << first_key3(at, bj < 0 ? LLONG_MAX : key_of(bj));
+        }
+        const int win = __ffs(at) - 1;
         bs = __shfl_sync(FULL, bs, win);
         bb = __shfl_sync(FULL, bb, win);
-        bk = __shfl_sync(FULL, bk, win);
         bj = __shfl_sync(FULL, bj, win);
-      } else {
-        const Hit3 hw = first_hit_tree(Hit3{bs, bb, bk, bj});
-        bs = hw.s;
-        bb = hw.b;
-        bk = hw.k;
-        bj = hw.j;
       }
       __syncwarp();
       if (le_nn(r, bs) && le_nn(r, sw)) {  // budget used up
-        if (lane == 0) {
-          CA[m] = P + (sg > 0 ? r : -r);
-          FA[m] = to_float_trunc(CA[m]);
-        }
+        if (lane == 0) CA[m] = P + (sg > 0 ? r : -r);
         break;
       }
       const int hi = n_leg & (kHist3 - 1);
@@ -600,7 +664,6 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
         kind = bj < nmem ? 0 : 1;
         if (lane == 0) {
           CA[m] = z;
-          FA[m] = to_float_trunc(z);
           hP[hi] = P;
           hE[hi] = z;
           hS[hi] = bs;
@@ -618,7 +681,7 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
         if (kind == 0) {  // lift
           ++n_li;
           m = bj;
-          if (lane == 0) touched[m] = 1;
+          if (lane == 0) mslot[m] |= 0x8000;
         } else {  // frozen sphere: back along the axis
           sg = -sg;
           ++n_fr;
@@ -627,10 +690,10 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
         kind = 2;
         if (lane == 0) {
           CA[m] = sg > 0 ? w : 0.0;
-          FA[m] = to_float_trunc(CA[m]);
           hP[hi] = P;
           hE[hi] = CA[m];
           hS[hi] = sw;
+          hT[hi] = 0.0;
           hM[hi] = m;
           hSg[hi] = sg;
           hK[hi] = 2;
@@ -670,26 +733,41 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
         const unsigned pb = __ballot_sync(FULL, per);
         if (pb != 0u) {
           const int K = 2 * __ffs(pb), b0 = n_leg - K;
+          // whole legs while the budget exceeds them (a wall's contact term
+          // is +0: it leaves the sum as it is)
+          const int64_t n_max = ecmc::kMaxEventsPerChain - 1 - iter - ch_rep;
+          // (one FP64 addition a leg: lane 2 the sum, the others the budget)
+          const double* const hx = lane == 2 ? hT : hS;
+          double z = lane == 2 ? sum_b : r;
+          const int n_cap = n_max > INT_MAX ? INT_MAX : (int)n_max;
+          int n = 0;
           int j = 0;
-          for (;;) {  // whole legs while the budget exceeds them
-            const int ij = (b0 + j) & (kHist3 - 1);
-            const double st_j = hS[ij];
-            if (le_nn(r, st_j) || iter + ch_rep + 1 >= ecmc::kMaxEventsPerChain) break;
-            r = r - st_j;
-            const int kd = hK[ij];
-            if (kd == 2) {
-              ++n_wa;
-              ++ch_wa;
-            } else {
-              ++n_ev;
-              ++ch_ev;
-              if (kd == 0) ++n_li;
-              else ++n_fr;
-              if (lane == 2) sum_b += hT[ij];
-            }
-            ++ch_rep;
-            ++n_rep;
+#pragma unroll 1
+          for (; n < n_cap; ++n) {
+            const double x = hx[(b0 + j) & (kHist3 - 1)];
+            if (__ballot_sync(FULL, le_nn(z, x)) & 1u) break;
+            z = z + flip_if(x, lane != 2);
             j = j + 1 == K ? 0 : j + 1;
+          }
+          if (lane == 2) sum_b = z;
+          r = __shfl_sync(FULL, z, 0);
+          if (n > 0) {
+            const int kd = lane < K ? hK[(b0 + lane) & (kHist3 - 1)] : -1;
+            const unsigned part = (1u << j) - 1u;
+            const unsigned li = __ballot_sync(FULL, kd == 0), fr = __ballot_sync(FULL, kd == 1);
+            const unsigned wa = __ballot_sync(FULL, kd == 2);
+            const int whole = n / K;
+            const int d_li = whole * __popc(li) + __popc(li & part);
+            const int d_fr = whole * __popc(fr) + __popc(fr & part);
+            const int d_wa = whole * __popc(wa) + __popc(wa & part);
+            n_li += d_li;
+            n_fr += d_fr;
+            n_wa += d_wa;
+            ch_wa += d_wa;
+            n_ev += d_li + d_fr;
+            ch_ev += d_li + d_fr;
+            ch_rep += n;
+            n_rep += n;
           }
           // the frame is as at the start of leg b0 (and of every K legs
           // after it); the recorded legs b0 .. b0 + j - 1 bring it to the
@@ -699,7 +777,6 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
             for (int i = 0; i < j; ++i) {
               const int ii = (b0 + i) & (kHist3 - 1);
               CA[hM[ii]] = hE[ii];
-              FA[hM[ii]] = to_float_trunc(hE[ii]);
             }
           m = hM[(b0 + j) & (kHist3 - 1)];
           sg = hSg[(b0 + j) & (kHist3 - 1)];
@@ -718,11 +795,15 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
   __syncwarp();
   // members that moved, back in box coordinates
   for (int q = lane; q < nmem; q += 32) {
-    if (!touched[q]) continue;
+    if (!(mslot[q] & 0x8000)) continue;
     const int i = sid[q];
-    px[i] = wrap_box0(C[0][q] + o[0], L);
-    py[i] = wrap_box0(C[1][q] + o[1], L);
-    pz[i] = wrap_box0(C[2][q] + o[2], L);
+    px[i] = wrap_box_i(C[0][q] + o[0], L);
+    py[i] = wrap_box_i(C[1][q] + o[1], L);
+    pz[i] = wrap_box_i(C[2][q] + o[2], L);
+    if (rel != nullptr)
+      rel[(int64_t)c * g.cap_mem + (mslot[q] & 0x7fff)] =
+          make_float4(to_float_trunc(C[0][q]), to_float_trunc(C[1][q]), to_float_trunc(C[2][q]),
+                      __int_as_float(i));
   }
   sum_b = __shfl_sync(FULL, sum_b, 2);  // the contact sum is kept on lane 2
   if (lane == 0) {
@@ -742,14 +823,15 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
 __global__ void __launch_bounds__(32 * kWarpsMax) k3_phase(
     Geom3 g, const State3* __restrict__ stp, int colour_index, double* __restrict__ px,
     double* __restrict__ py, double* __restrict__ pz, const int* __restrict__ cnt,
-    const int* __restrict__ ids, Cell3* __restrict__ cs, int* __restrict__ recs, int* err) {
+    const int* __restrict__ ids, float4* __restrict__ rel, Cell3* __restrict__ cs,
+    int* __restrict__ recs, int* err) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int warp = threadIdx.x >> 5;
   const int a = blockIdx.x * (blockDim.x >> 5) + warp;
   if (a >= g.nact) return;  // warp-uniform
   const State3 st = *stp;
   cell3<false>(g, st, colour_index, a, smem + (size_t)warp * g.warp_bytes, px, py, pz, cnt, ids,
-               cs, recs, err);
+               rel, cs, recs, err);
 }
 
 __device__ __forceinline__ unsigned long long global_ns3() {
@@ -772,10 +854,13 @@ __device__ __forceinline__ unsigned load_volatile3(const unsigned* p) {
 // for smaller items, taken earlier by running warps that wait only for still
 // smaller ones.  Every wait is bounded (global timer): on timeout the kernel
 // raises kWaitTimeout and an abort flag that makes every warp leave.
-__global__ void __launch_bounds__(32 * kWarpsMax) k3_sweep(
+// (five blocks: 95 registers instead of 121 and no spills, 541 us against 563
+// at N = 64^3; six spill: 615)
+__global__ void __launch_bounds__(32 * kWarpsMax, 5) k3_sweep(
     Geom3 g, const State3* __restrict__ stp, double* __restrict__ px, double* __restrict__ py,
     double* __restrict__ pz, const int* __restrict__ cnt, const int* __restrict__ ids,
-    Cell3* __restrict__ cs, int* __restrict__ recs, unsigned* sched, unsigned* done,
+    float4* __restrict__ rel, Cell3* __restrict__ cs, int* __restrict__ recs, unsigned* sched,
+    unsigned* done,
     unsigned long long wait_ns, int wait_test, int* err) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr unsigned FULL = 0xffffffffu;
@@ -827,7 +912,7 @@ __global__ void __launch_bounds__(32 * kWarpsMax) k3_sweep(
     }
     if (!__all_sync(FULL, ok)) break;
     __threadfence();  // the finished neighbours' positions are visible from here on
-    cell3<true>(g, st, ci, a, base, px, py, pz, cnt, ids, cs, recs, err);
+    cell3<true>(g, st, ci, a, base, px, py, pz, cnt, ids, rel, cs, recs, err);
     __syncwarp();
     if (lane == 0) {
       __threadfence();
@@ -1088,7 +1173,9 @@ struct ecmc3_ctx {
   double* history = nullptr;
   int64_t* hist_len = nullptr;
   unsigned long long* u64 = nullptr;
-  uint4* fq = nullptr;  // fixed-point positions by bucket slot (overlap check)
+  // by bucket slot: fixed-point positions (overlap check) or FP32 positions
+  // within cells (sweeps); optional
+  uint4* fq = nullptr;
   int warps = 1;
   int64_t t_host = 0;
   bool valid = false;
@@ -1143,25 +1230,30 @@ int check3(ecmc3_ctx* h) {
   return ECMC_OK;
 }
 
+// Positions within cells by bucket slot, rewritten by every binning: in the
+// buffer of the overlap check, which keeps nothing there between calls.
+float4* rel3(const ecmc3_ctx* h) { return reinterpret_cast<float4*>(h->fq); }
+
 int enqueue_sweep(ecmc3_ctx* h, bool records) {
   const Geom3& g = h->g;
   CK3(cudaMemsetAsync(h->cnt, 0, sizeof(int) * (size_t)g.ncell, h->stream));
   k3_begin<<<1, 32, 0, h->stream>>>(g, h->st, h->sched);
   k3_bin<<<(unsigned)((g.N + 255) / 256), 256, 0, h->stream>>>(g, h->st, h->px, h->py, h->pz,
                                                                h->cnt, h->ids, h->cell_of,
-                                                               h->err);
+                                                               rel3(h), h->err);
   const int wpb = h->warps;
   const size_t sm = (size_t)wpb * g.warp_bytes;
   if (h->persistent && h->fused_blocks > 0) {
     k3_sweep<<<(unsigned)h->fused_blocks, 32 * wpb, sm, h->stream>>>(
-        g, h->st, h->px, h->py, h->pz, h->cnt, h->ids, h->cs, records ? h->recs : nullptr,
+        g, h->st, h->px, h->py, h->pz, h->cnt, h->ids, rel3(h), h->cs,
+        records ? h->recs : nullptr,
         h->sched, h->done, h->wait_ns, h->wait_test, h->err);
   } else {
     const unsigned blocks = (unsigned)((g.nact + wpb - 1) / wpb);
     for (int ci = 0; ci < 8; ++ci)
       k3_phase<<<blocks, 32 * wpb, sm, h->stream>>>(g, h->st, ci, h->px, h->py, h->pz, h->cnt,
-                                                    h->ids, h->cs, records ? h->recs : nullptr,
-                                                    h->err);
+                                                    h->ids, rel3(h), h->cs,
+                                                    records ? h->recs : nullptr, h->err);
   }
   k3_end<<<1, 256, 0, h->stream>>>(g, h->st, h->cs, h->tot, h->history, h->hist_len);
   CK3(cudaGetLastError());
@@ -1174,7 +1266,7 @@ int bin_now(ecmc3_ctx* h) {
   k3_begin<<<1, 32, 0, h->stream>>>(g, h->st, h->sched);
   k3_bin<<<(unsigned)((g.N + 255) / 256), 256, 0, h->stream>>>(g, h->st, h->px, h->py, h->pz,
                                                                h->cnt, h->ids, h->cell_of,
-                                                               h->err);
+                                                               rel3(h), h->err);
   CK3(cudaGetLastError());
   return ECMC_OK;
 }
@@ -1269,12 +1361,14 @@ void free3(ecmc3_ctx* h) {
 // shared memory of one warp's frame, and the launch's warps per block
 int layout3(ecmc3_ctx* h) {
   Geom3& g = h->g;
-  g.warp_bytes = (int)(((size_t)g.cap_obj * (3 * sizeof(double) + sizeof(long long) +
-                                             3 * sizeof(float) + 2 * sizeof(int)) +
-                        (size_t)(2 * g.nbin * g.nbin + 1) * sizeof(int) +
-                        (size_t)g.cap_mem * 2 * sizeof(int) + 56 * sizeof(int) +
-                        (size_t)kHist3 * (4 * sizeof(double) + 3 * sizeof(int)) +
-                        (size_t)g.cap_mem + 15) &
+  const size_t nb2 = g.use_bins ? (size_t)g.nbin * g.nbin : 0;
+  g.warp_bytes = (int)(((size_t)g.cap_obj * (3 * sizeof(double) + sizeof(float2) + sizeof(int) +
+                                             (g.use_bins ? sizeof(short) : 0) + 1) +
+                        (size_t)g.cap_list * (sizeof(double) + sizeof(short)) +
+                        (2 * nb2 + 1) * sizeof(int) +
+                        (size_t)g.cap_mem * (2 * sizeof(int) + sizeof(short)) +
+                        56 * sizeof(int) +
+                        (size_t)kHist3 * (4 * sizeof(double) + 3 * sizeof(int)) + 15) &
                        ~(size_t)15);
   int dev = 0, optin = 0, n_sm = 0;
   CK3(cudaGetDevice(&dev));
@@ -1360,7 +1454,6 @@ int ecmc3_create(ecmc3_t* out, int64_t N, double L, double sigma, int cells, dou
   {
     const double M = g.w + 2.0 * sigma;
     const double d = 8.0 * std::ldexp(1.0, -24) * M;
-    g.scr_b = (float)(2.0 * d);
     const double c2 = sigma * sigma + 4.0 * d * sigma + 2.0 * d * d +
                       4.0 * std::ldexp(1.0, -24) * (sigma * sigma + 4.0 * M * M);
     g.scr_c2 = std::nextafter((float)(sigma * sigma + 2.0 * (c2 - sigma * sigma)), 1e30f);
@@ -1377,6 +1470,22 @@ int ecmc3_create(ecmc3_t* out, int64_t N, double L, double sigma, int cells, dou
   g.cap_mem = sphere_bound(g.w, sigma);
   g.cap_obj = sphere_bound(g.w + 2.0 * sigma, sigma);
   if ((int64_t)g.cap_mem > N) g.cap_mem = (int)N;
+  {
+    // spheres with centres within sigma of a line of length w + 2 sigma: they
+    // lie in a cylinder of radius 1.5 sigma and length w + 3 sigma, none
+    // denser than pi / (3 sqrt 2); a list of candidates (the FP32 screen adds
+    // a skin of 2^-18 sigma) always fits, several usually do
+    const int one = (int)std::floor(10.01 * (g.w + 3.0 * sigma) / sigma) + 4;
+    int cap = g.cap_obj / 2 + 8 > 96 ? g.cap_obj / 2 + 8 : 96;
+    cap = cap > one ? cap : one;
+    g.cap_list = cap < g.cap_obj ? cap : g.cap_obj;
+    // up to four bins a side a member's three rows and columns are most of the
+    // frame, and the counting sort costs more than it spares
+    g.use_bins = g.nbin > 4 ? 1 : 0;
+    const double eps = 1e-6 * (g.w + sigma) + 1e-12 * L;
+    g.near_lo = (float)(g.w - sigma - eps);
+    g.near_hi = (float)(sigma + eps);
+  }
   if ((double)g.ncell * g.cap_mem > 2.0e9) {
     delete h;
     return fail3(ECMC_ERR_ARG, "too many cells");
