@@ -340,14 +340,14 @@ int compute_layout(ecmc_ctx* h) {
   int fmode = auto_fmode(h);
   h->tpc = choose_tpc(h, fmode);
   // isotropic chains in the persistent kernel: the fewest lanes per cell that
-  // leave five warps per SM something to do in a colour phase, and not fewer
+  // leave twenty warps per SM something to do in a colour phase, and not fewer
   // than the frames' size asks for.  Measured on GB300, us per sweep with 4 / 8
-  // / 16 / 32 lanes at eta = 0.708, ell = 1.06: 4519 / 5299 / 7379 / 10073 at N =
-  // 2^20, 240^2 cells; 2657 / 2294 / 2433 / 2853 at 2^18, 120^2; 2478 / 1889 /
-  // 1523 / 1377 at 2^16, 60^2; 2160 / 1604 / 1226 / 955 at 2^12, 14^2
+  // / 16 / 32 lanes at eta = 0.708, ell = 1.06: 2796 / 2458 / 2739 / 3121 at N =
+  // 2^20, 240^2 cells; 1619 / 1191 / 1057 / 967 at 2^18, 120^2; 1503 / 1019 /
+  // 755 / 619 at 2^16, 60^2; 1327 / 885 / 624 / 472 at 2^12, 14^2
   if (chain_kind(h->b) == 1 && h->persist_param && !h->tpc_param && fmode < 2) {
     int t = h->tpc;
-    while (t < 32 && (int64_t)h->b.A_total * t / 32 < 5 * h->n_sm) t *= 2;
+    while (t < 32 && (int64_t)h->b.A_total * t / 32 < 20 * h->n_sm) t *= 2;
     if (phase_smem_bytes(layout_for(h, t), 1, fmode) <= limit &&
         fused_smem_bytes(layout_for(h, t)) <= limit / 2)
       h->tpc = t;

@@ -27,6 +27,21 @@
 // distance) are tested in FP64, so the first hit and the new position are
 // those of the full FP64 search.  Either way trajectories are bit-identical to
 // the reference.  Frames are built with axis 0 (frame coordinates a = x, b = y).
+//
+// What bounds it: the chain's serial dependence and the FP64 pipe, which one
+// warp instruction holds for some 57 cycles of its scheduler however few lanes
+// take part.  So a vector's components are shared out between two lanes (one
+// FP64 instruction for both), comparisons run on the integer pipes, the wall
+// distances are bounded in FP32 and divided exactly only where a wall can come
+// first (one division for both axes instead of one per axis and sign), and the
+// one candidate that the screen leaves in most events is tested by the whole
+// group, without a reduction.  About 45 FP64 instructions an event where there
+// were 130.  GB300, us per sweep at eta = 0.708, ell = 1.06, n_m = 2:
+//   N = 2^20, 240^2 cells: 2457 / 4522,  2^18, 120^2: 964 / 2281,
+//   2^16, 60^2: 619 / 1345,  2^12, 14^2: 470 / 953;
+//   2^16, 32^2 cells, ell = 8, n_m = 1: 1470 / 3091
+// against every lane doing all of an event's scalar work (with the lanes per
+// cell that were then the best).
 #pragma once
 
 #include "ecmc_chain.cuh"
@@ -59,19 +74,29 @@ __device__ __forceinline__ void iso_direction(int64_t t, int lc, int k, uint64_t
   dy = 0.0;
 }
 
+// `better` for distances >= +0 (or +inf), on the integer pipes
+__device__ __forceinline__ bool better_nn(double s, int key, double bs, int bkey) {
+  return lt_nn(s, bs) || (dbits(s) == dbits(bs) && key < bkey);
+}
+
 // FP64 hit test of candidate j along d, the reference expressions
 __device__ __forceinline__ bool iso_hit(const Frame& f, int j, int CPW, int gi, double X, double Y,
                                         double dx, double dy, double sig2, double& s, double& b) {
   const double ddx = f.a64[j * CPW + gi] - X;
   const double ddy = f.b64[j * CPW + gi] - Y;
   b = ddx * dx + ddy * dy;
-  if (!(b > 0.0)) return false;
+  if (dbits(b) <= 0) return false;
   const double cc = ddx * dy - ddy * dx;
   const double c2 = cc * cc;
-  if (!(c2 < sig2)) return false;
-  s = b - sqrt_rn(sig2 - c2);
-  if (s < 0.0) s = 0.0;
+  if (!lt_nn(c2, sig2)) return false;
+  s = clamp0(b - sqrt_rn(sig2 - c2));
   return true;
+}
+
+__device__ __forceinline__ float iso_sqrt(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // FP32 bracket [lo, hi] of the hit distance of candidate j (certain: j hits
@@ -90,8 +115,9 @@ __device__ __forceinline__ bool iso_bracket(const Frame& f, const Geom& g, int j
   const float cl = fmaxf(__fsub_rn(ac, e), 0.0f), ch = __fadd_rn(ac, e);
   const float xhi = fmaxf(__fsub_rn(g.sig2f, __fmul_rn(cl, cl)), 0.0f);
   const float xlo = fmaxf(__fsub_rn(g.sig2f, __fmul_rn(ch, ch)), 0.0f);
-  const float sq_hi = __fadd_rn(__fsqrt_rn(xhi), g.iso_sq);
-  const float sq_lo = fmaxf(__fsub_rn(__fsqrt_rn(xlo), g.iso_sq), 0.0f);
+  // (iso_sq leaves 2^-14 sigma for the SFU root's error of 2^-23 sigma)
+  const float sq_hi = __fadd_rn(iso_sqrt(xhi), g.iso_sq);
+  const float sq_lo = fmaxf(__fsub_rn(iso_sqrt(xlo), g.iso_sq), 0.0f);
   lo = __fsub_rn(__fsub_rn(__fsub_rn(b32, e), sq_hi), g.iso_r);
   hi = fmaxf(__fadd_rn(__fsub_rn(__fadd_rn(b32, e), sq_lo), g.iso_r), 0.0f);
   certain = __fsub_rn(b32, e) > 0.0f && __fadd_rn(ch, e) < g.iso_sig_lo;
@@ -132,6 +158,23 @@ __device__ __forceinline__ void run_group_iso(const Frame& f, const int* hdr, vo
   bool active = false;
   int m = 0;
   double X = 0.0, Y = 0.0, dx = 1.0, dy = 0.0, r = 0.0;
+  float dx32 = 1.0f, dy32 = 0.0f;  // the direction rounded to FP32
+  // Two lanes share the work on the two components of a vector: `own` picks
+  // this lane's component, `both` hands each lane the pair.
+  constexpr int NC = TPC >= 2 ? 1 : 2;
+  const int par = sub & 1;
+  auto own = [&](double x, double y, int q) { return (NC == 1 ? par : q) ? y : x; };
+  auto both = [&](const double* v, double& x, double& y) {
+    if constexpr (NC == 1) {
+      const double o = __shfl_xor_sync(FULL, v[0], 1);
+      x = par ? o : v[0];
+      y = par ? v[0] : o;
+    } else {
+      x = v[0];
+      y = v[NC - 1];
+    }
+  };
+  const float Wf = to_float_trunc(W), Hf = to_float_trunc(H);
   int64_t n_iter = 0;
   int ch_events = 0, ch_walls = 0, start_key = 0;
   bool done = (!valid) || nmem == 0;
@@ -151,6 +194,8 @@ __device__ __forceinline__ void run_group_iso(const Frame& f, const int* hdr, vo
         }
         m = f.mrank[idx * CPW + gi];
         iso_direction(t, lc, k, g.seed, g.replica, dx, dy);
+        dx32 = __double2float_rn(dx);
+        dy32 = __double2float_rn(dy);
         X = f.a64[m * CPW + gi];
         Y = f.b64[m * CPW + gi];
         r = g.ell;
@@ -170,26 +215,36 @@ __device__ __forceinline__ void run_group_iso(const Frame& f, const int* hdr, vo
     if (capped) atomicCAS(err, DEV_OK, DEV_CHAIN_CAP);
     const bool go = live && !capped;
 
-    // distances to the walls along d
-    double swx = INF, swy = INF;
-    if (dx > 0.0) swx = (W - X) / fabs(dx);
-    else if (dx < 0.0) swx = X / fabs(dx);
-    if (dy > 0.0) swy = (H - Y) / fabs(dy);
-    else if (dy < 0.0) swy = Y / fabs(dy);
-    if (swx < 0.0) swx = 0.0;
-    if (swy < 0.0) swy = 0.0;
-    const double swall = swx < swy ? swx : swy;
+    // FP32 bounds of the distance to the walls along d
+    const float X32 = to_float_trunc(X), Y32 = to_float_trunc(Y);
+    float wall_lo, wall_hi;
+    {
+      const float ax = fabsf(dx32), ay = fabsf(dy32);
+      float nx = dx32 > 0.0f ? Wf - X32 : X32, ny = dy32 > 0.0f ? Hf - Y32 : Y32;
+      if (ax < 0x1p-20f) nx = fminf(X32, Wf - X32);  // (its sign may be lost)
+      if (ay < 0x1p-20f) ny = fminf(Y32, Hf - Y32);
+      // numerators within iso_e; FP32 direction within 2^-24, quotients within
+      // the factors
+      const float qx = __fdividef(fmaxf(nx - g.iso_e, 0.0f), ax + 0x1p-20f);
+      const float qy = __fdividef(fmaxf(ny - g.iso_e, 0.0f), ay + 0x1p-20f);
+      wall_lo = fminf(qx, qy) * (1.0f - 0x1p-19f);
+      const float INF32 = __int_as_float(0x7f800000);
+      const float hx = ax > 0x1p-8f ? __fdividef(nx + g.iso_e, ax) : INF32;
+      const float hy = ay > 0x1p-8f ? __fdividef(ny + g.iso_e, ay) : INF32;
+      wall_hi = fminf(hx, hy) * (1.0f + 0x1p-12f);
+    }
 
     // first contact along d
     double best_s = INF, best_b = 0.0;
     int best_key = INT_MAX, best_j = m;
-    int nev = 0;
+    int nev = 0;     // FP64 evaluations (summed over the cell's lanes)
+    bool multi = go;  // the exact tests run over all the lanes
     auto consider = [&](int j) {
       double s, b;
       ++nev;
       if (iso_hit(f, j, CPW, gi, X, Y, dx, dy, sig2, s, b)) {
         const int kj = f.key[j * CPW + gi];
-        if (better(s, kj, best_s, best_key)) {
+        if (better_nn(s, kj, best_s, best_key)) {
           best_s = s;
           best_b = b;
           best_key = kj;
@@ -199,8 +254,6 @@ __device__ __forceinline__ void run_group_iso(const Frame& f, const int* hdr, vo
     };
     if (SCREEN) {
       // FP32 brackets; the candidates that can be the first hit go to FP64
-      const float X32 = to_float_trunc(X), Y32 = to_float_trunc(Y);
-      const float dx32 = __double2float_rn(dx), dy32 = __double2float_rn(dy);
       float U = __int_as_float(0x7f800000), L1 = U, L2 = U;
       int j1 = m;
       if (go) {
@@ -235,26 +288,45 @@ __device__ __forceinline__ void run_group_iso(const Frame& f, const int* hdr, vo
           L2 = nL2;
         }
       }
-      const float Lam = fminf(U, to_float_up_nn(r < swall ? r : swall));
+      const float Lam = fminf(U, fminf(to_float_up_nn(r), wall_hi));
       const bool need = go && (L1 <= Lam);
-      const bool multi = need && (L2 <= Lam);
-      if (need && !multi && sub == 0) consider(j1);
-      if (__any_sync(FULL, multi)) {
-        if (multi) {
-          for (int j = sub; j < nobj; j += TPC) {
-            if (j == m) continue;
-            float lo, hi;
-            bool certain;
-            if (!iso_bracket(f, g, j, CPW, gi, X32, Y32, dx32, dy32, lo, hi, certain)) continue;
-            if (lo <= Lam) consider(j);
-          }
+      multi = need && (L2 <= Lam);
+      // one candidate: iso_hit, a component a lane
+      const bool one = need && !multi;
+      const int jc = one ? j1 : m;
+      double v[NC], w2[NC], vx, vy;
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        const double dd = own(f.a64[jc * CPW + gi], f.b64[jc * CPW + gi], q) - own(X, Y, q);
+        v[q] = dd * own(dx, dy, q);
+        w2[q] = dd * own(dy, dx, q);
+      }
+      both(v, vx, vy);
+      const double b = vx + vy;
+      both(w2, vx, vy);
+      const double cc = vx - vy;
+      const double c2 = cc * cc;
+      if (one && dbits(b) > 0 && lt_nn(c2, sig2)) {
+        best_s = clamp0(b - sqrt_rn(sig2 - c2));
+        best_b = b;
+        best_key = f.key[jc * CPW + gi];
+        best_j = jc;
+      }
+      nev = one && sub == 0 ? 1 : 0;
+      if (multi) {
+        for (int j = sub; j < nobj; j += TPC) {
+          if (j == m) continue;
+          float lo, hi;
+          bool certain;
+          if (!iso_bracket(f, g, j, CPW, gi, X32, Y32, dx32, dy32, lo, hi, certain)) continue;
+          if (lo <= Lam) consider(j);
         }
       }
     } else if (go) {
       for (int j = sub; j < nobj; j += TPC)
         if (j != m) consider(j);
     }
-    if (TPC > 1) {
+    if (TPC > 1 && __any_sync(FULL, multi)) {
 #pragma unroll
       for (int o = 1; o < TPC; o <<= 1) {
         const double os = __shfl_xor_sync(FULL, best_s, o);
@@ -262,7 +334,7 @@ __device__ __forceinline__ void run_group_iso(const Frame& f, const int* hdr, vo
         const int ok = __shfl_xor_sync(FULL, best_key, o);
         const int oj = __shfl_xor_sync(FULL, best_j, o);
         nev += __shfl_xor_sync(FULL, nev, o);
-        if (better(os, ok, best_s, best_key)) {
+        if (better_nn(os, ok, best_s, best_key)) {
           best_s = os;
           best_b = ob;
           best_key = ok;
@@ -272,60 +344,108 @@ __device__ __forceinline__ void run_group_iso(const Frame& f, const int* hdr, vo
     }
     n_fp64 += go ? nev : 0;
 
-    bool end_chain = capped;
-    if (go) {
-      if (r <= best_s && r <= swall) {
-        // budget used up: the chain ends
-        X = X + r * dx;
-        Y = Y + r * dy;
-        end_chain = true;
-      } else if (best_s <= swall) {
-        const double s = best_s;
-        const double nX = X + s * dx, nY = Y + s * dy;
-        r = r - s;
-        sum_b += best_b - s;
-        ++n_events;
-        ++ch_events;
-        ++n_iter;
-        if (f.info[best_j * CPW + gi] >= 0) {
-          // lift: the hit member moves on along d
-          ++n_lifts;
-          // the stopped disk, in FP64 and in the FP32 copy the screen reads
-          f.a64[m * CPW + gi] = nX;
-          f.b64[m * CPW + gi] = nY;
-          f.a32[m * CPW + gi] = to_float_trunc(nX);
-          f.b32[m * CPW + gi] = to_float_trunc(nY);
-          m = best_j;
-          X = f.a64[m * CPW + gi];
-          Y = f.b64[m * CPW + gi];
-          f.touched[m * CPW + gi] = 1;
-        } else {
-          // frozen disk: specular reflection about the line of centres
-          ++n_frozen;
-          const double nx = f.a64[best_j * CPW + gi] - nX;
-          const double ny = f.b64[best_j * CPW + gi] - nY;
-          const double nn = nx * nx + ny * ny;
-          const double kk = 2.0 * (dx * nx + dy * ny) / nn;
-          dx = dx - kk * nx;
-          dy = dy - kk * ny;
-          X = nX;
-          Y = nY;
-        }
-      } else {
-        // wall: onto the wall, flip the normal component(s)
-        const double s = swall;
-        const bool flip_x = swx == swall, flip_y = swy == swall;
-        const double nX = flip_x ? (dx > 0.0 ? W : 0.0) : X + s * dx;
-        const double nY = flip_y ? (dy > 0.0 ? H : 0.0) : Y + s * dy;
-        X = nX;
-        Y = nY;
-        if (flip_x) dx = -dx;
-        if (flip_y) dy = -dy;
-        r = r - s;
-        ++n_walls;
-        ++ch_walls;
-        ++n_iter;
+    // Exact wall distances, unless the bounds leave no doubt: one division a
+    // lane, for a component each.  Without doubt they count as infinite.
+    const double q0 = min_nn(r, best_s);
+    const bool need_wall = go && !(to_float_up_nn(q0) < wall_lo);
+    double swx = INF, swy = INF;
+    if (__any_sync(FULL, need_wall)) {
+      double sw[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        const double P = own(X, Y, q), D = own(dx, dy, q);
+        const long long kD = dkey(D);
+        const double up = own(W, H, q) - P;
+        const double num = kD > 0 ? up : P;
+        const double den = kD == 0 ? 1.0 : flip_if(D, kD < 0);
+        sw[q] = kD == 0 ? INF : clamp0(num / den);
       }
+      both(sw, swx, swy);
+      swx = need_wall ? swx : INF;
+      swy = need_wall ? swy : INF;
+    }
+    const double swall = min_nn(swx, swy);
+
+    const bool is_end = go && le_nn(r, best_s) && le_nn(r, swall);  // budget used up
+    const bool is_hit = go && !is_end && le_nn(best_s, swall);
+    const bool is_wall = go && !is_end && !is_hit;
+    const bool flip_x = is_wall && dbits(swx) == dbits(swall);
+    const bool flip_y = is_wall && dbits(swy) == dbits(swall);
+    const double s = is_end ? r : (is_hit ? best_s : (is_wall ? swall : 0.0));
+    double v[NC], u[NC], nX, nY, r1, db;
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const double D = own(dx, dy, q);
+      v[q] = own(X, Y, q) + s * D;
+      // onto the wall
+      if ((NC == 1 ? par : q) ? flip_y : flip_x) v[q] = dkey(D) > 0 ? own(W, H, q) : 0.0;
+      u[q] = own(r, best_b, q) - s;
+    }
+    both(v, nX, nY);
+    both(u, r1, db);
+    bool end_chain = capped || is_end;
+    bool frozen = false;
+    if (is_hit) {
+      r = r1;
+      sum_b += db;
+      ++n_events;
+      ++ch_events;
+      ++n_iter;
+      frozen = f.info[best_j * CPW + gi] < 0;
+    } else if (is_wall) {  // the normal component(s) flip
+      r = r1;
+      if (flip_x) {
+        dx = -dx;
+        dx32 = -dx32;
+      }
+      if (flip_y) {
+        dy = -dy;
+        dy32 = -dy32;
+      }
+      ++n_walls;
+      ++ch_walls;
+      ++n_iter;
+    }
+    if (__any_sync(FULL, frozen)) {
+      // frozen disk: specular reflection about the line of centres
+      double n1[NC], n2[NC], n3[NC], vx, vy;
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        n1[q] = own(f.a64[best_j * CPW + gi], f.b64[best_j * CPW + gi], q) - own(nX, nY, q);
+        n2[q] = n1[q] * n1[q];
+        n3[q] = own(dx, dy, q) * n1[q];
+      }
+      both(n2, vx, vy);
+      const double nn = vx + vy;
+      both(n3, vx, vy);
+      const double dot = vx + vy;
+      const double kk = 2.0 * dot / (frozen ? nn : 1.0);
+#pragma unroll
+      for (int q = 0; q < NC; ++q) n1[q] = own(dx, dy, q) - kk * n1[q];
+      both(n1, vx, vy);
+      if (frozen) {
+        ++n_frozen;
+        dx = vx;
+        dy = vy;
+        dx32 = __double2float_rn(dx);
+        dy32 = __double2float_rn(dy);
+      }
+    }
+    if (is_hit && !frozen) {
+      // lift: the hit member moves on along d
+      ++n_lifts;
+      // the stopped disk, in FP64 and in the FP32 copy the screen reads
+      f.a64[m * CPW + gi] = nX;
+      f.b64[m * CPW + gi] = nY;
+      f.a32[m * CPW + gi] = to_float_trunc(nX);
+      f.b32[m * CPW + gi] = to_float_trunc(nY);
+      m = best_j;
+      X = f.a64[m * CPW + gi];
+      Y = f.b64[m * CPW + gi];
+      f.touched[m * CPW + gi] = 1;
+    } else if (go) {
+      X = nX;
+      Y = nY;
     }
     if (end_chain) {
       f.a64[m * CPW + gi] = X;
