@@ -47,6 +47,13 @@ namespace ecmc {
 int report_error(int code, const char* msg) { return fail(code, "%s", msg); }
 }  // namespace ecmc
 
+constexpr int64_t kPinHistory = 1024;  // sweeps
+struct PinRead {
+  int err;
+  RunTotals totals;
+  double history[2 * kPinHistory];
+};
+
 struct ecmc_ctx {
   std::vector<Geom> geo;        // host copy of every replica's geometry
   std::vector<int> cell_rep;    // replica of every global cell
@@ -113,6 +120,10 @@ struct ecmc_ctx {
   // synchronisation
   SweepState* pin_states = nullptr;       // [R]
   unsigned long long* pin_bits = nullptr;  // [2]: initial and resulting minimum
+  // and for what a caller reads back between sweeps: copies into pageable
+  // memory wait for the stream one by one (a replica's pressure took three
+  // such waits, 30 us; one now)
+  PinRead* pin_read = nullptr;
 };
 
 namespace {
@@ -529,9 +540,10 @@ int ensure_history(ecmc_ctx* h, int64_t extra) {
 }
 
 int check_device_error(ecmc_ctx* h) {
-  int e = 0;
-  CK(cudaMemcpyAsync(&e, h->b.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaMemcpyAsync(&h->pin_read->err, h->b.err, sizeof(int), cudaMemcpyDeviceToHost,
+                     h->stream));
   CK(cudaStreamSynchronize(h->stream));
+  const int e = h->pin_read->err;
   if (h->timing) harvest_timing(h);
   if (e == DEV_CAPACITY) {
     h->valid_state = false;
@@ -671,6 +683,7 @@ void free_all(ecmc_ctx* h) {
   cudaFree(h->undo);
   cudaFreeHost(h->pin_states);
   cudaFreeHost(h->pin_bits);
+  cudaFreeHost(h->pin_read);
   for (auto& e : h->pending) {
     cudaEventDestroy(e.a);
     cudaEventDestroy(e.b);
@@ -851,7 +864,8 @@ int create_impl(ecmc_t* out, const ecmc_replica_desc_t* desc, int R) {
       cudaMalloc(&h->int_tmp, sizeof(int) * (size_t)N_total) != cudaSuccess ||
       cudaMalloc(&h->u64_tmp, sizeof(unsigned long long) * 4) != cudaSuccess ||
       cudaMallocHost(&h->pin_states, sizeof(SweepState) * R) != cudaSuccess ||
-      cudaMallocHost(&h->pin_bits, sizeof(unsigned long long) * 2) != cudaSuccess)
+      cudaMallocHost(&h->pin_bits, sizeof(unsigned long long) * 2) != cudaSuccess ||
+      cudaMallocHost(&h->pin_read, sizeof(PinRead)) != cudaSuccess)
     return bail(fail(ECMC_ERR_OOM, "device allocation failed"));
   cudaMemsetAsync(b.totals, 0, sizeof(RunTotals) * R, h->stream);
   cudaMemsetAsync(b.err, 0, sizeof(int), h->stream);
@@ -912,13 +926,17 @@ int pressure_of(ecmc_ctx* h, int r, double* betaP, double* se) {
   const int64_t n = h->hist_len_host < h->b.history_cap ? h->hist_len_host : h->b.history_cap;
   if (n < 1) return fail(ECMC_ERR_STATE, "no sweep since the last reset");
   const Geom& g = h->geo[r];
-  std::vector<double> hist(2 * (size_t)n);
-  CK(cudaMemcpyAsync(hist.data(), h->b.history + 2 * (size_t)r * h->b.history_cap,
-                     sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, h->stream));
-  RunTotals t;
-  CK(cudaMemcpyAsync(&t, h->b.totals + r, sizeof(t), cudaMemcpyDeviceToHost, h->stream));
+  const bool long_run = n > kPinHistory;
+  std::vector<double> long_hist(long_run && se ? 2 * (size_t)n : 0);
+  double* const hist = long_run ? long_hist.data() : h->pin_read->history;
+  if (se)
+    CK(cudaMemcpyAsync(hist, h->b.history + 2 * (size_t)r * h->b.history_cap,
+                       sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaMemcpyAsync(&h->pin_read->totals, h->b.totals + r, sizeof(RunTotals),
+                     cudaMemcpyDeviceToHost, h->stream));
   int rc = check_device_error(h);
   if (rc) return rc;
+  const RunTotals t = h->pin_read->totals;
   const double rho_s2 = (double)g.N / (g.L * g.L) * g.sig2;
   if (!(t.sum_disp_w > 0.0)) return fail(ECMC_ERR_STATE, "no displacement since the last reset");
   *betaP = rho_s2 * (1.0 + t.sum_b_w / t.sum_disp_w);
@@ -1331,10 +1349,8 @@ int ecmc_reset_stats(ecmc_t h) {
   if (!h) return fail(ECMC_ERR_ARG, "NULL handle");
   CK(cudaStreamSynchronize(h->stream));
   CK(cudaMemsetAsync(h->b.totals, 0, sizeof(RunTotals) * h->b.R, h->stream));
-  const int64_t zero = 0;
-  for (int r = 0; r < h->b.R; ++r)
-    CK(cudaMemcpyAsync((char*)(h->b.state + r) + offsetof(SweepState, history_len), &zero,
-                       sizeof(zero), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemset2DAsync((char*)h->b.state + offsetof(SweepState, history_len), sizeof(SweepState),
+                       0, sizeof(int64_t), (size_t)h->b.R, h->stream));
   h->hist_len_host = 0;
   CK(cudaMemsetAsync(h->gr_counts, 0, sizeof(unsigned long long) * h->gr_nbins * h->geo.size(),
                      h->stream));
