@@ -40,23 +40,23 @@ UNIT = "events/s"
 # FP64 (16 B) coordinates, plus 16 B to read and write the active disk
 # (smem_bytes_per_event below).
 #
-# Counters of the persistent sweep kernel k_sweep_fused<8 lanes per cell,
-# FP32 screening, axis chains> that need more than one ncu pass, for both
-# placements of the FP64 frame coordinates the autotuner chooses between
-# (frame mode 1, global scratch: its choice at N = 1M; frame mode 0, shared
-# memory): captured at N = 640,000, eta = 0.72 with the paper's parameters
-# (188 x 188 cells, about 8,800 active cells per phase), one launch = one sweep
-# (profiles/k_sweep_fused_n640k_paper_params.md); the full-size workload is
-# profiled with single-pass metric sets only.  Both scale with the work:
-# DRAM bytes with the disks (every cell and its halo are read once per colour
-# phase), FP64 warp-instructions with the event-loop iterations.
+# Counters of the persistent sweep kernel k_sweep_axis<8 lanes per cell> that
+# need more than one ncu pass, for both placements of the frame coordinates
+# the autotuner chooses between (frame mode 1, global scratch; frame mode 0,
+# shared memory): captured at N = 640,000, eta = 0.72 with the parameters of
+# the full size (188 x 188 cells, about 8,800 active cells per phase), one
+# launch = one sweep (profiles/k_sweep_axis_n640k_paper_params.md); the
+# full-size workload is profiled with single-pass metric sets only.  Both
+# scale with the work: DRAM bytes with the disks (every cell and its halo are
+# read once per colour phase), FP64 warp-instructions with the event-loop
+# iterations.
 FUSED_CAPTURE_N = 640000
-FUSED_ITERATIONS_CAPTURE = 1524505               # contacts + walls + chain ends per launch
+FUSED_ITERATIONS_CAPTURE = 1526651               # contacts + walls + chain ends per launch
 FUSED_CAPTURES = {
     # frame mode: dram__bytes_read.sum + _write.sum, smsp__inst_executed_pipe_fp64.sum,
     # sm__pipe_fp64_cycles_active (% of active cycles)
-    1: {"dram_bytes": 24786688 + 492544, "fp64_winst": 5594937, "fp64_pipe_pct": 37.95},
-    0: {"dram_bytes": 24617216 + 1792, "fp64_winst": 5594741, "fp64_pipe_pct": 37.01},
+    1: {"dram_bytes": 35535616 + 2022912, "fp64_winst": 3459317, "fp64_pipe_pct": 43.19},
+    0: {"dram_bytes": 35166976 + 162816, "fp64_winst": 3458624, "fp64_pipe_pct": 41.71},
 }
 FUSED_CAPTURE_FRAME_MODE = 1                     # the autotuner's choice at N = 1M
 FUSED_DRAM_BYTES_CAPTURE = FUSED_CAPTURES[1]["dram_bytes"]
@@ -1116,8 +1116,8 @@ def chain_roofline(w, descs, c, iters, kt, prec, smem_peak, persistent, captured
     achieved = per * events_per_launch / (launch_ms * 1e-3) / 1e9
     cap = fused_capture(captured)
     traffic = (cap["dram_bytes"] * w.N / FUSED_CAPTURE_N) if cap else None
-    return {"kernel": "k_sweep_fused (persistent sweep kernel)" if persistent
-                      else "k_phase (chain kernel)",
+    return {"kernel": "k_sweep_axis, isotropic k_sweep_iso (persistent sweep kernel)" if persistent
+                      else "k_sweep_axis or k_phase (a launch per colour phase)",
             "bound": "smem", "achieved": achieved, "peak": smem_peak, "unit": "GB/s",
             "frac": achieved / smem_peak if smem_peak else None, "traffic": traffic,
             "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch "
