@@ -40,9 +40,9 @@
 //
 // What bounds it: a chain is a serial dependence and the kernel's time is that
 // of its instructions -- about 22,000 warp instructions per group of four cells
-// of 18 disks, half of them in the build, at 1.4 per cycle and SM (waits for
-// fixed latencies, shared memory and instruction fetch); HBM and the FP64 pipe
-// are below 35 %.  Measured on GB300, us per sweep, this kernel against the
+// of 18 disks, half of them in the build, at 1.5 per cycle and SM (waits for
+// fixed latencies, shared memory and instruction fetch); the FP64 pipe is 43 %
+// busy, HBM 1 %.  Measured on GB300, us per sweep, this kernel against the
 // one that searched strips of candidates at every event (ecmc_chain.cuh):
 //   N = 2^20, eta = 0.72,  240^2 cells, ell = 1.04, n_m = 2:   694 / 1140
 //   N = 2^22, eta = 0.716, 484^2 cells, ell = 1.05, n_m = 2:  2610 / 6135
