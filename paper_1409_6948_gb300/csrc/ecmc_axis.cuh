@@ -44,10 +44,10 @@
 // fixed latencies, shared memory and instruction fetch); the FP64 pipe is 43 %
 // busy, HBM 1 %.  Measured on GB300, us per sweep, this kernel against the
 // one that searched strips of candidates at every event (ecmc_chain.cuh):
-//   N = 2^20, eta = 0.72,  240^2 cells, ell = 1.04, n_m = 2:   694 / 1140
-//   N = 2^22, eta = 0.716, 484^2 cells, ell = 1.05, n_m = 2:  2610 / 6135
-//   N = 2^16, eta = 0.708, 32^2 cells,  ell = 8,    n_m = 1:   310 / 1217
-//   N = 256,  eta = 0.70,  2^2 cells,   ell = 4,    n_m = 2:   325 / 642
+//   N = 2^20, eta = 0.72,  240^2 cells, ell = 1.04, n_m = 2:   682 / 1140
+//   N = 2^22, eta = 0.716, 484^2 cells, ell = 1.05, n_m = 2:  2576 / 6135
+//   N = 2^16, eta = 0.708, 32^2 cells,  ell = 8,    n_m = 1:   309 / 1217
+//   N = 256,  eta = 0.70,  2^2 cells,   ell = 4,    n_m = 2:   324 / 642
 #pragma once
 #include <climits>
 
