@@ -29,9 +29,9 @@
 // the correctly rounded sqrt_rn), a replayed leg takes one FP64 addition, and
 // the neighbours' spheres pass an FP32 test of their positions within their
 // cells (rel) before their coordinates are fetched.  N = 64^3, eta = 0.45,
-// 32^3 cells, ell = 2, n_m = 1, GB300: 541 us a sweep, 758 with a search of
+// 32^3 cells, ell = 2, n_m = 1, GB300: 525 us a sweep, 758 with a search of
 // the bins at every event and FP64 tests of all 26 neighbours; frames alone
-// 297 / 403; 8^3 cells, n_m = 32: 12.3 / 18.7 ms; 16^3 spheres in 4^3 cells:
+// 279 / 403; 8^3 cells, n_m = 32: 12.3 / 18.7 ms; 16^3 spheres in 4^3 cells:
 // 1.16 / 1.75 ms.  Positions live in sphere-id order; a cell reads its frozen
 // neighbours' positions, which no warp writes while it runs (later colours
 // wait for it, earlier ones have finished).
@@ -132,6 +132,7 @@ __global__ void k3_begin(Geom3 g, State3* st, unsigned* sched) {
   sched[0] = 0u;
   sched[1] += 1u;
   sched[2] = 0u;
+  sched[3] = 0u;  // blocks of k3_end that have finished
   State3 s = *st;
   const U64x4 u = philox((uint64_t)s.t, ecmc::kPurposeSweep, 0, 0, g.seed, g.replica);
   for (int a = 0; a < 3; ++a) s.s[a] = unit_double(u.v[a]) * g.w;
@@ -922,16 +923,26 @@ __global__ void __launch_bounds__(32 * kWarpsMax, 5) k3_sweep(
   }
 }
 
-// End of sweep (one block of 256): the cells' sums in a fixed order, the
-// running totals, the sweep's member-weighted pressure sums, t + 1.
-__global__ void __launch_bounds__(256) k3_end(Geom3 g, State3* st, const Cell3* __restrict__ cs,
-                                             Totals3* tot, double* history, int64_t* hist_len) {
-  __shared__ double sd[2][8];
-  __shared__ long long sl[6][8];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+// End of sweep: the cells' sums in a fixed order (256 strided threads, trees
+// over their warps, the eight warps in turn), the running totals, the sweep's
+// member-weighted pressure sums, t + 1.  Each of the eight warps is a block of
+// its own, the last to finish adds them up: with 32^3 cells the FP64 pipe of
+// one SM set the pace, 541 us a sweep against
+// 525 now.
+struct Part3 {
+  double b, bw;
+  long long v[6];
+};
+constexpr int kEndWarps = 8;
+
+__global__ void __launch_bounds__(32) k3_end(Geom3 g, State3* st, const Cell3* __restrict__ cs,
+                                             unsigned* sched, Part3* part, Totals3* tot,
+                                             double* history, int64_t* hist_len) {
+  const int lane = threadIdx.x, tid = 32 * blockIdx.x + lane;
   double b = 0.0, bw = 0.0;
   long long v[6] = {0, 0, 0, 0, 0, 0};
-  for (int c = tid; c < g.ncell; c += 256) {
+#pragma unroll 8
+  for (int c = tid; c < g.ncell; c += 32 * kEndWarps) {
     const Cell3 s = cs[c];
     b += s.sum_b;
     bw += (double)s.n_mem * s.sum_b;
@@ -947,19 +958,22 @@ __global__ void __launch_bounds__(256) k3_end(Geom3 g, State3* st, const Cell3* 
     bw += __shfl_down_sync(0xffffffffu, bw, off);
     for (int q = 0; q < 6; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
   }
-  if (lane == 0) {
-    sd[0][wid] = b;
-    sd[1][wid] = bw;
-    for (int q = 0; q < 6; ++q) sl[q][wid] = v[q];
-  }
-  __syncthreads();
-  if (tid != 0) return;
+  if (lane != 0) return;
+  volatile Part3* mine = part + blockIdx.x;
+  mine->b = b;
+  mine->bw = bw;
+  for (int q = 0; q < 6; ++q) mine->v[q] = v[q];
+  __threadfence();
+  if (atomicAdd(&sched[3], 1u) != kEndWarps - 1) return;
+  __threadfence();
+  const volatile Part3* all = part;
   double B = 0.0, BW = 0.0;
   long long V[6] = {0, 0, 0, 0, 0, 0};
-  for (int wv = 0; wv < 8; ++wv) {
-    B += sd[0][wv];
-    BW += sd[1][wv];
-    for (int q = 0; q < 6; ++q) V[q] += sl[q][wv];
+#pragma unroll
+  for (int wv = 0; wv < kEndWarps; ++wv) {
+    B += all[wv].b;
+    BW += all[wv].bw;
+    for (int q = 0; q < 6; ++q) V[q] += all[wv].v[q];
   }
   const double dw = (double)g.N * (double)g.n_m * g.ell;
   Totals3& T = *tot;
@@ -1163,7 +1177,8 @@ struct ecmc3_ctx {
   cudaStream_t stream = nullptr, own = nullptr;
   double *px = nullptr, *py = nullptr, *pz = nullptr, *xyz_tmp = nullptr;
   int *cnt = nullptr, *ids = nullptr, *cell_of = nullptr, *err = nullptr, *recs = nullptr;
-  unsigned *sched = nullptr, *done = nullptr;  // persistent sweep: work counter, epoch, abort
+  // persistent sweep: work counter, epoch, abort; k3_end: blocks finished, their sums
+  unsigned *sched = nullptr, *done = nullptr;
   int persistent = 1, fused_blocks = 0;
   unsigned long long wait_ns = 5000000000ull;
   int wait_test = 0;
@@ -1255,7 +1270,9 @@ int enqueue_sweep(ecmc3_ctx* h, bool records) {
                                                     h->ids, rel3(h), h->cs,
                                                     records ? h->recs : nullptr, h->err);
   }
-  k3_end<<<1, 256, 0, h->stream>>>(g, h->st, h->cs, h->tot, h->history, h->hist_len);
+  k3_end<<<kEndWarps, 32, 0, h->stream>>>(g, h->st, h->cs, h->sched,
+                                          reinterpret_cast<Part3*>(h->sched + 4), h->tot,
+                                          h->history, h->hist_len);
   CK3(cudaGetLastError());
   return ECMC_OK;
 }
@@ -1515,7 +1532,7 @@ int ecmc3_create(ecmc3_t* out, int64_t N, double L, double sigma, int cells, dou
       cudaMalloc(&h->history, sizeof(double) * 2 * kHistoryCap) != cudaSuccess ||
       cudaMalloc(&h->hist_len, sizeof(int64_t)) != cudaSuccess ||
       cudaMalloc(&h->u64, sizeof(unsigned long long)) != cudaSuccess ||
-      cudaMalloc(&h->sched, sizeof(unsigned) * 4) != cudaSuccess ||
+      cudaMalloc(&h->sched, sizeof(unsigned) * 4 + sizeof(Part3) * kEndWarps) != cudaSuccess ||
       cudaMalloc(&h->done, sizeof(unsigned) * (size_t)g.ncell) != cudaSuccess) {
     cudaGetLastError();
     free3(h);

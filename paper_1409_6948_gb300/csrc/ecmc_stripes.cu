@@ -378,9 +378,9 @@ __global__ void __launch_bounds__(kThreads) ks_phase(
 // bound by the scan over all N stripe indices and the scattered fetches of
 // the members' coordinates, so both are done 32 at a time and the sort goes
 // through buckets of a few objects.  N = 2^16, 32 stripes, ell = 8, one chain
-// a stripe, GB300: 607 us a sweep; 1937 with the frame built by ordered
+// a stripe, GB300: 598 us a sweep; 1937 with the frame built by ordered
 // compaction of 512 ids at a time, a rank over whole strips (110 objects) and
-// FP64 comparisons.  With no chains' work (ell -> 0): 138 against 1401.
+// FP64 comparisons.  With no chains' work (ell -> 0): 130 against 1401.
 constexpr int kSortThreads = 512;
 constexpr int kLanesPerStrip = 6;
 
@@ -1028,23 +1028,50 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
     }
 }
 
-__global__ void ks_end(GeomS g, StateS* st, const StripeS* __restrict__ stats, TotalsS* tot,
-                       double* history, int64_t* hist_len) {
-  if (threadIdx.x != 0) return;
+// End of sweep (one warp): the stripes' sums in stripe order.  The lanes load 32
+// stripes at a time and form their terms; the four FP64 sums are taken in
+// order on a lane each (one thread: 607 us a sweep at 32 stripes, now
+// 598).
+__global__ void __launch_bounds__(32) ks_end(GeomS g, StateS* st,
+                                             const StripeS* __restrict__ stats, TotalsS* tot,
+                                             double* history, int64_t* hist_len) {
+  __shared__ double term[32][4];
+  const int lane = threadIdx.x;
+  const unsigned FULL = 0xffffffffu;
   TotalsS T = *tot;
-  double bw = 0.0, dw = 0.0;
-  for (int k = 0; k < g.S; ++k) {
-    const StripeS o = stats[k];
-    T.sum_b += o.sum_b;
-    T.sum_disp += (double)o.accepted * g.ell;
-    bw += (double)o.n_mem * o.sum_b;
-    dw += (double)o.n_mem * ((double)o.accepted * g.ell);
-    T.chains += o.chains;
-    T.events += o.events;
-    T.lifts += o.lifts;
-    T.frozen += o.frozen;
-    T.rejected += o.rejected;
+  double acc = lane == 0 ? T.sum_b : (lane == 1 ? T.sum_disp : 0.0);
+  long long v[5] = {0, 0, 0, 0, 0};
+  for (int k = 0; k < g.S; k += 32) {
+    if (k + lane < g.S) {
+      const StripeS o = stats[k + lane];
+      const double disp = (double)o.accepted * g.ell;
+      term[lane][0] = o.sum_b;
+      term[lane][1] = disp;
+      term[lane][2] = (double)o.n_mem * o.sum_b;
+      term[lane][3] = (double)o.n_mem * disp;
+      v[0] += o.chains;
+      v[1] += o.events;
+      v[2] += o.lifts;
+      v[3] += o.frozen;
+      v[4] += o.rejected;
+    }
+    __syncwarp();
+    if (lane < 4)
+      for (int i = 0; i < 32 && k + i < g.S; ++i) acc += term[i][lane];
+    __syncwarp();
   }
+#pragma unroll
+  for (int q = 0; q < 5; ++q)
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(FULL, v[q], o);
+  T.sum_b = __shfl_sync(FULL, acc, 0);
+  T.sum_disp = __shfl_sync(FULL, acc, 1);
+  const double bw = __shfl_sync(FULL, acc, 2), dw = __shfl_sync(FULL, acc, 3);
+  if (lane != 0) return;
+  T.chains += v[0];
+  T.events += v[1];
+  T.lifts += v[2];
+  T.frozen += v[3];
+  T.rejected += v[4];
   T.sum_b_w += bw;
   T.sum_disp_w += dw;
   T.sweeps++;
