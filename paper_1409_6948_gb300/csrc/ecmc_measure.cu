@@ -529,8 +529,9 @@ constexpr int kHexMaxCand = 64;
 // / 2 each within hx_e.  tlo and thi are bracketed by b / a -+ (hx_e (1 + |t|)) /
 // (|a| - hx_e) and the rounding of t.  A pair with |a| <= 8 hx_e cuts at |t| >
 // 1000 when |b| > 0.1 sigma^2, which closed cells never reach: it decides
-// nothing if b > 0 and removes l if b < 0.  All cell vertices within rc / 2
-// also mean that no disk beyond rc takes part.  Non-overlapping disks leave at
+// nothing if b > 0 and removes l if b < 0.  A closed cell with all its vertices
+// within rc / 2 also means that no disk beyond rc takes part; a disk without a
+// candidate has no cell and goes to k_hexatic.  Non-overlapping disks leave at
 // most 58 centres within 3.5 sigma, so the 64-disk limit needs no count.
 // One warp per 32 members of a cell: its lanes scan the same cells, so the
 // loads are broadcast.
@@ -646,7 +647,8 @@ __global__ void __launch_bounds__(64) k_hexatic_fixed(
   }
   if (!act) return;
   const int64_t id = g.n_off + pid[i];
-  if (!known) {
+  // (no edge: nobody within rc, but perhaps within rs)
+  if (!known || nb_mask == 0) {
     undecided[atomicAdd(n_undecided, 1ull)] = i;
     return;
   }
