@@ -114,12 +114,13 @@ struct ecmc_ctx {
   double* xy_tmp = nullptr;
   int* int_tmp = nullptr;
   unsigned long long* u64_tmp = nullptr;
+  unsigned long long* d_min2 = nullptr;  // [R] squared smallest distances
   UndoEntry* undo = nullptr;  // rejecting boundary rule: [C_total][cap] undo logs
   // pinned staging for the small copies of ecmc_set_positions, so that the
   // whole load (states up, binning, overlap check, result down) needs one
   // synchronisation
   SweepState* pin_states = nullptr;       // [R]
-  unsigned long long* pin_bits = nullptr;  // [2]: initial and resulting minimum
+  unsigned long long* pin_bits = nullptr;  // [2R]: initial and resulting minima
   // and for what a caller reads back between sweeps: copies into pageable
   // memory wait for the stream one by one (a replica's pressure took three
   // such waits, 30 us; one now)
@@ -563,29 +564,38 @@ int check_device_error(ecmc_ctx* h) {
   return ECMC_OK;
 }
 
-// smallest pair distance squared over all replicas (pairs closer than 2
-// sigma), enqueued: the result lands in pin_bits[1] once the stream has
+// smallest pair distance squared of every replica (pairs closer than 2
+// sigma), enqueued: the results land in pin_bits[R ..] once the stream has
 // passed it
 int enqueue_min_dist2(ecmc_ctx* h) {
+  const int R = h->b.R;
   double sig_max = 0.0;
   for (const Geom& g : h->geo) sig_max = g.sigma > sig_max ? g.sigma : sig_max;
   const double r2 = 4.0 * sig_max * sig_max;
-  std::memcpy(&h->pin_bits[0], &r2, sizeof(r2));
-  CK(cudaMemcpyAsync(h->u64_tmp, &h->pin_bits[0], sizeof(unsigned long long),
+  for (int r = 0; r < R; ++r) std::memcpy(&h->pin_bits[r], &r2, sizeof(r2));
+  CK(cudaMemcpyAsync(h->d_min2, h->pin_bits, sizeof(unsigned long long) * R,
                      cudaMemcpyHostToDevice, h->stream));
-  launch_min_dist(h->geo.data(), h->b, h->u64_tmp, h->stream);
+  launch_min_dist(h->geo.data(), h->b, h->d_min2, h->stream);
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(&h->pin_bits[1], h->u64_tmp, sizeof(unsigned long long),
+  CK(cudaMemcpyAsync(h->pin_bits + R, h->d_min2, sizeof(unsigned long long) * R,
                      cudaMemcpyDeviceToHost, h->stream));
   return ECMC_OK;
 }
 
+double min_dist2_of(const ecmc_ctx* h, int r) {
+  double d2 = 0.0;
+  std::memcpy(&d2, &h->pin_bits[h->b.R + r], sizeof(d2));
+  return d2;
+}
+
+// over all replicas
 int min_dist2(ecmc_ctx* h, double* d2) {
   int rc = enqueue_min_dist2(h);
   if (rc) return rc;
   rc = check_device_error(h);
   if (rc) return rc;
-  std::memcpy(d2, &h->pin_bits[1], sizeof(*d2));
+  *d2 = min_dist2_of(h, 0);
+  for (int r = 1; r < h->b.R; ++r) *d2 = std::fmin(*d2, min_dist2_of(h, r));
   return ECMC_OK;
 }
 
@@ -605,20 +615,19 @@ int load_positions_dev(ecmc_ctx* h, const double* xy_dev, int64_t t0) {
   h->t_host = t0;
   h->valid_state = true;
   // the overlap check follows in the same stream; one synchronisation reports
-  // a binning error and delivers the smallest distance
+  // a binning error and delivers the smallest distances
   int rc = enqueue_min_dist2(h);
   if (rc) return rc;
   rc = check_device_error(h);
   if (rc) return rc;
-  double d2 = 0.0;
-  std::memcpy(&d2, &h->pin_bits[1], sizeof(d2));
-  // no two disks may overlap beyond rounding
-  double sig2_min = 1e300;
-  for (const Geom& g : h->geo) sig2_min = g.sig2 < sig2_min ? g.sig2 : sig2_min;
-  if (d2 < sig2_min * (1.0 - 1e-9)) {
-    h->valid_state = false;
-    return fail(ECMC_ERR_OVERLAP, "positions overlap: smallest distance %.17g < sigma",
-                std::sqrt(d2));
+  // no two disks of a replica may overlap beyond rounding
+  for (int r = 0; r < h->b.R; ++r) {
+    const double d2 = min_dist2_of(h, r);
+    if (d2 < h->geo[r].sig2 * (1.0 - 1e-9)) {
+      h->valid_state = false;
+      return fail(ECMC_ERR_OVERLAP, "positions overlap: smallest distance %.17g < sigma = %.17g"
+                  " (replica %d)", std::sqrt(d2), h->geo[r].sigma, r);
+    }
   }
   return ECMC_OK;
 }
@@ -680,6 +689,7 @@ void free_all(ecmc_ctx* h) {
   cudaFree(h->xy_tmp);
   cudaFree(h->int_tmp);
   cudaFree(h->u64_tmp);
+  cudaFree(h->d_min2);
   cudaFree(h->undo);
   cudaFreeHost(h->pin_states);
   cudaFreeHost(h->pin_bits);
@@ -863,8 +873,9 @@ int create_impl(ecmc_t* out, const ecmc_replica_desc_t* desc, int R) {
       cudaMalloc(&h->xy_tmp, sizeof(double) * 2 * (size_t)N_total) != cudaSuccess ||
       cudaMalloc(&h->int_tmp, sizeof(int) * (size_t)N_total) != cudaSuccess ||
       cudaMalloc(&h->u64_tmp, sizeof(unsigned long long) * 4) != cudaSuccess ||
+      cudaMalloc(&h->d_min2, sizeof(unsigned long long) * R) != cudaSuccess ||
       cudaMallocHost(&h->pin_states, sizeof(SweepState) * R) != cudaSuccess ||
-      cudaMallocHost(&h->pin_bits, sizeof(unsigned long long) * 2) != cudaSuccess ||
+      cudaMallocHost(&h->pin_bits, sizeof(unsigned long long) * 2 * R) != cudaSuccess ||
       cudaMallocHost(&h->pin_read, sizeof(PinRead)) != cudaSuccess)
     return bail(fail(ECMC_ERR_OOM, "device allocation failed"));
   cudaMemsetAsync(b.totals, 0, sizeof(RunTotals) * R, h->stream);

@@ -314,9 +314,12 @@ __global__ void __launch_bounds__(256) k_min_dist_fixed(
     const int* __restrict__ cnt, unsigned long long* __restrict__ out) {
   const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (c >= C_total) return;  // warp-uniform
-  const Geom& g = rg[cell_rep[c]];
-  if (g.md_path == 1) min_dist_cell<true>(g, c - g.cell_off, cap, px, py, fxy, cnt, out);
-  else if (g.md_path == 2) min_dist_cell<false>(g, c - g.cell_off, cap, px, py, fxy, cnt, out);
+  const int rep = cell_rep[c];
+  const Geom& g = rg[rep];
+  if (g.md_path == 1)
+    min_dist_cell<true>(g, c - g.cell_off, cap, px, py, fxy, cnt, out + rep);
+  else if (g.md_path == 2)
+    min_dist_cell<false>(g, c - g.cell_off, cap, px, py, fxy, cnt, out + rep);
 }
 
 // ---- pair-correlation histogram on fixed-point positions ------------------
@@ -432,7 +435,9 @@ void set_min_dist(Geom& g) {
   g.md_path = !(rcut < 0.25 * g.L) ? 0 : (half ? 1 : 2);
 }
 
-// geo: the R replicas' geometry on the host.
+// geo: the R replicas' geometry on the host.  out[R]: squared minima, lowered
+// to those of the replicas' pairs (each replica is checked against its own
+// diameter).
 void launch_min_dist(const Geom* geo, const DevBufs& b, unsigned long long* out, cudaStream_t s) {
   bool fixed = false;
   for (int r = 0; r < b.R; ++r) {
@@ -444,7 +449,7 @@ void launch_min_dist(const Geom* geo, const DevBufs& b, unsigned long long* out,
     const int bs = 128;
     const int64_t total = (int64_t)g.ncell * b.cap;
     k_pairs<false><<<(unsigned)((total + bs - 1) / bs), bs, 0, s>>>(
-        g, b.cap, b.px[b.cur], b.py[b.cur], b.count[b.cur], 2.0 * g.sigma, 0.0, 0, out);
+        g, b.cap, b.px[b.cur], b.py[b.cur], b.count[b.cur], 2.0 * g.sigma, 0.0, 0, out + r);
   }
   if (!fixed) return;
   const uint2* fxy = launch_fixed_point(b, s);
