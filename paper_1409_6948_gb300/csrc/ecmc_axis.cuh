@@ -403,7 +403,10 @@ __device__ __noinline__ void axis_shuffled_list(int* pl, int n, int first, int64
 // FP64 addition forms the mover's end, the budget left and the contact sum on
 // three lanes.  An FP64 instruction of a warp takes its scheduler's unit for
 // 57 cycles, whatever the number of lanes.  The lanes of one group hold the
-// same chain state, but the contact sum is kept on lane 2 of each quad.
+// same chain state, but the contact sum is kept on lane 2 of each quad, and
+// what a group keeps in memory (coordinates, latest legs, history, undo log)
+// is written by its first lane.  Votes and shuffles order no memory: a
+// __syncwarp stands wherever other lanes read or write the same words.
 template <int TPC, bool REJECT>
 __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, int64_t t,
                                             int lc, int c, bool run, bool irregular,
@@ -447,46 +450,49 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
   int t_em = -1, t_tot = 0, t_walls = 0, t_frozen = 0, n_turn = 0;
   double t_P = 0.0;
   float t_r = 0.0f;
-  int gap = 0;  // legs since the mover's previous one
+  int gap = 0;  // legs since the mover's previous one (first lane)
 
   // Everything that needs the lanes of a group to work together is done by
   // the whole warp, for all the groups it concerns: collectives on part of a
   // warp would make its groups run one after the other.
   bool need = nmem > 0, starting = true;  // a group wants its next chain; any does
+  const bool any_irregular = __any_sync(FULL, irregular);
 #pragma unroll 1
   for (;;) {
     if (starting) {
+      __syncwarp();
       const bool go = need && k < n_m;
       const bool refill = go && (k & (kStarts - 1)) == 0;
       if (__any_sync(FULL, refill)) {
         if (refill)
           axis_draws<TPC>(f.starts, k, n_m, nmem, g.dir_mode, t, lc, g.seed, g.replica, sub);
         __syncwarp();
+        // the list takes the room of the leg history
+        if (refill && shuffled && k == 0 && sub == 0)
+          axis_shuffled_list((int*)f.leg, nmem, f.starts[0], t, lc, g.seed, g.replica);
+        __syncwarp();
       }
       if (need) active = go;
       need = false;
       if (go) {
         int idx = f.starts[k & (kStarts - 1)];
-        if (shuffled) {
-          // every lane of the group writes the same list into the leg history
-          int* pl = (int*)f.leg;
-          if (k == 0) axis_shuffled_list(pl, nmem, idx, t, lc, g.seed, g.replica);
-          idx = pl[k % nmem];
-        }
+        if (shuffled) idx = ((const int*)f.leg)[k % nmem];
         const int m = f.rank[idx];
         em = m * 2 + f.starts[kStarts + (k & (kStarts - 1))];
         P = f.a[m];
         r = ell;
         if (REJECT) {
-          UndoEntry& u = g.undo[(int64_t)c * g.undo_stride];
-          u.a = P;
-          u.m = m;
-          u.touched = f.last[m];
+          if (sub == 0) {
+            UndoEntry& u = g.undo[(int64_t)c * g.undo_stride];
+            u.a = P;
+            u.m = m;
+            u.touched = f.last[m];
+          }
           n_undo = 1;
           ch_b = 0.0;
         }
         gap = kLegGapMax;
-        f.last[m] = n_tot + 1;
+        if (sub == 0) f.last[m] = n_tot + 1;
         start_key = f.key[m];
         tot0 = n_tot;
         wall0 = n_walls;
@@ -514,9 +520,10 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
       // still on their way when this one's loads were issued (its candidates
       // lie ahead, so the stopped disk is not among them)
       const double rz = __shfl_sync(FULL, z, quad0 + 1);
+      if (any_irregular) __syncwarp();  // (there it may be: the search decides)
       if (moved >= 0) {
         r = rz;
-        if (q4 == 0) f.a[moved] = z;
+        if (sub == 0) f.a[moved] = z;
         moved = -1;
       }
       const bool neg = dbits(d) < 0;
@@ -564,6 +571,7 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
         }
       }
     }
+    if (any_irregular) __syncwarp();
     if (irregular && active) {
       const AxisStop st = axis_search<TPC>(f.a, f.b, f.key, f.nobj, em >> 1, P, dir, sig2, sub,
                                            gmask);
@@ -603,8 +611,8 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
       }
     }
     const int m = em >> 1;
-    if (active && keep_legs && !is_end) {
-      // every lane of the group writes the same values
+    if (TPC == 2) __syncwarp();  // both lanes have read the mover's coordinate
+    if (active && keep_legs && !is_end && sub == 0) {
       AxisLeg q;
       q.P = P;
       q.S = step;
@@ -622,29 +630,33 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
       if (QUAD) {
         moved = m;
       } else {
-        f.a[m] = Pnew;
+        if (sub == 0) f.a[m] = Pnew;
         r = rnew;
       }
       em = bj * 2 + dir;
       P = aw;
-      if (REJECT) {
-        if (n_undo < g.cap_mem) {
-          UndoEntry& u = g.undo[(int64_t)c * g.undo_stride + n_undo];
-          u.a = P;
-          u.m = bj;
-          u.touched = f.last[bj];
-        } else {
-          atomicCAS(err, DEV_OK, DEV_CAPACITY);
+      if (sub == 0) {
+        const int latest = f.last[bj];
+        if (REJECT) {
+          if (n_undo < g.cap_mem) {
+            UndoEntry& u = g.undo[(int64_t)c * g.undo_stride + n_undo];
+            u.a = P;
+            u.m = bj;
+            u.touched = latest;
+          } else {
+            atomicCAS(err, DEV_OK, DEV_CAPACITY);
+          }
         }
-        ++n_undo;
+        const int back = n_tot + 1 - latest;  // n_tot + 1 if it never moved
+        gap = back < kLegGapMax ? back : kLegGapMax;
+        f.last[bj] = n_tot + 1;
       }
-      const int back = n_tot + 1 - f.last[bj];  // n_tot + 1 if it never moved
-      gap = back < kLegGapMax ? back : kLegGapMax;
-      f.last[bj] = n_tot + 1;
+      if (REJECT) ++n_undo;
     }
     if (!__any_sync(FULL, slow)) continue;
 
     // turn-backs and chain ends
+    __syncwarp();
     if (QUAD) {
       Pnew = __shfl_sync(FULL, z, quad0);
       rnew = __shfl_sync(FULL, z, quad0 + 1);
@@ -655,7 +667,7 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
       P = is_wall && !is_end ? aw : Pnew;
       need = is_end;
       if (is_end) {
-        f.a[m] = P;
+        if (sub == 0) f.a[m] = P;
         if (REJECT) sum_b += ch_b;
       } else {
         ++n_tot;
@@ -678,7 +690,7 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
           em ^= 1;
           turned = keep_legs;
           gap = 1;
-          f.last[m] = n_tot + 1;
+          if (sub == 0) f.last[m] = n_tot + 1;
         }
       }
     }
@@ -700,6 +712,7 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
         const bool same = !cyc || axis_cycle_holds<TPC>(f, sub, n_tot, K, em >> 1);
         const unsigned differ = __ballot_sync(FULL, !same);
         cyc = cyc && ((differ >> gshift) & GM) == 0;
+        __syncwarp();  // the comparison has read what the replay writes
         if (cyc) {
           axis_replay<TPC>(f, gmask, gshift, sub, K, len, cw, cf, tot0, n_tot, em, P, r, sum_b,
                            n_frozen, n_walls, n_replayed);
@@ -722,7 +735,7 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
     }
     if (slow && n_tot - tot0 >= (int)kMaxEventsPerChain) {
       atomicCAS(err, DEV_OK, DEV_CHAIN_CAP);
-      if (!need) f.a[em >> 1] = P;
+      if (!need && sub == 0) f.a[em >> 1] = P;
       need = true;
     }
     if (need && recs != nullptr && sub == 0) {

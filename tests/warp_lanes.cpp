@@ -1,0 +1,123 @@
+// The lanes of warp_lanes.h.  Compiled without ThreadSanitizer, so that the
+// scheduler's own data do not count; it only reports the fibers and the memory
+// order of __syncwarp.
+#include <cstdint>
+#include <cstdio>
+#include <cstdlib>
+#include <functional>
+
+#include <ucontext.h>
+
+extern "C" {
+void* __tsan_get_current_fiber(void);
+void* __tsan_create_fiber(unsigned flags);
+void __tsan_switch_to_fiber(void* fiber, unsigned flags);
+void __tsan_acquire(void* at);
+void __tsan_release(void* at);
+}
+
+namespace warp {
+struct Index {
+  int x;
+};
+namespace {
+constexpr unsigned kNoSync = 1;  // a switch of fibers orders nothing
+constexpr size_t kStack = 1 << 19;
+struct Lane {
+  ucontext_t ctx;
+  void* fiber;
+  char* stack;
+  bool done, waiting;
+  unsigned mask;
+  int line;
+  uint64_t val;
+  volatile uint64_t out[32];
+};
+Lane lanes[32];
+ucontext_t home;
+void* home_fiber;
+int current;
+const std::function<void(int)>* body;
+char token[32][33];  // one per mask of a lane group: first lane, number of lanes
+
+void enter(int l) {
+  (*body)(l);
+  lanes[l].done = true;
+  __tsan_switch_to_fiber(home_fiber, 0);
+  swapcontext(&lanes[l].ctx, &home);
+}
+}  // namespace
+
+Index thread_idx() { return Index{current}; }
+
+void meet(unsigned mask, uint64_t val, uint64_t out[32], int line, bool orders_memory) {
+  Lane& me = lanes[current];
+  const int l = current;
+  if (!(mask >> l & 1)) {
+    std::printf("lane %d is not in its mask %x, line %d\n", l, mask, line);
+    std::exit(2);
+  }
+  char* const t = &token[__builtin_ctz(mask)][__builtin_popcount(mask)];
+  if (orders_memory) __tsan_release(t);
+  me.mask = mask;
+  me.val = val;
+  me.line = line;
+  me.waiting = true;
+  __tsan_switch_to_fiber(home_fiber, kNoSync);
+  swapcontext(&me.ctx, &home);
+  if (orders_memory) __tsan_acquire(t);
+  for (int i = 0; i < 32; ++i) out[i] = me.out[i];
+}
+
+bool run(const std::function<void(int)>& f, bool downwards) {
+  body = &f;
+  home_fiber = __tsan_get_current_fiber();
+  for (int l = 0; l < 32; ++l) {
+    Lane& me = lanes[l];
+    me.done = me.waiting = false;
+    if (!me.stack) me.stack = (char*)std::malloc(kStack);
+    me.fiber = __tsan_create_fiber(0);
+    getcontext(&me.ctx);
+    me.ctx.uc_stack.ss_sp = me.stack;
+    me.ctx.uc_stack.ss_size = kStack;
+    me.ctx.uc_link = &home;
+    makecontext(&me.ctx, (void (*)())enter, 1, l);
+  }
+  for (;;) {
+    bool ran = false, all = true;
+    for (int i = 0; i < 32; ++i) {
+      const int l = downwards ? 31 - i : i;
+      if (lanes[l].done) continue;
+      all = false;
+      if (lanes[l].waiting) continue;
+      ran = true;
+      current = l;
+      __tsan_switch_to_fiber(lanes[l].fiber, kNoSync);
+      swapcontext(&home, &lanes[l].ctx);
+    }
+    if (all) return true;
+    for (int l = 0; l < 32; ++l) {
+      if (lanes[l].done || !lanes[l].waiting) continue;
+      const unsigned m = lanes[l].mask;
+      bool ready = true;
+      for (int i = 0; i < 32; ++i)
+        if (m >> i & 1)
+          ready = ready && !lanes[i].done && lanes[i].waiting && lanes[i].mask == m &&
+                  lanes[i].line == lanes[l].line;
+      if (!ready) continue;
+      ran = true;
+      for (int i = 0; i < 32; ++i)
+        if (m >> i & 1) {
+          for (int q = 0; q < 32; ++q) lanes[i].out[q] = m >> q & 1 ? lanes[q].val : 0;
+          lanes[i].waiting = false;
+        }
+    }
+    if (!ran) {
+      for (int l = 0; l < 32; ++l)
+        std::printf("lane %d done %d waits at line %d, mask %x\n", l, lanes[l].done,
+                    lanes[l].line, lanes[l].mask);
+      return false;
+    }
+  }
+}
+}  // namespace warp
