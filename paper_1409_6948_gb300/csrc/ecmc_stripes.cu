@@ -933,6 +933,9 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
           done = 3;
           break;
         }
+        // (votes and shuffles order no memory: the search has read what lane 0
+        // writes from here on)
+        __syncwarp();
         if (ecmc::le_nn(r, bs)) {  // budget used up: the chain ends
           const double x = Um + ecmc::flip_if(r, dsg < 0);
           if (lane == 0) {
@@ -984,6 +987,7 @@ __global__ void __launch_bounds__(kSortThreads) ks_phase_sorted(
           d = -d;
         }
       }
+      __syncwarp();  // lane 0 has written where the last disk stopped
       if (done == 2) {
         for (int q0 = lane; q0 < n_mem; q0 += 32 * kUnroll) {
           double u0[kUnroll];

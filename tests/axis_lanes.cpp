@@ -133,7 +133,7 @@ int main(int argc, char** argv) {
                    1099511628211ull;
     }
   };
-  const bool fine = warp::run(lane_main, std::atoi(argv[9]) != 0);
+  const bool fine = warp::run(lane_main, 32, std::atoi(argv[9]) != 0);
   for (int gi = 0; gi < CPW && gi < n_active; ++gi) {
     const CellStats& s = cs[2 * (gi % (cells / 2)) + 2 * (gi / (cells / 2)) * cells];
     std::printf("cell %d irregular %llu: chains %d events %d lifts %d frozen %d walls %d replayed %d "

@@ -6,19 +6,11 @@ one lane writes and another reads or writes without a __syncwarp between them
 is reported as a data race.  Results must not depend on the order in which the
 lanes run, nor on the number of lanes per cell.
 """
-import os
 import re
-import shutil
-import subprocess
 
 import pytest
 
-HERE = os.path.dirname(os.path.abspath(__file__))
-ROOT = os.path.dirname(HERE)
-CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
-
-if shutil.which("g++") is None or not os.path.exists(os.path.join(CUDA, "include/cuda_runtime.h")):
-    pytest.skip("needs g++ and the CUDA headers", allow_module_level=True)
+import lanes
 
 LANES = (2, 4, 8, 32)
 # k, eta, cells per side, ell, n_m, boundary, list mode, start
@@ -36,43 +28,15 @@ CASES = {
 
 @pytest.fixture(scope="module")
 def programs(tmp_path_factory):
-    d = tmp_path_factory.mktemp("lanes")
-    probe = d / "probe"
-    (d / "probe.cpp").write_text("int main() { return 0; }\n")
-    if subprocess.run(["g++", "-fsanitize=thread", str(d / "probe.cpp"), "-o", str(probe)],
-                      capture_output=True).returncode or \
-            subprocess.run([str(probe)], capture_output=True).returncode:
-        pytest.skip("ThreadSanitizer does not run here")
-    flags = ["-std=c++20", "-O1", "-g", "-Wno-unknown-pragmas"]
-    lanes_o = str(d / "warp_lanes.o")
-    subprocess.run(["g++", *flags, "-fno-tree-loop-distribute-patterns", "-c",
-                    os.path.join(HERE, "warp_lanes.cpp"), "-o", lanes_o], check=True)
-    jobs, out = [], {}
-    for n in LANES:
-        out[n] = str(d / ("axis_lanes%d" % n))
-        jobs.append(subprocess.Popen(
-            ["g++", *flags, "-fsanitize=thread", "-DLANES=%d" % n,
-             "-I", os.path.join(CUDA, "include"), "-I", os.path.join(ROOT, "include"),
-             "-I", os.path.join(ROOT, "paper_1409_6948_gb300", "csrc"),
-             os.path.join(HERE, "axis_lanes.cpp"), lanes_o, "-o", out[n]]))
-    assert [j.wait() for j in jobs] == [0] * len(jobs)
-    return out
-
-
-def run(program, case, downwards):
-    r = subprocess.run([program, *CASES[case].split(), str(downwards)], capture_output=True,
-                       text=True, timeout=300, env={**os.environ, "TSAN_OPTIONS": "atexit_sleep_ms=0"})
-    races = r.stderr.count("WARNING: ThreadSanitizer")
-    assert races == 0, "%d data races\n%s" % (races, r.stderr[:4000])
-    assert r.returncode == 0, r.stdout + r.stderr[:4000]
-    return r.stdout.splitlines()
+    return lanes.build(tmp_path_factory.mktemp("lanes"), "axis_lanes.cpp",
+                       {n: ["-DLANES=%d" % n] for n in LANES})
 
 
 @pytest.mark.parametrize("case", sorted(CASES))
 def test_lanes_order_their_memory(programs, case):
     first = None
     for n in LANES:
-        up, down = run(programs[n], case, 0), run(programs[n], case, 1)
+        up, down = (lanes.run(programs[n], CASES[case] + d) for d in (" 0", " 1"))
         assert up == down
         assert len(up) == min(16, 32 // n)
         # how much of a chain is replayed depends on the lanes, what it does not

@@ -22,7 +22,8 @@ struct Index {
 };
 namespace {
 constexpr unsigned kNoSync = 1;  // a switch of fibers orders nothing
-constexpr size_t kStack = 1 << 19;
+constexpr size_t kStack = 1 << 18;
+constexpr int kMost = 1024;
 struct Lane {
   ucontext_t ctx;
   void* fiber;
@@ -33,12 +34,13 @@ struct Lane {
   uint64_t val;
   volatile uint64_t out[32];
 };
-Lane lanes[32];
+Lane lanes[kMost];
 ucontext_t home;
 void* home_fiber;
 int current;
 const std::function<void(int)>* body;
-char token[32][33];  // one per mask of a lane group: first lane, number of lanes
+// one per mask of a lane group: first lane, number of lanes
+char token[kMost / 32][32][33], block_token;
 
 void enter(int l) {
   (*body)(l);
@@ -52,12 +54,12 @@ Index thread_idx() { return Index{current}; }
 
 void meet(unsigned mask, uint64_t val, uint64_t out[32], int line, bool orders_memory) {
   Lane& me = lanes[current];
-  const int l = current;
+  const int l = current & 31;
   if (!(mask >> l & 1)) {
     std::printf("lane %d is not in its mask %x, line %d\n", l, mask, line);
     std::exit(2);
   }
-  char* const t = &token[__builtin_ctz(mask)][__builtin_popcount(mask)];
+  char* const t = &token[current >> 5][__builtin_ctz(mask)][__builtin_popcount(mask)];
   if (orders_memory) __tsan_release(t);
   me.mask = mask;
   me.val = val;
@@ -69,10 +71,22 @@ void meet(unsigned mask, uint64_t val, uint64_t out[32], int line, bool orders_m
   for (int i = 0; i < 32; ++i) out[i] = me.out[i];
 }
 
-bool run(const std::function<void(int)>& f, bool downwards) {
+// mask 0: the whole block
+void block_barrier(int line) {
+  Lane& me = lanes[current];
+  __tsan_release(&block_token);
+  me.mask = 0;
+  me.line = line;
+  me.waiting = true;
+  __tsan_switch_to_fiber(home_fiber, kNoSync);
+  swapcontext(&me.ctx, &home);
+  __tsan_acquire(&block_token);
+}
+
+bool run(const std::function<void(int)>& f, int n, bool downwards) {
   body = &f;
   home_fiber = __tsan_get_current_fiber();
-  for (int l = 0; l < 32; ++l) {
+  for (int l = 0; l < n; ++l) {
     Lane& me = lanes[l];
     me.done = me.waiting = false;
     if (!me.stack) me.stack = (char*)std::malloc(kStack);
@@ -84,37 +98,45 @@ bool run(const std::function<void(int)>& f, bool downwards) {
     makecontext(&me.ctx, (void (*)())enter, 1, l);
   }
   for (;;) {
-    bool ran = false, all = true;
-    for (int i = 0; i < 32; ++i) {
-      const int l = downwards ? 31 - i : i;
+    bool ran = false, all = true, block = true;
+    for (int i = 0; i < n; ++i) {
+      const int l = downwards ? n - 1 - i : i;
       if (lanes[l].done) continue;
       all = false;
-      if (lanes[l].waiting) continue;
-      ran = true;
-      current = l;
-      __tsan_switch_to_fiber(lanes[l].fiber, kNoSync);
-      swapcontext(&home, &lanes[l].ctx);
+      if (!lanes[l].waiting) {
+        ran = true;
+        current = l;
+        __tsan_switch_to_fiber(lanes[l].fiber, kNoSync);
+        swapcontext(&home, &lanes[l].ctx);
+      }
     }
     if (all) return true;
-    for (int l = 0; l < 32; ++l) {
+    for (int l = 0; l < n; ++l) {
       if (lanes[l].done || !lanes[l].waiting) continue;
       const unsigned m = lanes[l].mask;
+      if (m == 0) continue;
+      Lane* const w = &lanes[l & ~31];
       bool ready = true;
       for (int i = 0; i < 32; ++i)
         if (m >> i & 1)
-          ready = ready && !lanes[i].done && lanes[i].waiting && lanes[i].mask == m &&
-                  lanes[i].line == lanes[l].line;
+          ready = ready && !w[i].done && w[i].waiting && w[i].mask == m && w[i].line == lanes[l].line;
       if (!ready) continue;
       ran = true;
       for (int i = 0; i < 32; ++i)
         if (m >> i & 1) {
-          for (int q = 0; q < 32; ++q) lanes[i].out[q] = m >> q & 1 ? lanes[q].val : 0;
-          lanes[i].waiting = false;
+          for (int q = 0; q < 32; ++q) w[i].out[q] = m >> q & 1 ? w[q].val : 0;
+          w[i].waiting = false;
         }
     }
+    for (int l = 0; l < n; ++l)
+      block = block && !lanes[l].done && lanes[l].waiting && lanes[l].mask == 0;
+    if (block) {
+      ran = true;
+      for (int l = 0; l < n; ++l) lanes[l].waiting = false;
+    }
     if (!ran) {
-      for (int l = 0; l < 32; ++l)
-        std::printf("lane %d done %d waits at line %d, mask %x\n", l, lanes[l].done,
+      for (int l = 0; l < n; ++l)
+        std::printf("thread %d done %d waits at line %d, mask %x\n", l, lanes[l].done,
                     lanes[l].line, lanes[l].mask);
       return false;
     }
