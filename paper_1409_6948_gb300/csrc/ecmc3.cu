@@ -591,6 +591,7 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
               break;
             }
             // no room: drop the lists and start this one over
+            __syncwarp();  // (every lane has read lst[m]; votes order no memory)
             for (int q = lane; q < nmem; q += 32) lst[q] = -1;
             n_list = 0;
             nl = 0;
@@ -733,6 +734,7 @@ __device__ __forceinline__ void cell3(const Geom3& g, const State3& st, int colo
         }
         const unsigned pb = __ballot_sync(FULL, per);
         if (pb != 0u) {
+          __syncwarp();  // the search for K has read what lane 0 writes below
           const int K = 2 * __ffs(pb), b0 = n_leg - K;
           // whole legs while the budget exceeds them (a wall's contact term
           // is +0: it leaves the sum as it is)
