@@ -335,7 +335,8 @@ ECMC_API int ecmc_autotune(ecmc_t h, int trial_sweeps, ecmc_tune_result_t* best,
 ECMC_API int ecmc_destroy(ecmc_t h);
 
 /* Set / query one ECMC_PARAM_* value.  ECMC_ERR_ARG for an unknown key or a
- * value out of range. */
+ * value out of range.  A launch shape that is refused (ECMC_ERR_UNSUPPORTED)
+ * or finds no memory leaves the handle with the shape and values it had. */
 ECMC_API int ecmc_set_param(ecmc_t h, int key, double value);
 ECMC_API int ecmc_get_param(ecmc_t h, int key, double* value);
 

@@ -74,6 +74,7 @@ struct ecmc_ctx {
   int persistent = 0;    // in use
   int fused_blocks = 0;  // grid of the persistent sweep kernel
   int axis = 0;          // axis chains through their static candidates (ecmc_axis.cuh)
+  bool layout_ok = false;  // the launch shape and its buffers are complete
   AxisShape axis_shape;
   double wait_ms = 5000.0;
   int n_sm = 0;
@@ -334,7 +335,14 @@ int axis_layout(ecmc_ctx* h, int* used) {
   return ECMC_OK;
 }
 
+int finish_layout(ecmc_ctx* h) {
+  const int rc = upload_geometry(h);
+  h->layout_ok = rc == ECMC_OK;
+  return rc;
+}
+
 int compute_layout(ecmc_ctx* h) {
+  h->layout_ok = false;
   for (Geom& g : h->geo) set_strip_bins(g, h->strip_w);
   const size_t limit = kSmemLimit;
   if (h->n_sm == 0) {
@@ -348,7 +356,7 @@ int compute_layout(ecmc_ctx* h) {
   int used = 0;
   const int rc_axis = axis_layout(h, &used);
   if (rc_axis) return rc_axis;
-  if (used) return upload_geometry(h);
+  if (used) return finish_layout(h);
   int fmode = auto_fmode(h);
   h->tpc = choose_tpc(h, fmode);
   // isotropic chains in the persistent kernel: the fewest lanes per cell that
@@ -415,7 +423,7 @@ int compute_layout(ecmc_ctx* h) {
       cudaGetLastError();
     }
   }
-  return upload_geometry(h);
+  return finish_layout(h);
 }
 
 void drop_graphs(ecmc_ctx* h) {
@@ -424,6 +432,43 @@ void drop_graphs(ecmc_ctx* h) {
       cudaGraphExecDestroy(h->graph[i]);
       h->graph[i] = nullptr;
     }
+}
+
+// The parameters that the launch shape follows from.
+struct LayoutParams {
+  int tpc, warps, fmode, persist, dir_mode, iso, boundary, reject;
+  float strip_w;
+};
+
+LayoutParams layout_params(const ecmc_ctx* h) {
+  return {h->tpc_param, h->warps_param,      h->fmode_param,     h->persist_param,
+          h->geo[0].dir_mode, h->b.iso, h->geo[0].boundary, h->b.reject, h->strip_w};
+}
+
+// One of them has changed: the new launch shape.  Where that is refused or
+// finds no memory, the handle keeps the shape it had, as the buffers of one
+// shape do not fit the kernels of another.
+int relayout(ecmc_ctx* h, const LayoutParams& old) {
+  drop_graphs(h);
+  const int rc = compute_layout(h);
+  if (rc == ECMC_OK) return rc;
+  cudaGetLastError();
+  char msg[sizeof(g_msg)];
+  std::memcpy(msg, g_msg, sizeof(msg));
+  h->tpc_param = old.tpc;
+  h->warps_param = old.warps;
+  h->fmode_param = old.fmode;
+  h->persist_param = old.persist;
+  h->strip_w = old.strip_w;
+  h->b.iso = old.iso;
+  h->b.reject = old.reject;
+  for (Geom& g : h->geo) {
+    g.dir_mode = old.dir_mode;
+    g.boundary = old.boundary;
+  }
+  compute_layout(h);  // (ecmc_sweep refuses to run should this fail, too)
+  std::memcpy(g_msg, msg, sizeof(msg));
+  return rc;
 }
 
 cudaEvent_t get_event(ecmc_ctx* h) {
@@ -1075,6 +1120,7 @@ int ecmc_set_stream(ecmc_t h, void* stream) {
 int ecmc_set_param(ecmc_t h, int key, double v) {
   if (!h) return fail(ECMC_ERR_ARG, "NULL handle");
   CK(cudaStreamSynchronize(h->stream));
+  const LayoutParams old = layout_params(h);
   switch (key) {
     case ECMC_PARAM_N_CHAINS: {
       if (!(v >= 1.0 && v <= 1e6) || v != std::floor(v)) return fail(ECMC_ERR_ARG, "n_m");
@@ -1090,8 +1136,7 @@ int ecmc_set_param(ecmc_t h, int key, double v) {
         return fail(ECMC_ERR_UNSUPPORTED, "the rejecting boundary rule needs axis chains");
       for (Geom& g : h->geo) g.dir_mode = (int)v;
       h->b.iso = v == 2.0 ? 1 : 0;
-      drop_graphs(h);
-      return compute_layout(h);
+      return relayout(h, old);
     }
     case ECMC_PARAM_PRECISION:
       if (v != 0.0 && v != 1.0) return fail(ECMC_ERR_ARG, "precision");
@@ -1108,21 +1153,18 @@ int ecmc_set_param(ecmc_t h, int key, double v) {
       if ((double)t != v || !(t == 0 || t == 1 || t == 2 || t == 4 || t == 8 || t == 16 || t == 32))
         return fail(ECMC_ERR_ARG, "lanes per cell must be 0 or a power of two <= 32");
       h->tpc_param = t;
-      drop_graphs(h);
-      return compute_layout(h);
+      return relayout(h, old);
     }
     case ECMC_PARAM_WARPS_PER_BLOCK: {
       const int w = (int)v;
       if ((double)w != v || w < 0 || w > 8) return fail(ECMC_ERR_ARG, "warps per block");
       h->warps_param = w;
-      drop_graphs(h);
-      return compute_layout(h);
+      return relayout(h, old);
     }
     case ECMC_PARAM_STRIP_WIDTH:
       if (!(v >= 0.125 && v <= 2.0)) return fail(ECMC_ERR_ARG, "strip width");
       h->strip_w = (float)v;
-      drop_graphs(h);
-      return compute_layout(h);
+      return relayout(h, old);
     case ECMC_PARAM_GR_DR:
       if (!(v > 0.0 && v < 10.0)) return fail(ECMC_ERR_ARG, "g(r) bin width");
       h->gr_dr = v;
@@ -1145,8 +1187,7 @@ int ecmc_set_param(ecmc_t h, int key, double v) {
     case ECMC_PARAM_PERSISTENT:
       if (v != 0.0 && v != 1.0) return fail(ECMC_ERR_ARG, "persistent must be 0 or 1");
       h->persist_param = (int)v;
-      drop_graphs(h);
-      return compute_layout(h);
+      return relayout(h, old);
     case ECMC_PARAM_WAIT_LIMIT_MS:
       if (!(v >= 0.001 && v <= 600000.0)) return fail(ECMC_ERR_ARG, "wait limit out of range");
       h->wait_ms = v;
@@ -1193,8 +1234,7 @@ int ecmc_set_param(ecmc_t h, int key, double v) {
         g.undo_stride = h->b.cap;
       }
       h->b.reject = (int)v;
-      drop_graphs(h);
-      return compute_layout(h);
+      return relayout(h, old);
     }
     case ECMC_PARAM_REPLAY:
       if (v != 0.0 && v != 1.0) return fail(ECMC_ERR_ARG, "replay must be 0 or 1");
@@ -1205,8 +1245,7 @@ int ecmc_set_param(ecmc_t h, int key, double v) {
       const int m = (int)v;
       if ((double)m != v || m < -1 || m > 2) return fail(ECMC_ERR_ARG, "frame mode");
       h->fmode_param = m;
-      drop_graphs(h);
-      return compute_layout(h);
+      return relayout(h, old);
     }
     default:
       return fail(ECMC_ERR_ARG, "unknown parameter %d", key);
@@ -1257,6 +1296,7 @@ int ecmc_sweep(ecmc_t h, int64_t n) {
   if (!h) return fail(ECMC_ERR_ARG, "NULL handle");
   if (n < 0) return fail(ECMC_ERR_ARG, "n < 0");
   if (!h->valid_state) return fail(ECMC_ERR_STATE, "state invalid after an earlier error");
+  if (!h->layout_ok) return fail(ECMC_ERR_STATE, "no launch shape after an earlier error");
   int rc = ensure_history(h, n);
   if (rc) return rc;
   const bool graph = h->use_graph && !h->timing;
