@@ -1433,10 +1433,11 @@ int ecmc_replica_gr_measure(ecmc_t h, int r) {
   const int R = (int)h->geo.size();
   if (r < -1 || r >= R) return fail(ECMC_ERR_ARG, "replica %d out of range", r);
   const int r0 = r < 0 ? 0 : r, r1 = r < 0 ? R : r + 1;
+  const int c0 = h->geo[r0].cell_off, c1 = h->geo[r1 - 1].cell_off + h->geo[r1 - 1].ncell;
   bool have_fixed = false;
   for (int q = r0; q < r1; ++q) {
     launch_gr(h->geo[q], h->b, h->gr_dr, h->gr_nbins, h->gr_counts + (size_t)q * h->gr_nbins,
-              &have_fixed, h->stream);
+              c0, c1, &have_fixed, h->stream);
     h->gr_meas[q] += 1;
   }
   CK(cudaGetLastError());

@@ -238,7 +238,7 @@ int launch_hexatic(const Geom* geo, const DevBufs& b, double rs, double2* psi_k,
 void set_min_dist(Geom& g);
 void launch_min_dist(const Geom* geo, const DevBufs& b, unsigned long long* out, cudaStream_t s);
 void launch_gr(const Geom& g, const DevBufs& b, double dr, int nbins, unsigned long long* counts,
-               bool* have_fixed, cudaStream_t s);
+               int c0, int c1, bool* have_fixed, cudaStream_t s);
 size_t frame_build_smem(const RecLayout& lay);
 size_t frame_stage_bytes(const RecLayout& lay);
 int configure_frame_build(const RecLayout& lay);
