@@ -317,6 +317,13 @@ int axis_layout(ecmc_ctx* h, int* used) {
     cudaGetLastError();
     return ECMC_OK;
   }
+  // the cells' relative positions: kept by the binning for this kernel only
+  if (!h->b.rel &&
+      cudaMalloc(&h->b.rel, sizeof(float2) * (size_t)h->b.C_total * h->b.cap) != cudaSuccess) {
+    cudaGetLastError();
+    h->b.rel = nullptr;
+    return ECMC_OK;
+  }
   const int n_items = 4 * n_groups;
   h->persistent = h->persist_param;
   h->fused_blocks = h->persistent ? (per_sm * h->n_sm < n_items ? per_sm * h->n_sm : n_items)
@@ -357,6 +364,8 @@ int compute_layout(ecmc_ctx* h) {
   const int rc_axis = axis_layout(h, &used);
   if (rc_axis) return rc_axis;
   if (used) return finish_layout(h);
+  cudaFree(h->b.rel);
+  h->b.rel = nullptr;
   int fmode = auto_fmode(h);
   h->tpc = choose_tpc(h, fmode);
   // isotropic chains in the persistent kernel: the fewest lanes per cell that
@@ -905,7 +914,6 @@ int create_impl(ecmc_t* out, const ecmc_replica_desc_t* desc, int R) {
       cudaMalloc(&b.cell_stats, sizeof(CellStats) * (size_t)C_total) != cudaSuccess ||
       cudaMalloc(&b.totals, sizeof(RunTotals) * R) != cudaSuccess ||
       cudaMalloc(&b.err, sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&b.rel, sizeof(float2) * slots) != cudaSuccess ||
       cudaMalloc(&b.sched, sizeof(unsigned) * 4) != cudaSuccess ||
       cudaMalloc(&b.done, sizeof(unsigned) * (size_t)C_total) != cudaSuccess ||
       cudaMalloc(&h->d_geo, sizeof(Geom) * R) != cudaSuccess ||

@@ -186,7 +186,8 @@ struct DevBufs {
   int* count[2];
   int cur;  // buffer holding the current positions
   float2* rel;  // per slot of the current buffer: FP32 position relative to its cell's
-                // corner, within 2^-21 (L + w) (the axis-chain kernel's screen; or NULL)
+                // corner, within 2^-21 (L + w): the axis-chain kernel's screen (NULL where
+                // another kernel runs: the binning then leaves it out)
   SweepState* state;       // [R]
   CellStats* cell_stats;   // [C_total]
   RunTotals* totals;       // [R]
