@@ -1464,7 +1464,7 @@ int ecmc_hexatic(ecmc_t h, double rs, double* psi, double* psi_k, int32_t* n_nb,
   unsigned long long* bad = h->u64_tmp + 1;
   CK(cudaMemsetAsync(bad, 0, 2 * sizeof(unsigned long long), h->stream));
   double2* pk = reinterpret_cast<double2*>(h->xy_tmp);
-  if (launch_hexatic(h->geo.data(), h->b, rs, pk, h->int_tmp, bad, h->stream))
+  if (launch_hexatic(h->geo.data(), h->b, h->n_sm, rs, pk, h->int_tmp, bad, h->stream))
     return fail(ECMC_ERR_CUDA, "hexatic kernel launch failed: %s",
                 cudaGetErrorString(cudaGetLastError()));
   std::vector<double> hk(2 * (size_t)N);

@@ -234,7 +234,7 @@ void launch_sweep_end(const DevBufs& b, cudaStream_t s);
 void launch_gather(const DevBufs& b, double* xy_out, cudaStream_t s);
 void launch_load_flat(const DevBufs& b, const double* xy_dev, cudaStream_t s);
 void launch_cells_of(const Geom& g, const DevBufs& b, int* cell_of_id, cudaStream_t s);
-int launch_hexatic(const Geom* geo, const DevBufs& b, double rs, double2* psi_k, int* nn,
+int launch_hexatic(const Geom* geo, const DevBufs& b, int n_sm, double rs, double2* psi_k, int* nn,
                    unsigned long long* bad, cudaStream_t s);
 void set_min_dist(Geom& g);
 void launch_min_dist(const Geom* geo, const DevBufs& b, unsigned long long* out, cudaStream_t s);

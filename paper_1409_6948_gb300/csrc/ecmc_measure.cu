@@ -829,7 +829,7 @@ __global__ void __launch_bounds__(128) k_hexatic(
 // geo: the R replicas' geometry on the host.  bad[0] counts the uncertified
 // disks, bad[1] is scratch; both zero on entry.  The undecided disks are listed
 // in the position buffer the next binning overwrites.
-int launch_hexatic(const Geom* geo, const DevBufs& b, double rs, double2* psi_k, int* nn,
+int launch_hexatic(const Geom* geo, const DevBufs& b, int n_sm, double rs, double2* psi_k, int* nn,
                    unsigned long long* bad, cudaStream_t s) {
   // the FP32 decision needs the packing bound of the 64-disk limit
   bool fixed = true;
@@ -847,7 +847,7 @@ int launch_hexatic(const Geom* geo, const DevBufs& b, double rs, double2* psi_k,
   }
   // enough warps to fill the GPU when every disk is left to it
   const int64_t most = ((int64_t)b.C_total * b.cap + 3) / 4;
-  const int64_t blocks = most < 152 * 12 ? most : 152 * 12;
+  const int64_t blocks = most < 12 * (int64_t)n_sm ? most : 12 * (int64_t)n_sm;
   k_hexatic<<<(unsigned)blocks, 128, 0, s>>>(
       b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], b.pid[b.cur],
       b.count[b.cur], rs, psi_k, nn, fixed ? list : nullptr, n_list, bad);
