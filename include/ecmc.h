@@ -175,7 +175,9 @@ typedef struct {
   int64_t lifts;       /* contacts with an active disk (budget passed on)       */
   int64_t frozen_hits; /* contacts with a frozen disk (chain reflected)         */
   int64_t wall_hits;   /* reflections at a cell wall (not counted as events)    */
-  int64_t fp64_evals;  /* candidates evaluated in FP64                          */
+  int64_t fp64_evals;  /* candidates evaluated in FP64 (axis chains with static
+                        * candidates: three a leg, and every object of the
+                        * frame in cells that have none)                       */
   double sum_b;        /* sum over contacts of the separation along d           */
   double sum_disp;     /* sum over chains of the displacement budget ell        */
   int64_t replayed_legs; /* reflection legs (frozen disk or wall) of a chain that

@@ -757,9 +757,11 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
     s.lifts = n_tot - n_walls - n_frozen;
     s.frozen = n_frozen;
     s.walls = n_walls;
-    // three candidates for every leg that was not replayed, the last legs of
-    // the chains among them
-    s.fp64_evals = 3 * (n_tot - n_replayed + n_chains - n_rejected);
+    // for every leg that was not replayed, the last legs of the chains among
+    // them: the three windows' candidates (whether or not an object is there)
+    // and, without static candidates, every other object of the frame
+    const long long legs = (long long)n_tot - n_replayed + n_chains - n_rejected;
+    s.fp64_evals = legs * (irregular ? 2 + f.nobj : 3);
     s.chains = n_chains;
     s.n_mem = nmem;
     s.replayed = n_replayed;

@@ -51,8 +51,9 @@ struct SweepState {
 // Per-cell results of one sweep (written by the cell's phase).
 struct CellStats {
   double sum_b;     // contact sum of the cell's chains, in chain order
+  long long fp64_evals;
   int events, lifts, frozen, walls;
-  int fp64_evals, chains, n_mem, replayed;
+  int chains, n_mem, replayed;
   int rejected;     // chains rejected under the rejecting boundary rule
 };
 
