@@ -75,8 +75,8 @@ extern "C" {
  * ECMC_PREC_FP32_GEOM (default) = candidates screened in FP32 cell-relative
  * coordinates with rigorous error bounds, the contact decided in FP64.  Both
  * give bit-identical trajectories.  Axis chains in cells small enough for
- * shared memory find a disk's few candidates once per colour phase and test
- * them in FP64 under either value. */
+ * shared memory find a disk's few candidates once per colour phase, by either
+ * method, and test them in FP64 under both. */
 #define ECMC_PARAM_PRECISION 3
 /* Replica number: second word of the Philox key (seed, replica); an integer
  * in [0, 9e15], so that the double passed to set_param holds it exactly. */

@@ -2,7 +2,7 @@
 // candidates and chains of the active cells of one colour phase.  Prints the
 // cells' counters and a hash of the members' coordinates, which have to be the
 // same in whatever order the lanes run.
-//   axis_lanes k eta cells ell n_m boundary list_mode start downwards
+//   axis_lanes k eta cells ell n_m boundary list_mode start precision downwards
 // k^2 disks; start 0: square lattice, displaced; 1: rows staggered by sigma / 2
 // (cells without static candidates).
 #include "warp_lanes.h"
@@ -11,7 +11,17 @@ namespace ecmc {
 inline double sqrt_rn(double x) { return std::sqrt(x); }
 }  // namespace ecmc
 
+#include "ecmc_device.cuh"
+#include "ecmc_internal.cuh"
+// comparisons of the FP64 search for candidates
+static long n_exact;
+static bool counted_dlt(double a, double b) {
+  __atomic_fetch_add(&n_exact, 1, __ATOMIC_RELAXED);
+  return ecmc::dlt(a, b);
+}
+#define dlt counted_dlt
 #include "ecmc_axis.cuh"
+#undef dlt
 
 #include <cstdio>
 #include <cstdlib>
@@ -24,7 +34,7 @@ using namespace ecmc;
 #endif
 
 int main(int argc, char** argv) {
-  if (argc != 10) return 2;
+  if (argc != 11) return 2;
   constexpr int TPC = LANES, CPW = 32 / TPC;
   const int k = std::atoi(argv[1]), cells = std::atoi(argv[3]), N = k * k;
   const double eta = std::atof(argv[2]), L = std::sqrt(N * M_PI / (4.0 * eta));
@@ -42,6 +52,7 @@ int main(int argc, char** argv) {
   g.n_m = std::atoi(argv[5]);
   g.list_mode = std::atoi(argv[7]);
   g.boundary = reject;
+  g.precision = std::atoi(argv[9]);
   g.seed = 1;
   double M = 1.0;
   while (M < g.w + 1.01) M *= 2.0;
@@ -133,12 +144,16 @@ int main(int argc, char** argv) {
                    1099511628211ull;
     }
   };
-  const bool fine = warp::run(lane_main, 32, std::atoi(argv[9]) != 0);
+  const bool fine = warp::run(lane_main, 32, std::atoi(argv[10]) != 0);
   for (int gi = 0; gi < CPW && gi < n_active; ++gi) {
     const CellStats& s = cs[2 * (gi % (cells / 2)) + 2 * (gi / (cells / 2)) * cells];
     std::printf("cell %d irregular %llu: chains %d events %d lifts %d frozen %d walls %d replayed %d "
                 "rejected %d sum_b %.17g hash %016llx\n", gi, irr[gi], s.chains, s.events, s.lifts,
                 s.frozen, s.walls, s.replayed, s.rejected, s.sum_b, hash[gi]);
   }
+  int members = 0;
+  for (int gi = 0; gi < CPW && gi < n_active; ++gi)
+    members += cs[2 * (gi % (cells / 2)) + 2 * (gi / (cells / 2)) * cells].n_mem;
+  std::printf("members %d fp64 comparisons %ld\n", members, n_exact);
   return fine && err == 0 ? 0 : 3;
 }

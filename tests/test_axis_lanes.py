@@ -36,7 +36,7 @@ def programs(tmp_path_factory):
 def test_lanes_order_their_memory(programs, case):
     first = None
     for n in LANES:
-        up, down = (lanes.run(programs[n], CASES[case] + d) for d in (" 0", " 1"))
+        up, down = (lanes.run(programs[n], CASES[case] + " 1" + d)[:-1] for d in (" 0", " 1"))
         assert up == down
         assert len(up) == min(16, 32 // n)
         # how much of a chain is replayed depends on the lanes, what it does not
@@ -49,3 +49,16 @@ def test_lanes_order_their_memory(programs, case):
     n_rej = sum(int(re.search(r"rejected (\d+)", c).group(1)) for c in first)
     n_ch = sum(int(re.search(r"chains (\d+)", c).group(1)) for c in first)
     assert (0 < n_rej < n_ch) if "rejected" in case else n_rej == 0
+
+
+@pytest.mark.parametrize("n", LANES)
+def test_fp64_candidates_are_chosen_in_fp64(programs, n):
+    # the same candidates either way; FP32 leaves next to nothing to FP64 here,
+    # and the FP64 setting compares every object of a window's strips
+    case = CASES["turn_backs"]
+    fp32, fp64 = (lanes.run(programs[n], case + p) for p in (" 1 0", " 0 0"))
+    assert fp32[:-1] == fp64[:-1]
+    counts = [[int(v) for v in re.findall(r"\d+", x[-1].replace("fp64", ""))]
+              for x in (fp32, fp64)]
+    members = counts[0][0]
+    assert counts[0][1] < members < 3 * members <= counts[1][1]
