@@ -261,6 +261,52 @@ int choose_axis_tpc(ecmc_ctx* h) {
   return 32;
 }
 
+// lambda0 of Sec. 4
+double mean_free_path(const Geom& g) {
+  const double pi = 3.14159265358979323846;
+  const double eta = (double)g.N * pi * g.sigma * g.sigma / (4.0 * g.L * g.L);
+  const double eta_hcp = pi / (2.0 * std::sqrt(3.0));
+  return g.sigma * (eta_hcp - eta) / (2.0 * eta_hcp);
+}
+
+// Whether the axis-chain kernel is the faster one.  It finds the candidates of
+// every member of a cell, in a time that grows with the members times the
+// objects of a strip of width sigma (mean numbers m, s); the per-phase kernels
+// search a strip at every leg instead.  So few legs in a large cell are the
+// per-phase kernels' case.  Measured on GB300, eta = 0.72, us per sweep with
+// this kernel / the per-phase ones, for about 2, 40, 160 and 640 legs a cell:
+//   side  8.4, 32^2 cells: 156 / 161,  234 / 737,   588 / 3078, 2127 / 12767
+//   side 16.7, 16^2:       458 / 159,  667 / 907,  1041 / 2979, 2677 / 10959
+//   side 22.3, 12^2:       870 / 218, 1058 / 754,  1904 / 2376, 4211 / 8940
+//   side 26.7, 10^2:      1315 / 214, 1997 / 775,  2569 / 2474, 4330 / 8611
+//   side 35.9, 10^2:      2828 / 394, 4245 / 1017, 5324 / 2887, 6741 / 10009
+// They meet at m s / 120 legs; with the candidates chosen in FP64 (16.7: 1002 /
+// 179, 1175 / 1332; 35.9: 10405 / 4680, 14140 / 16867) at m s / 80.  Below m s =
+// 1000 neither lost.  Cells too large for FP32 to choose the candidates at all
+// (38 sigma and more) lost at any number of legs: 14775 / 5474 at side 38.9 and
+// 320 legs, 23391 / 9235 at 690.
+bool axis_pays(const ecmc_ctx* h) {
+  double gain = 0.0;  // legs above the meeting point, over the active cells
+  for (const Geom& g : h->geo) {
+    const double rho = (double)g.N / (g.L * g.L);
+    const double m = rho * g.w * g.h;
+    const double s = rho * g.sigma * (0.5 * (g.w + g.h) + 2.0 * g.sigma);
+    const double o = rho * (g.w + 2.0 * g.sigma) * (g.h + 2.0 * g.sigma);
+    // as in axis_build: the error of FP32 and of the fixed point for o objects
+    const double ext = (g.w > g.h ? g.w : g.h) + 2.0 * g.sigma;
+    const int bits = std::ilogb(o + 3.0 * std::sqrt(o) + 1.0) + 1;
+    const bool coarse =
+        2.0 * g.eps_d + (4e-7 - 2e-4) * g.sigma + ext * std::ldexp(1.0, bits - 29) > 0.0;
+    const double lambda0 = mean_free_path(g);
+    const double side = g.w > g.h ? g.w : g.h;
+    const double ell = g.boundary == 1 && g.ell > side ? side : g.ell;
+    const double legs = lambda0 > 0.0 ? g.n_m * (1.0 + ell / lambda0) : 1e9 * g.n_m;
+    const double even = m * s < 1000.0 ? 0.0 : m * s / (g.precision == 0 ? 80.0 : 120.0);
+    gain += (double)g.nact * (coarse ? -m * s : legs - even);
+  }
+  return gain > 0.0;
+}
+
 constexpr size_t kSmemLimit = 232448;  // opt-in shared memory per block on sm_103
 
 // Frame placement of the per-phase kernels: whole frames in shared memory when
@@ -286,8 +332,8 @@ int need_records(ecmc_ctx* h, size_t need) {
   return ECMC_OK;
 }
 
-// Axis chains: the kernel of ecmc_axis.cuh wherever a cell fits in its shared
-// memory, in one persistent launch per sweep or one launch per phase.  *used
+// Axis chains: the kernel of ecmc_axis.cuh wherever it pays and a cell fits in
+// its shared memory, in one persistent launch per sweep or one launch per phase.  *used
 // says whether it does.
 int axis_layout(ecmc_ctx* h, int* used) {
   *used = 0;
@@ -296,6 +342,7 @@ int axis_layout(ecmc_ctx* h, int* used) {
   if (h->tpc_param && h->tpc_param != 32 &&
       phase_smem_bytes(layout_for(h, h->tpc_param), 1, auto_fmode(h)) > kSmemLimit)
     return ECMC_OK;  // refused by compute_layout: frames too large for so few lanes
+  if (!axis_pays(h)) return ECMC_OK;
   const int tpc = choose_axis_tpc(h);
   const AxisShape s = axis_shape_for(h, tpc);
   if (s.co_h > kAxisMaxObjects) return ECMC_OK;
@@ -445,13 +492,18 @@ void drop_graphs(ecmc_ctx* h) {
 
 // The parameters that the launch shape follows from.
 struct LayoutParams {
-  int tpc, warps, fmode, persist, dir_mode, iso, boundary, reject;
+  int tpc, warps, fmode, persist, dir_mode, iso, boundary, reject, precision;
   float strip_w;
+  std::vector<int> n_m;
 };
 
 LayoutParams layout_params(const ecmc_ctx* h) {
-  return {h->tpc_param, h->warps_param,      h->fmode_param,     h->persist_param,
-          h->geo[0].dir_mode, h->b.iso, h->geo[0].boundary, h->b.reject, h->strip_w};
+  LayoutParams p = {h->tpc_param,       h->warps_param, h->fmode_param,
+                    h->persist_param,   h->geo[0].dir_mode, h->b.iso,
+                    h->geo[0].boundary, h->b.reject,    h->precision,
+                    h->strip_w,         {}};
+  for (const Geom& g : h->geo) p.n_m.push_back(g.n_m);
+  return p;
 }
 
 // One of them has changed: the new launch shape.  Where that is refused or
@@ -471,9 +523,13 @@ int relayout(ecmc_ctx* h, const LayoutParams& old) {
   h->strip_w = old.strip_w;
   h->b.iso = old.iso;
   h->b.reject = old.reject;
-  for (Geom& g : h->geo) {
+  h->precision = old.precision;
+  for (size_t r = 0; r < h->geo.size(); ++r) {
+    Geom& g = h->geo[r];
     g.dir_mode = old.dir_mode;
     g.boundary = old.boundary;
+    g.precision = old.precision;
+    g.n_m = old.n_m[r];
   }
   compute_layout(h);  // (ecmc_sweep refuses to run should this fail, too)
   std::memcpy(g_msg, msg, sizeof(msg));
@@ -687,10 +743,7 @@ int load_positions_dev(ecmc_ctx* h, const double* xy_dev, int64_t t0) {
 }
 
 int default_nm(const Geom& g) {
-  const double pi = 3.14159265358979323846;
-  const double eta = (double)g.N * pi * g.sigma * g.sigma / (4.0 * g.L * g.L);
-  const double eta_hcp = pi / (2.0 * std::sqrt(3.0));
-  const double lambda0 = g.sigma * (eta_hcp - eta) / (2.0 * eta_hcp);
+  const double lambda0 = mean_free_path(g);
   if (!(g.ell > 0.0) || !(lambda0 > 0.0)) return 1;
   const double nm = (double)g.N / (double)g.ncell * lambda0 / g.ell;
   const double r = std::floor(nm + 0.5);
@@ -1133,8 +1186,7 @@ int ecmc_set_param(ecmc_t h, int key, double v) {
     case ECMC_PARAM_N_CHAINS: {
       if (!(v >= 1.0 && v <= 1e6) || v != std::floor(v)) return fail(ECMC_ERR_ARG, "n_m");
       for (Geom& g : h->geo) g.n_m = (int)v;
-      drop_graphs(h);
-      int rc = upload_geometry(h);
+      int rc = relayout(h, old);
       if (rc) return rc;
       return realloc_chain_recs(h);
     }
@@ -1150,8 +1202,7 @@ int ecmc_set_param(ecmc_t h, int key, double v) {
       if (v != 0.0 && v != 1.0) return fail(ECMC_ERR_ARG, "precision");
       h->precision = (int)v;
       for (Geom& g : h->geo) g.precision = (int)v;
-      drop_graphs(h);
-      return upload_geometry(h);
+      return relayout(h, old);
     case ECMC_PARAM_REPLICA:
       if (!(v >= 0.0) || v != std::floor(v) || v > 9.0e15) return fail(ECMC_ERR_ARG, "replica");
       h->geo[0].replica = (uint64_t)v;
