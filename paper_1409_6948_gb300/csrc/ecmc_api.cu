@@ -261,48 +261,52 @@ int choose_axis_tpc(ecmc_ctx* h) {
   return 32;
 }
 
-// lambda0 of Sec. 4
-double mean_free_path(const Geom& g) {
-  const double pi = 3.14159265358979323846;
-  const double eta = (double)g.N * pi * g.sigma * g.sigma / (4.0 * g.L * g.L);
-  const double eta_hcp = pi / (2.0 * std::sqrt(3.0));
-  return g.sigma * (eta_hcp - eta) / (2.0 * eta_hcp);
-}
-
 // Whether the axis-chain kernel is the faster one.  It finds the candidates of
-// every member of a cell, in a time that grows with the members times the
-// objects of a strip of width sigma (mean numbers m, s); the per-phase kernels
-// search a strip at every leg instead.  So few legs in a large cell are the
-// per-phase kernels' case.  Measured on GB300, eta = 0.72, us per sweep with
-// this kernel / the per-phase ones, for about 2, 40, 160 and 640 legs a cell:
-//   side  8.4, 32^2 cells: 156 / 161,  234 / 737,   588 / 3078, 2127 / 12767
-//   side 16.7, 16^2:       458 / 159,  667 / 907,  1041 / 2979, 2677 / 10959
-//   side 22.3, 12^2:       870 / 218, 1058 / 754,  1904 / 2376, 4211 / 8940
-//   side 26.7, 10^2:      1315 / 214, 1997 / 775,  2569 / 2474, 4330 / 8611
-//   side 35.9, 10^2:      2828 / 394, 4245 / 1017, 5324 / 2887, 6741 / 10009
-// They meet at m s / 120 legs; with the candidates chosen in FP64 (16.7: 1002 /
-// 179, 1175 / 1332; 35.9: 10405 / 4680, 14140 / 16867) at m s / 80.  Below m s =
-// 1000 neither lost.  Cells too large for FP32 to choose the candidates at all
-// (38 sigma and more) lost at any number of legs: 14775 / 5474 at side 38.9 and
-// 320 legs, 23391 / 9235 at 690.
+// every member of a cell, in a time that grows with the members m and the
+// objects s of a strip of width sigma; the per-phase kernels search a strip at
+// every leg instead, so that few legs in a large cell are their case.  The
+// difference of the fixed costs, 0.4 m + 0.08 m s - 20 us a sweep, against the
+// gain per leg of a cell, 2.5 us and more where chains are dense or cells below
+// 24 sigma, is a fit to 300 pairs on GB300 (eta 0.1 to 0.72, sides of 12 to 35
+// sigma, 6^2 and 24^2 cells, 4 to 1500 legs a cell): the worst choice costs 4 %
+// (14 % with the candidates chosen in FP64, where both costs are higher).  us
+// per sweep, this kernel / the per-phase ones, 24^2 cells, for 4, 20, 100, 400 and
+// 1500 legs a cell:
+//   eta 0.72, side 12:  278 / 175,   318 / 405,   490 / 1614, 1167 / 5766, 3666 / 20916
+//   eta 0.72, side 23: 1230 / 246,  1312 / 401,  1608 / 1079, 2679 / 3608, 6308 / 12717
+//   eta 0.72, side 35: 3806 / 402,  3902 / 569,  4321 / 1340, 5291 / 4151, 7881 / 13689
+//   eta 0.25, side 23:  334 / 133,   392 / 240,   601 / 734,  1507 / 2512, 4764 / 9015
+// and in FP64 at eta 0.72, side 23: 2642 / 273, 2716 / 516, 3003 / 1627, 4115 /
+// 5730, 8048 / 20452.  Cells too
+// large for FP32 to choose the candidates at all (38 sigma and more) lost at any
+// number of legs: 14775 / 5474 at side 38.9 and 520 legs, 23391 / 9235 at 1100.
 bool axis_pays(const ecmc_ctx* h) {
-  double gain = 0.0;  // legs above the meeting point, over the active cells
+  double gain = 0.0;  // us a sweep, over the active cells
   for (const Geom& g : h->geo) {
-    const double rho = (double)g.N / (g.L * g.L);
+    const double pi = 3.14159265358979323846;
+    const double rho = (double)g.N / (g.L * g.L), s1 = g.sigma;
+    const double eta = rho * pi * s1 * s1 / 4.0;
     const double m = rho * g.w * g.h;
-    const double s = rho * g.sigma * (0.5 * (g.w + g.h) + 2.0 * g.sigma);
-    const double o = rho * (g.w + 2.0 * g.sigma) * (g.h + 2.0 * g.sigma);
+    const double s = rho * s1 * (0.5 * (g.w + g.h) + 2.0 * s1);
+    const double o = rho * (g.w + 2.0 * s1) * (g.h + 2.0 * s1);
     // as in axis_build: the error of FP32 and of the fixed point for o objects
-    const double ext = (g.w > g.h ? g.w : g.h) + 2.0 * g.sigma;
+    const double side = g.w > g.h ? g.w : g.h;
     const int bits = std::ilogb(o + 3.0 * std::sqrt(o) + 1.0) + 1;
     const bool coarse =
-        2.0 * g.eps_d + (4e-7 - 2e-4) * g.sigma + ext * std::ldexp(1.0, bits - 29) > 0.0;
-    const double lambda0 = mean_free_path(g);
-    const double side = g.w > g.h ? g.w : g.h;
-    const double ell = g.boundary == 1 && g.ell > side ? side : g.ell;
-    const double legs = lambda0 > 0.0 ? g.n_m * (1.0 + ell / lambda0) : 1e9 * g.n_m;
-    const double even = m * s < 1000.0 ? 0.0 : m * s / (g.precision == 0 ? 80.0 : 120.0);
-    gain += (double)g.nact * (coarse ? -m * s : legs - even);
+        2.0 * g.eps_d + (4e-7 - 2e-4) * s1 + (side + 2.0 * s1) * std::ldexp(1.0, bits - 29) > 0.0;
+    // legs a cell: contacts at the rate 2 rho sigma g(sigma) with Henderson's
+    // contact value for hard disks (a few per cent off up to eta = 0.68, low
+    // above), reflections at the walls, the last leg; a rejected chain ends at
+    // its first reflection
+    const double contact = (1.0 - 7.0 * eta / 16.0) / ((1.0 - eta) * (1.0 - eta));
+    const double ell = g.boundary == 1 && g.ell > 0.5 * side ? 0.5 * side : g.ell;
+    const double legs = g.n_m * (1.0 + ell * (2.0 * rho * s1 * contact + 1.0 / side));
+    const double dense = eta > 0.6 ? (eta - 0.6) / 0.12 : 0.0;
+    const bool fp64 = g.precision == 0;
+    const double small = side < 24.0 * s1 ? 3.0 - side / (12.0 * s1) : 1.0;
+    const double fixed = fp64 ? 0.6 * m + 0.28 * m * s - 20.0 : 0.4 * m + 0.08 * m * s - 20.0;
+    const double per_leg = small * (fp64 ? 4.0 + 10.0 * dense : 2.5 + 3.0 * dense);
+    gain += (double)g.nact * (coarse ? -fixed : legs * per_leg - fixed);
   }
   return gain > 0.0;
 }
@@ -743,7 +747,10 @@ int load_positions_dev(ecmc_ctx* h, const double* xy_dev, int64_t t0) {
 }
 
 int default_nm(const Geom& g) {
-  const double lambda0 = mean_free_path(g);
+  const double pi = 3.14159265358979323846;
+  const double eta = (double)g.N * pi * g.sigma * g.sigma / (4.0 * g.L * g.L);
+  const double eta_hcp = pi / (2.0 * std::sqrt(3.0));
+  const double lambda0 = g.sigma * (eta_hcp - eta) / (2.0 * eta_hcp);
   if (!(g.ell > 0.0) || !(lambda0 > 0.0)) return 1;
   const double nm = (double)g.N / (double)g.ncell * lambda0 / g.ell;
   const double r = std::floor(nm + 0.5);

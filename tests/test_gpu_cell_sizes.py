@@ -27,11 +27,12 @@ def compare(g, x, y, st):
         (st.events, st.lifts, st.frozen_hits, st.wall_hits)
 
 
-# about 30 legs a chain; static candidates pay from m s / 120 legs a cell (m
-# members, s objects of a strip one sigma wide), m s / 80 under ECMC_PREC_FP64
+# about 49 legs a chain; static candidates pay from 49, 117, 308 and 462 legs a cell
+# of 16.7, 20.9, 27.1 and 31.3 sigma, from 389 at 27.1 sigma under ECMC_PREC_FP64
 @pytest.mark.parametrize("k,side,nm,prec,persistent,fmode,kernels", [
-    (32, 16.7, 1, 1, 1, -1, 12),
     (32, 16.7, 2, 1, 1, -1, 5),
+    (40, 20.9, 1, 1, 1, -1, 12),
+    (40, 20.9, 4, 1, 1, -1, 5),
     (52, 27.1, 8, 1, 1, -1, 5),
     (52, 27.1, 8, 1, 0, -1, 8),
     (52, 27.1, 8, 1, 1, 0, 5),       # candidate lists in shared memory
