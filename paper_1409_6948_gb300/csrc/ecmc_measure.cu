@@ -689,13 +689,14 @@ __global__ void __launch_bounds__(64) k_hexatic_fixed(
 }
 
 // The FP64 decision, a warp per disk.  list: the bucket slots to work on
-// (*n_list of them), or NULL for every slot.
+// (*n_list of them; more than `most` are left to k_hexatic_many), or NULL for
+// every slot.
 __global__ void __launch_bounds__(128) k_hexatic(
     const Geom* __restrict__ rg, const int* __restrict__ cell_rep, int C_total, int cap,
     const double* __restrict__ px, const double* __restrict__ py, const int* __restrict__ pid,
     const int* __restrict__ cnt, double rs_arg, double2* __restrict__ psi_out,
     int* __restrict__ nn_out, const int* __restrict__ list, const unsigned long long* n_list,
-    unsigned long long* bad) {
+    int64_t most, unsigned long long* bad) {
   constexpr unsigned FULL = 0xffffffffu;
   __shared__ double2 s_raw[4][kHexMaxCand], s_cand[4][kHexMaxCand];
   __shared__ int s_id[4][kHexMaxCand];
@@ -704,6 +705,7 @@ __global__ void __launch_bounds__(128) k_hexatic(
   double2* const cand = s_cand[warp];
   int* const cid = s_id[warp];
   const int64_t total = list != nullptr ? (int64_t)*n_list : (int64_t)C_total * cap;
+  if (list != nullptr && total > most) return;
   const int64_t step = (int64_t)gridDim.x * 4;
   for (int64_t at = (int64_t)blockIdx.x * 4 + warp; at < total; at += step) {
     const int i = list != nullptr ? list[at] : (int)at;
@@ -826,6 +828,130 @@ __global__ void __launch_bounds__(128) k_hexatic(
   }
 }
 
+// The same decision, a thread per disk, where many disks are left to FP64
+// (crystals, rs above 3.5 sigma).  A warp shortens one disk's chain of
+// dependent divisions, but its 32 lanes seldom all have work: once threads fill
+// the GPU, a thread per disk is the faster one.  GB300, us per call with a warp
+// / a thread per disk: the undecided disks of a square lattice of 2^14 2520 /
+// 1860, of 2^16 9590 / 4630, of 2^20 144700 / 46000; every slot, rs = 3.9 sigma,
+// N = 2^14 3000 / 3780, 25,600 4420 / 5180, 2^16 11930 / 8430, 2^20 156100 /
+// 126900.
+__global__ void __launch_bounds__(32) k_hexatic_many(
+    const Geom* __restrict__ rg, const int* __restrict__ cell_rep, int C_total, int cap,
+    const double* __restrict__ px, const double* __restrict__ py, const int* __restrict__ pid,
+    const int* __restrict__ cnt, double rs_arg, double2* __restrict__ psi_out,
+    int* __restrict__ nn_out, const int* __restrict__ list, const unsigned long long* n_list,
+    int64_t most, unsigned long long* bad) {
+  extern __shared__ __align__(16) unsigned char hsm[];
+  double2* const cand = reinterpret_cast<double2*>(hsm) + (size_t)threadIdx.x * kHexMaxCand;
+  int* const cid = reinterpret_cast<int*>(reinterpret_cast<double2*>(hsm) +
+                                          (size_t)blockDim.x * kHexMaxCand) +
+                   (size_t)threadIdx.x * kHexMaxCand;
+  const int64_t total = list != nullptr ? (int64_t)*n_list : (int64_t)C_total * cap;
+  if (list != nullptr && total <= most) return;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; at < total; at += step) {
+    const int i = list != nullptr ? list[at] : (int)at;
+    const int c = i / cap, k = i - c * cap;
+    if (k >= min(cnt[c], cap)) continue;
+    const Geom& g = rg[cell_rep[c]];
+    const int lcell = c - g.cell_off;
+    const int cx = lcell % g.cells_x, cy = lcell / g.cells_x;
+    const double xi = px[i], yi = py[i];
+    const double L = g.L;
+    const double rs = rs_arg > 0.0 ? rs_arg : 3.5 * g.sigma;
+    const double rs2 = rs * rs, v2max = 0.25 * rs * rs;
+    const int Rx = (int)ceil(rs * g.inv_w * (1.0 + 1e-9));
+    const int Ry = (int)ceil(rs * g.inv_h * (1.0 + 1e-9));
+    const NbRange rx = nb_range(Rx, g.cells_x), ry = nb_range(Ry, g.cells_y);
+    const bool absx = (2 * Rx + 1 >= g.cells_x), absy = (2 * Ry + 1 >= g.cells_y);
+    int nc = 0;
+    bool over = false;
+    for (int oy = 0; oy < ry.n; ++oy) {
+      const int qy = absy ? oy : ((cy + ry.first + oy) % g.cells_y + g.cells_y) % g.cells_y;
+      for (int ox = 0; ox < rx.n; ++ox) {
+        const int qx = absx ? ox : ((cx + rx.first + ox) % g.cells_x + g.cells_x) % g.cells_x;
+        const int q = g.cell_off + qy * g.cells_x + qx;
+        const int nq = min(cnt[q], cap), b0 = q * cap;
+        for (int kk = 0; kk < nq; ++kk) {
+          const int j = b0 + kk;
+          if (j == i) continue;
+          const double ddx = wrap_half(px[j] - xi, L);
+          const double ddy = wrap_half(py[j] - yi, L);
+          if (!(ddx * ddx + ddy * ddy < rs2)) continue;
+          if (nc == kHexMaxCand) {
+            over = true;
+            continue;
+          }
+          // insertion by disk id (the order the sums below run in)
+          const int id = pid[j];
+          int pos = nc;
+          while (pos > 0 && cid[pos - 1] > id) {
+            cand[pos] = cand[pos - 1];
+            cid[pos] = cid[pos - 1];
+            --pos;
+          }
+          cand[pos] = make_double2(ddx, ddy);
+          cid[pos] = id;
+          ++nc;
+        }
+      }
+    }
+    const int64_t id = g.n_off + pid[i];
+    if (over) {
+      atomicAdd(bad, 1ull);
+      psi_out[id] = make_double2(0.0, 0.0);
+      nn_out[id] = -1;
+      continue;
+    }
+    double re = 0.0, im = 0.0;
+    int n = 0;
+    bool ok = true;
+    for (int l = 0; l < nc; ++l) {
+      const double2 dl = cand[l];
+      const double ux = -dl.y, uy = dl.x;
+      const double px0 = 0.5 * dl.x, py0 = 0.5 * dl.y;
+      double tlo = -__longlong_as_double(0x7ff0000000000000ll);
+      double thi = __longlong_as_double(0x7ff0000000000000ll);
+      for (int m = 0; m < nc && tlo < thi; ++m) {
+        if (m == l) continue;
+        const double2 dm = cand[m];
+        const double a = ux * dm.x + uy * dm.y;
+        const double b = 0.5 * (dm.x * dm.x + dm.y * dm.y) - (px0 * dm.x + py0 * dm.y);
+        if (a > 0.0) {
+          const double t = b / a;
+          if (t < thi) thi = t;
+        } else if (a < 0.0) {
+          const double t = b / a;
+          if (t > tlo) tlo = t;
+        } else if (b < 0.0) {
+          thi = -__longlong_as_double(0x7ff0000000000000ll);
+        }
+      }
+      if (!(tlo < thi)) continue;
+      if (isinf(tlo) || isinf(thi)) {
+        ok = false;
+      } else {
+        const double vx0 = px0 + tlo * ux, vy0 = py0 + tlo * uy;
+        const double vx1 = px0 + thi * ux, vy1 = py0 + thi * uy;
+        if (!(vx0 * vx0 + vy0 * vy0 < v2max) || !(vx1 * vx1 + vy1 * vy1 < v2max)) ok = false;
+      }
+      const double zx = dl.x, zy = dl.y;
+      const double z2x = zx * zx - zy * zy, z2y = 2.0 * zx * zy;
+      const double z3x = z2x * zx - z2y * zy, z3y = z2x * zy + z2y * zx;
+      const double z6x = z3x * z3x - z3y * z3y, z6y = 2.0 * z3x * z3y;
+      const double r2 = zx * zx + zy * zy;
+      const double r6 = r2 * r2 * r2;
+      re += z6x / r6;
+      im += z6y / r6;
+      ++n;
+    }
+    if (!ok) atomicAdd(bad, 1ull);
+    psi_out[id] = make_double2(n > 0 ? re / (double)n : 0.0, n > 0 ? im / (double)n : 0.0);
+    nn_out[id] = n;
+  }
+}
+
 // geo: the R replicas' geometry on the host.  bad[0] counts the uncertified
 // disks, bad[1] is scratch; both zero on entry.  The undecided disks are listed
 // in the position buffer the next binning overwrites.
@@ -845,12 +971,27 @@ int launch_hexatic(const Geom* geo, const DevBufs& b, int n_sm, double rs, doubl
         b.rg, b.cell_rep, b.C_total, b.cap, chunks, b.px[b.cur], b.py[b.cur], b.pid[b.cur], fxy,
         b.count[b.cur], rs, psi_k, nn, list, n_list);
   }
-  // enough warps to fill the GPU when every disk is left to it
-  const int64_t most = ((int64_t)b.C_total * b.cap + 3) / 4;
-  const int64_t blocks = most < 12 * (int64_t)n_sm ? most : 12 * (int64_t)n_sm;
-  k_hexatic<<<(unsigned)blocks, 128, 0, s>>>(
-      b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], b.pid[b.cur],
-      b.count[b.cur], rs, psi_k, nn, fixed ? list : nullptr, n_list, bad);
+  // either kernel with enough blocks to fill the GPU; with a list both are
+  // launched and its length, known on the device, picks one
+  const int64_t slots = (int64_t)b.C_total * b.cap;
+  const int64_t most = (fixed ? 96 : 256) * (int64_t)n_sm;  // disks a warp each
+  const int* const which = fixed ? list : nullptr;
+  if (fixed || b.N_total <= most) {
+    const int64_t need = (slots + 3) / 4;
+    const int64_t blocks = need < 12 * (int64_t)n_sm ? need : 12 * (int64_t)n_sm;
+    k_hexatic<<<(unsigned)blocks, 128, 0, s>>>(
+        b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], b.pid[b.cur],
+        b.count[b.cur], rs, psi_k, nn, which, n_list, most, bad);
+  }
+  if (b.N_total > most) {
+    const size_t sm = 32 * kHexMaxCand * (sizeof(double2) + sizeof(int));
+    const int64_t need = (slots + 31) / 32;
+    // a list is dealt out over the threads that fit at once, slots by the block
+    const int64_t blocks = fixed && need > 5 * (int64_t)n_sm ? 5 * (int64_t)n_sm : need;
+    k_hexatic_many<<<(unsigned)blocks, 32, sm, s>>>(
+        b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], b.pid[b.cur],
+        b.count[b.cur], rs, psi_k, nn, which, n_list, most, bad);
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
