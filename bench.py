@@ -41,7 +41,7 @@ UNIT = "events/s"
 # (smem_bytes_per_event below).
 #
 # Counters of the persistent sweep kernel k_sweep_axis<8 lanes per cell> that
-# need more than one ncu pass, for both placements of the frame coordinates
+# need more than one ncu pass, for both placements of the candidate lists
 # the autotuner chooses between (frame mode 1, global scratch; frame mode 0,
 # shared memory): captured at N = 640,000, eta = 0.72 with the parameters of
 # the full size (188 x 188 cells, about 8,800 active cells per phase), one
@@ -55,8 +55,8 @@ FUSED_ITERATIONS_CAPTURE = 1526651               # contacts + walls + chain ends
 FUSED_CAPTURES = {
     # frame mode: dram__bytes_read.sum + _write.sum, smsp__inst_executed_pipe_fp64.sum,
     # sm__pipe_fp64_cycles_active (% of active cycles)
-    1: {"dram_bytes": 35535616 + 2022912, "fp64_winst": 3459317, "fp64_pipe_pct": 43.19},
-    0: {"dram_bytes": 35166976 + 162816, "fp64_winst": 3458624, "fp64_pipe_pct": 41.71},
+    1: {"dram_bytes": 35534336 + 2530560, "fp64_winst": 3459062, "fp64_pipe_pct": 42.24},
+    0: {"dram_bytes": 35170304 + 202240, "fp64_winst": 3459385, "fp64_pipe_pct": 40.49},
 }
 FUSED_CAPTURE_FRAME_MODE = 1                     # the autotuner's choice at N = 1M
 FUSED_DRAM_BYTES_CAPTURE = FUSED_CAPTURES[1]["dram_bytes"]
@@ -974,8 +974,8 @@ def run_ours(args):
         ms_max, events_all, sweeps_all = ms, float(events), float(sweeps)
     value = events_all / (ms_max * 1e-3)
 
-    # batches: the same sweeps again with every candidate tested in FP64,
-    # from the same state; the two forms must give the same pressures
+    # batches: the same sweeps again with every candidate chosen and tested in
+    # FP64, from the same state; the two forms must give the same pressures
     precision_cmp = None
     if descs is not None:
         p32 = [g.replica_pressure(r)[0] for r in range(len(descs))]

@@ -100,9 +100,9 @@ extern "C" {
 /* 1 = capture each sweep in a CUDA graph and replay it (default 1). */
 #define ECMC_PARAM_USE_GRAPH 12
 /* Where the chain kernel keeps the cell frames: 0 = shared memory, 1 = part of
- * them in global memory (axis chains: the disks' candidate lists, in a
- * per-warp scratch area; isotropic chains, per-phase launches: the FP64
- * coordinates), 2 = global memory (cells too large for shared memory), -1 =
+ * them in global memory (axis chains that follow their disks' candidate
+ * lists: the lists, in a per-warp scratch area; the per-phase kernels: the
+ * FP64 coordinates), 2 = global memory (cells too large for shared memory), -1 =
  * automatic (default).  The persistent sweep kernel uses 0 or 1.  Changes only
  * the speed, never the result. */
 #define ECMC_PARAM_FRAME_MODE 13
@@ -127,8 +127,11 @@ extern "C" {
  * that faults nothing; default 0). */
 #define ECMC_PARAM_WAIT_TEST 17
 /* Read-only: kernel launches per sweep of the current configuration (5 with
- * the persistent kernel; with per-phase launches 8 for axis chains whose cells
- * fit in shared memory, which build their frames themselves, and 12 else). */
+ * the persistent kernel; with per-phase launches 8 for axis chains that follow
+ * their disks' candidate lists, and 12 else).  Axis chains follow such lists
+ * where their frames fit in shared memory and a cell's chains are long enough
+ * to pay for them, which depends on the cells, n_m, ell, the boundary rule and
+ * the precision; otherwise they run by per-phase launches. */
 #define ECMC_PARAM_KERNELS_PER_SWEEP 18
 /* Start lists (Sec. 3.4 step 5): ECMC_LIST_WITH_REPL (default), every start
  * disk drawn independently among the members (the paper's correct rule);
