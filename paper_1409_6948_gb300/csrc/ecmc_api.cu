@@ -249,8 +249,8 @@ AxisShape axis_shape_for(ecmc_ctx* h, int tpc) {
 
 // Lanes per cell of the axis-chain kernel: the fewest, from 8 up, that leave
 // eight warps per SM something to do in a colour phase.  Measured on GB300, us
-// per sweep with 8 / 16 / 32 lanes: 697 / 804 / 1124 at N = 2^20, 240^2 cells;
-// 347 / 267 / 299 at N = 2^18, 120^2 cells; 741 / 458 / 322 at N = 2^16, 32^2
+// per sweep with 8 / 16 / 32 lanes: 694 / 801 / 1119 at N = 2^20, 240^2 cells;
+// 346 / 265 / 296 at N = 2^18, 120^2 cells; 739 / 458 / 318 at N = 2^16, 32^2
 // cells.  Fewer lanes lost everywhere (780 with 4 at N = 2^20).
 int choose_axis_tpc(ecmc_ctx* h) {
   if (h->tpc_param) return h->tpc_param;
@@ -353,8 +353,8 @@ int axis_layout(ecmc_ctx* h, int* used) {
   const int n_groups = (h->b.A_total + s.cpw - 1) / s.cpw;
   // candidate lists in shared memory, unless they leave room for fewer than
   // four warps per SM, or keep groups of a phase waiting that registers (16
-  // warps per SM) would admit: at N = 2^22, 484^2 cells, 8 lanes, 2641 us per
-  // sweep against 2727; with all groups resident the lists in L1 cost 3-15 %
+  // warps per SM) would admit: at N = 2^22, 484^2 cells, 8 lanes, 2610 us per
+  // sweep against 2715; with all groups resident the lists in L1 cost 3-15 %
   int fm = h->fmode_param;
   if (fm < 0) {
     const int w0 = (int)(kSmemLimit / axis_smem(s, 0));

@@ -44,10 +44,10 @@
 // fixed latencies, shared memory and instruction fetch); the FP64 pipe is 43 %
 // busy, HBM 1 %.  Measured on GB300, us per sweep, this kernel against the
 // one that searched strips of candidates at every event (ecmc_chain.cuh):
-//   N = 2^20, eta = 0.72,  240^2 cells, ell = 1.04, n_m = 2:   697 / 1140
-//   N = 2^22, eta = 0.716, 484^2 cells, ell = 1.05, n_m = 2:  2624 / 6135
-//   N = 2^16, eta = 0.708, 32^2 cells,  ell = 8,    n_m = 1:   322 / 1217
-//   N = 256,  eta = 0.70,  2^2 cells,   ell = 4,    n_m = 2:   334 / 642
+//   N = 2^20, eta = 0.72,  240^2 cells, ell = 1.04, n_m = 2:   693 / 1140
+//   N = 2^22, eta = 0.716, 484^2 cells, ell = 1.05, n_m = 2:  2602 / 6135
+//   N = 2^16, eta = 0.708, 32^2 cells,  ell = 8,    n_m = 1:   318 / 1217
+//   N = 256,  eta = 0.70,  2^2 cells,   ell = 4,    n_m = 2:   328 / 642
 // (682, 2576, 309 and 324 before every exchange between the lanes of a cell was
 // ordered by a __syncwarp.)  It loses where few legs follow in a large cell: the
 // rule is axis_pays in ecmc_api.cu.
@@ -464,6 +464,10 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
   for (;;) {
     if (starting) {
       __syncwarp();
+      if (!REJECT) {
+        if (need && active && sub == 0) f.a[em >> 1] = P;  // where the last chain ended
+        __syncwarp();
+      }
       const bool go = need && k < n_m;
       const bool refill = go && (k & (kStarts - 1)) == 0;
       if (__any_sync(FULL, refill)) {
@@ -638,9 +642,10 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
       }
       em = bj * 2 + dir;
       P = aw;
-      if (sub == 0) {
-        const int latest = f.last[bj];
-        if (REJECT) {
+      int latest = 0;
+      if (sub == 0) latest = f.last[bj];
+      if (REJECT) {
+        if (sub == 0) {
           if (n_undo < g.cap_mem) {
             UndoEntry& u = g.undo[(int64_t)c * g.undo_stride + n_undo];
             u.a = P;
@@ -650,16 +655,16 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
             atomicCAS(err, DEV_OK, DEV_CAPACITY);
           }
         }
-        const int back = n_tot + 1 - latest;  // n_tot + 1 if it never moved
-        gap = back < kLegGapMax ? back : kLegGapMax;
-        f.last[bj] = n_tot + 1;
+        ++n_undo;
       }
-      if (REJECT) ++n_undo;
+      const int back = n_tot + 1 - latest;  // n_tot + 1 if it never moved
+      gap = back < kLegGapMax ? back : kLegGapMax;
+      if (sub == 0) f.last[bj] = n_tot + 1;
     }
     if (!__any_sync(FULL, slow)) continue;
 
     // turn-backs and chain ends
-    __syncwarp();
+    if (REJECT) __syncwarp();
     if (QUAD) {
       Pnew = __shfl_sync(FULL, z, quad0);
       rnew = __shfl_sync(FULL, z, quad0 + 1);
@@ -670,7 +675,7 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
       P = is_wall && !is_end ? aw : Pnew;
       need = is_end;
       if (is_end) {
-        if (sub == 0) f.a[m] = P;
+        if (REJECT && sub == 0) f.a[m] = P;
         if (REJECT) sum_b += ch_b;
       } else {
         ++n_tot;
@@ -702,6 +707,7 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
           __ballot_sync(FULL, turned && t_em == em && dbits(t_P) == dbits(P) &&
                                   n_tot - t_tot <= kLegs);
       if (match) {
+        __syncwarp();
         unsigned mine = (match >> gshift) & GM;
         bool cyc = mine != 0;
         // the latest of the matching turn-backs: turn n lives on lane n mod TPC
@@ -738,7 +744,7 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
     }
     if (slow && n_tot - tot0 >= (int)kMaxEventsPerChain) {
       atomicCAS(err, DEV_OK, DEV_CHAIN_CAP);
-      if (!need && sub == 0) f.a[em >> 1] = P;
+      if (REJECT && !need && sub == 0) f.a[em >> 1] = P;
       need = true;
     }
     if (need && recs != nullptr && sub == 0) {
