@@ -196,7 +196,7 @@ __device__ __forceinline__ double pair_d2(const double* __restrict__ px,
   return ddx * ddx + ddy * ddy;
 }
 
-// A row of gridDim.y warps per cell of all replicas (one launch for a batch:
+// A row of gridDim.y warps per cell of all replicas (one launch for a large batch:
 // loading 96 replicas took 3.26 ms with two launches each, 1.49 ms now); lane l
 // of warp y takes members 32 y + l, then every 32 gridDim.y-th.  More than one
 // warp where the mean cell holds more than 32 disks: 45 us against 73 with one
@@ -308,7 +308,20 @@ __device__ __forceinline__ void min_dist_cell(const Geom& g, int lcell, int cap,
   if (lane == 0 && best < r2_bits) atomicMin(out, best);
 }
 
+// One replica, its geometry a kernel argument in the constant bank; read from
+// the replicas' table it cost 10 % a few sweeps after a lattice and 21 % on the
+// lattice itself (N = 2^20: 225 / 250 us and 1185 / 1440 us a call).
+template <bool HALF>
 __global__ void __launch_bounds__(256) k_min_dist_fixed(
+    const __grid_constant__ Geom g, int cap, const double* __restrict__ px,
+    const double* __restrict__ py, const uint2* __restrict__ fxy, const int* __restrict__ cnt,
+    unsigned long long* __restrict__ out) {
+  const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (c >= g.ncell) return;  // warp-uniform
+  min_dist_cell<HALF>(g, c, cap, px, py, fxy, cnt, out);
+}
+
+__global__ void __launch_bounds__(256) k_min_dist_batch(
     const Geom* __restrict__ rg, const int* __restrict__ cell_rep, int C_total, int cap,
     const double* __restrict__ px, const double* __restrict__ py, const uint2* __restrict__ fxy,
     const int* __restrict__ cnt, unsigned long long* __restrict__ out) {
@@ -454,10 +467,24 @@ void launch_min_dist(const Geom* geo, const DevBufs& b, unsigned long long* out,
   if (!fixed) return;
   const uint2* fxy = launch_fixed_point(b, 0, b.C_total, s);
   const int bs = 256;
-  const dim3 grid((unsigned)(((int64_t)b.C_total * 32 + bs - 1) / bs),
-                  warps_per_cell(b.N_total, b.C_total, b.cap));
-  k_min_dist_fixed<<<grid, bs, 0, s>>>(
-      b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], fxy, b.count[b.cur], out);
+  if (b.R > 4) {  // one launch for all of them
+    const dim3 grid((unsigned)(((int64_t)b.C_total * 32 + bs - 1) / bs),
+                    warps_per_cell(b.N_total, b.C_total, b.cap));
+    k_min_dist_batch<<<grid, bs, 0, s>>>(
+        b.rg, b.cell_rep, b.C_total, b.cap, b.px[b.cur], b.py[b.cur], fxy, b.count[b.cur], out);
+    return;
+  }
+  for (int r = 0; r < b.R; ++r) {
+    const Geom& g = geo[r];
+    const dim3 grid((unsigned)(((int64_t)g.ncell * 32 + bs - 1) / bs),
+                    warps_per_cell(g.N, g.ncell, b.cap));
+    if (g.md_path == 1)
+      k_min_dist_fixed<true><<<grid, bs, 0, s>>>(g, b.cap, b.px[b.cur], b.py[b.cur], fxy,
+                                                  b.count[b.cur], out + r);
+    else if (g.md_path == 2)
+      k_min_dist_fixed<false><<<grid, bs, 0, s>>>(g, b.cap, b.px[b.cur], b.py[b.cur], fxy,
+                                                   b.count[b.cur], out + r);
+  }
 }
 
 // The fixed-point histogram needs rcut < L / 4, int32 slot indices, a half
