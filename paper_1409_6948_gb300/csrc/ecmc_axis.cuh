@@ -34,9 +34,13 @@
 //     1/2 + g) it is sqrt(2 e) + 1.15 g > 1.4e-8 (e >= 2^-53); opposite
 //     corners of window 1 (|c| = 1/2 - g) leave 2 sqrt(g).  With g >= 2^-24
 //     both exceed the overlap and the rounding, also after s is clamped at 0.
-// A cell that holds a pair with | |db| - sigma/2 | <= 2^-24 sigma or at equal
-// coordinates along the axis (a few in 10^5 random cells; crystals aligned
-// with the axes) searches its whole frame at every event instead.
+// A member with an object at | |db| - sigma/2 | <= 2^-24 sigma, or at equal
+// coordinates along the axis in one of its windows, searches the whole frame
+// at every event instead.  (Crystals aligned with the axes; otherwise a few
+// cells in 10^5 of 18 members hold such a pair, but one in 400 of 750 members,
+// where a search takes four times a leg: with every member of the cell
+// searching, a sweep over 384 cells of 28.6 sigma that held one took 22 ms
+// instead of 6.9.)
 //
 // What bounds it: a chain is a serial dependence and the kernel's time is that
 // of its instructions -- about 22,000 warp instructions per group of four cells
@@ -120,11 +124,12 @@ constexpr int kLegGap = 22, kLegGapMax = 63;
 struct AxisFrame {
   double* a;                // along the axis; objects 0 .. nmem-1 are the members in
   double* b;                // bucket order, the frozen images follow; a[co], a[co+1]: walls
-  int* key;                 // disk id * 16 + image
+  int* key;                 // disk id * 16 + image (of members 4, 12: searches the frame)
   AxisEntry* list;          // [member * 2 + direction]
   int* last;                // 1 + number of the member's latest leg; 0: never in a chain
   unsigned short* rank;     // members in id order
   const int* zero;          // {0, 0}
+  int* irr;                 // 1 if a member searches the frame, plus 2 for every search
   unsigned short* starts;   // start draws: [kStarts] member ranks, [kStarts] signs
   AxisLeg* leg;             // history, leg n at n mod kLegs
   int nmem, nobj, co;
@@ -394,8 +399,8 @@ __device__ __noinline__ void axis_shuffled_list(int* pl, int n, int first, int64
 }
 
 // The chains of the warp's cells (Sec. 3.4 steps 5-6) and their statistics.
-// run: this lane group has a cell in this pass; irregular: it searches its
-// whole frame.
+// run: this lane group has a cell in this pass; irregular: some of its members
+// search their whole frame.
 //
 // One turn of the loop is one leg of every running chain of the warp.  Its
 // length is a chain of dependent operations: two loads, two FP64 additions,
@@ -579,7 +584,8 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
       }
     }
     if (any_irregular) __syncwarp();
-    if (irregular && active) {
+    if (irregular && active && (f.key[em >> 1] & 8)) {
+      if (sub == 0) *f.irr += 2;
       const AxisStop st = axis_search<TPC>(f.a, f.b, f.key, f.nobj, em >> 1, P, dir, sig2, sub,
                                            gmask);
       const double wall = f.a[f.co + dir];
@@ -767,10 +773,10 @@ __device__ __forceinline__ void axis_chains(const AxisFrame& f, const Geom& g, i
     s.frozen = n_frozen;
     s.walls = n_walls;
     // for every leg that was not replayed, the last legs of the chains among
-    // them: the three windows' candidates (whether or not an object is there)
-    // and, without static candidates, every other object of the frame
+    // them: the three windows' candidates (whether or not an object is there),
+    // and every other object of the frame where that was searched
     const long long legs = (long long)n_tot - n_replayed + n_chains - n_rejected;
-    s.fp64_evals = legs * (irregular ? 2 + f.nobj : 3);
+    s.fp64_evals = 3 * legs + (long long)(*f.irr >> 1) * (f.nobj - 1);
     s.chains = n_chains;
     s.n_mem = nmem;
     s.replayed = n_replayed;
@@ -800,7 +806,7 @@ struct AxisHead {
   int pre[10];  // prefix sums of their disk counts (the centre and repeats count 0)
   int cnt;      // objects of the frame
   int ovf;      // more of them than this pass allows
-  int irr;      // the cell has no static candidates
+  int irr;      // AxisFrame::irr
   int zero[2];
 };
 static_assert(sizeof(AxisHead) + 4 * kStarts <= kAxisHead, "head of a cell");
@@ -895,10 +901,11 @@ __device__ __noinline__ void axis_images(double* a, double* b, int* key, int* cn
 
 // The first objects ahead of and behind member j in its window w, decided in
 // FP64, among the sorted objects p0 .. p1 - 1: the first | the second << 16
-// (j: nobody).  Sets *irr when the cell has no static candidates.
-__device__ __noinline__ int axis_scan_exact(const double* a, const double* b,
-                                            const unsigned short* si, int p0, int p1, int j,
-                                            int w, double sigma, double sig2, int* irr) {
+// (j: nobody), and bit 31 when j has no static candidates.
+__device__ __noinline__ unsigned axis_scan_exact(const double* a, const double* b,
+                                                 const unsigned short* si, int p0, int p1, int j,
+                                                 int w, double sigma, double sig2) {
+  unsigned none = 0;
   const double half = 0.5 * sigma, guard = 0x1p-24 * sigma;
   const double aj = a[j], bj = b[j];
   int jp = j, jm = j;
@@ -907,7 +914,7 @@ __device__ __noinline__ int axis_scan_exact(const double* a, const double* b,
     const int o = si[p];
     if (o == j) continue;
     const double d = b[o] - bj, d1 = fabs(d), ao = a[o];
-    if (dlt(fabs(d1 - half), guard)) *irr = 1;
+    if (dlt(fabs(d1 - half), guard)) none = 0x80000000u;
     const bool in = w == 1 ? dlt(d1, half)
                            : (!dlt(d1, half) && lt_nn(d * d, sig2) && (dbits(d) >= 0) == (w == 2));
     if (!in) continue;
@@ -916,10 +923,10 @@ __device__ __noinline__ int axis_scan_exact(const double* a, const double* b,
     } else if (dlt(ao, aj)) {
       if (jm == j || dlt(a[jm], ao)) jm = o;
     } else {
-      *irr = 1;
+      none = 0x80000000u;
     }
   }
-  return jp | (int)((unsigned)jm << 16);
+  return (unsigned)jp | (unsigned)jm << 16 | none;
 }
 
 // Build the frames of the warp's cells of one pass: each lane group of TPC
@@ -980,6 +987,7 @@ __device__ __forceinline__ void axis_build(AxisFrame& f, AxisHead& h, unsigned c
     h.irr = 0;
   }
   f.zero = h.zero;
+  f.irr = &h.irr;
   __syncwarp();
   int T = 0;
   {
@@ -1230,9 +1238,13 @@ __device__ __forceinline__ void axis_build(AxisFrame& f, AxisHead& h, unsigned c
     if (up != kNobody) jp = si[up & pm];
     if (down != kNobody) jm = si[down & pm];
     if (amb) {
-      const int res = axis_scan_exact(f.a, f.b, si, p0, p1, j, w, sigma, sig2, &h.irr);
-      jp = res & 0xffff;
-      jm = (int)((unsigned)res >> 16);
+      const unsigned res = axis_scan_exact(f.a, f.b, si, p0, p1, j, w, sigma, sig2);
+      jp = (int)(res & 0xffffu);
+      jm = (int)(res >> 16 & 0x7fffu);
+      if (res >> 31) {
+        atomicOr(&f.key[j], 8);
+        atomicOr(&h.irr, 1);
+      }
     }
     // square roots of both (of a placeholder where nobody is there)
     const double dP = f.b[jp] - bj, dM = f.b[jm] - bj;

@@ -174,7 +174,7 @@ inline RecLayout make_layout(int cpw, int nbin, int cap_mem, int cap_obj) {
 // warp, strips across the axis, and the room for objects per frame (co) and
 // members (mp): _s when the warp's cells are worked on together (co_s per
 // cell, mp_s over all of them), _h for one cell at its packing bound alone.
-constexpr int kAxisMaxObjects = 65533;  // candidate indices have 16 bits
+constexpr int kAxisMaxObjects = 32765;  // candidate indices have 15 bits
 struct AxisShape {
   int cpw, nbin, co_s, mp_s, co_h, mp_h;
 };

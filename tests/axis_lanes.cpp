@@ -138,7 +138,7 @@ int main(int argc, char** argv) {
       axis_chains<TPC, false>(f, g, 3, c, c, go, go && h.irr != 0, cs.data(), nullptr, 1, 1,
                               &err);
     if (sub == 0 && go) {
-      irr[gi] = (unsigned long long)h.irr;
+      irr[gi] = (unsigned long long)(h.irr & 1);
       for (int q = 0; q < nc; ++q)
         hash[gi] = (hash[gi] ^ (unsigned long long)dbits(f.a[q]) ^ (f.last[q] != 0 ? 1u : 0u)) *
                    1099511628211ull;

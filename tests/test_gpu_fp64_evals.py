@@ -72,3 +72,45 @@ def test_legs_of_moving_chains():
     assert c.replayed_legs == 0 and c.fp64_evals >= 3 * legs
     assert c.fp64_evals <= 3 * legs + 0.01 * legs * 60  # (a stray irregular cell)
     g.close()
+
+
+@pytest.mark.parametrize("boundary,persistent", [(0, 1), (0, 0), (1, 1)])
+def test_only_the_pair_on_an_edge_searches(boundary, persistent):
+    # one pair of a melted configuration exactly sigma / 2 apart across the
+    # axis: the legs of these two search their frame, those of the cell's other
+    # 670 members do not
+    N, cells, (nm, ell) = 2704, 2, ((30, 3.0) if boundary == 0 else (60, 0.4))
+    L = W.box_side(N, 0.72)
+    p = oracle.make_params(N, L, 1.0, cells, cells, ell, nm, 5, boundary=boundary)
+    x, y = W.square_lattice(N, L)
+    oracle.sweeps(oracle.make_params(N, L, 1.0, 12, 12, 2.0, 10, 6), x, y, 0, 60)
+    sx, _, _ = oracle.sweep_draws(p, 1)
+    w, done = L / cells, 0
+    for o in range(N):
+        u = np.mod(x - sx, L)
+        near = np.nonzero((np.abs(np.abs(x - x[o]) - 0.5) < 2e-3) & (u // w == u[o] // w)
+                          & (np.abs(y - y[o]) < 6.0))[0]
+        for j in near:
+            old = x[o]
+            x[o] = x[j] + np.copysign(0.5, old - x[j])
+            if 0 < x[o] < L and oracle.min_dist2(L, x, y) > 1.0 - 1e-10:
+                done += 1
+                break
+            x[o] = old
+        if done:
+            break
+    assert done
+    g = P.Ecmc(N, L, 1.0, cells, cells, ell, 5)
+    g.set_param(E.PARAM_N_CHAINS, nm)
+    g.set_param(E.PARAM_BOUNDARY, boundary)
+    g.set_param(E.PARAM_PERSISTENT, persistent)
+    assert g.get_param(E.PARAM_KERNELS_PER_SWEEP) == (5 if persistent else 8)
+    g.set_positions(np.stack([x, y], 1).ravel(), t0=1)
+    g.sweep(1)
+    oracle.sweeps(p, x, y, 1, 1)
+    xy = g.positions()
+    assert np.array_equal(xy[0::2], x) and np.array_equal(xy[1::2], y)
+    c = g.counters()
+    legs = c.events + c.wall_hits + c.chains - c.replayed_legs - c.rejected_chains
+    assert 3 * legs <= c.fp64_evals < 3 * legs + 0.03 * legs * 800
+    g.close()

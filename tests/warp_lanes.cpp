@@ -21,6 +21,7 @@ struct Index {
   int x;
 };
 namespace {
+struct Token;
 constexpr unsigned kNoSync = 1;  // a switch of fibers orders nothing
 constexpr size_t kStack = 1 << 18;
 constexpr int kMost = 1024;
@@ -30,6 +31,7 @@ struct Lane {
   char* stack;
   bool done, waiting;
   unsigned mask;
+  Token* token;  // a barrier's
   int line;
   uint64_t val;
   volatile uint64_t out[32];
@@ -39,8 +41,14 @@ ucontext_t home;
 void* home_fiber;
 int current;
 const std::function<void(int)>* body;
-// one per mask of a lane group: first lane, number of lanes
-char token[kMost / 32][32][33], block_token;
+// What orders memory at a barrier, one per mask of a lane group (first lane,
+// number of lanes) and one for the block.  A lane resumes from a barrier when
+// others may be at the next one already, which must not count: two in turn.
+struct Token {
+  char at[2];
+  unsigned passed;
+};
+Token token[kMost / 32][32][33], block_token;
 
 void enter(int l) {
   (*body)(l);
@@ -59,9 +67,11 @@ void meet(unsigned mask, uint64_t val, uint64_t out[32], int line, bool orders_m
     std::printf("lane %d is not in its mask %x, line %d\n", l, mask, line);
     std::exit(2);
   }
-  char* const t = &token[current >> 5][__builtin_ctz(mask)][__builtin_popcount(mask)];
+  Token& k = token[current >> 5][__builtin_ctz(mask)][__builtin_popcount(mask)];
+  char* const t = &k.at[k.passed & 1];
   if (orders_memory) __tsan_release(t);
   me.mask = mask;
+  me.token = orders_memory ? &k : nullptr;
   me.val = val;
   me.line = line;
   me.waiting = true;
@@ -74,13 +84,14 @@ void meet(unsigned mask, uint64_t val, uint64_t out[32], int line, bool orders_m
 // mask 0: the whole block
 void block_barrier(int line) {
   Lane& me = lanes[current];
-  __tsan_release(&block_token);
+  char* const t = &block_token.at[block_token.passed & 1];
+  __tsan_release(t);
   me.mask = 0;
   me.line = line;
   me.waiting = true;
   __tsan_switch_to_fiber(home_fiber, kNoSync);
   swapcontext(&me.ctx, &home);
-  __tsan_acquire(&block_token);
+  __tsan_acquire(t);
 }
 
 bool run(const std::function<void(int)>& f, int n, bool downwards) {
@@ -122,6 +133,7 @@ bool run(const std::function<void(int)>& f, int n, bool downwards) {
           ready = ready && !w[i].done && w[i].waiting && w[i].mask == m && w[i].line == lanes[l].line;
       if (!ready) continue;
       ran = true;
+      if (lanes[l].token) ++lanes[l].token->passed;
       for (int i = 0; i < 32; ++i)
         if (m >> i & 1) {
           for (int q = 0; q < 32; ++q) w[i].out[q] = m >> q & 1 ? w[q].val : 0;
@@ -132,6 +144,7 @@ bool run(const std::function<void(int)>& f, int n, bool downwards) {
       block = block && !lanes[l].done && lanes[l].waiting && lanes[l].mask == 0;
     if (block) {
       ran = true;
+      ++block_token.passed;
       for (int l = 0; l < n; ++l) lanes[l].waiting = false;
     }
     if (!ran) {
