@@ -55,8 +55,8 @@ FUSED_ITERATIONS_CAPTURE = 1526651               # contacts + walls + chain ends
 FUSED_CAPTURES = {
     # frame mode: dram__bytes_read.sum + _write.sum, smsp__inst_executed_pipe_fp64.sum,
     # sm__pipe_fp64_cycles_active (% of active cycles)
-    1: {"dram_bytes": 35523072 + 2239488, "fp64_winst": 3459144, "fp64_pipe_pct": 42.77},
-    0: {"dram_bytes": 35169280 + 203008, "fp64_winst": 3459576, "fp64_pipe_pct": 40.81},
+    1: {"dram_bytes": 35527168 + 2220800, "fp64_winst": 3419175, "fp64_pipe_pct": 43.71},
+    0: {"dram_bytes": 35171328 + 201472, "fp64_winst": 3418447, "fp64_pipe_pct": 41.50},
 }
 FUSED_CAPTURE_FRAME_MODE = 1                     # the autotuner's choice at N = 1M
 FUSED_DRAM_BYTES_CAPTURE = FUSED_CAPTURES[1]["dram_bytes"]

@@ -249,8 +249,8 @@ AxisShape axis_shape_for(ecmc_ctx* h, int tpc) {
 
 // Lanes per cell of the axis-chain kernel: the fewest, from 8 up, that leave
 // eight warps per SM something to do in a colour phase.  Measured on GB300, us
-// per sweep with 8 / 16 / 32 lanes: 694 / 801 / 1119 at N = 2^20, 240^2 cells;
-// 346 / 265 / 296 at N = 2^18, 120^2 cells; 739 / 458 / 318 at N = 2^16, 32^2
+// per sweep with 8 / 16 / 32 lanes: 679 / 796 / 1119 at N = 2^20, 240^2 cells;
+// 333 / 263 / 297 at N = 2^18, 120^2 cells; 737 / 453 / 319 at N = 2^16, 32^2
 // cells.  Fewer lanes lost everywhere (780 with 4 at N = 2^20).
 int choose_axis_tpc(ecmc_ctx* h) {
   if (h->tpc_param) return h->tpc_param;
@@ -268,8 +268,8 @@ int choose_axis_tpc(ecmc_ctx* h) {
 // difference of the fixed costs, 0.4 m + 0.08 m s - 20 us a sweep, against the
 // gain per leg of a cell, 2.5 us and more where chains are dense or cells below
 // 24 sigma, is a fit to 300 pairs on GB300 (eta 0.1 to 0.72, sides of 12 to 35
-// sigma, 6^2 and 24^2 cells, 4 to 1500 legs a cell): the worst choice costs 4 %
-// (14 % with the candidates chosen in FP64, where both costs are higher).  us
+// sigma, 6^2 and 24^2 cells, 4 to 1500 legs a cell): the worst choice costs 6 %
+// (15 % with the candidates chosen in FP64, where both costs are higher).  us
 // per sweep, this kernel / the per-phase ones, 24^2 cells, for 4, 20, 100, 400 and
 // 1500 legs a cell:
 //   eta 0.72, side 12:  278 / 175,   318 / 405,   490 / 1614, 1167 / 5766, 3666 / 20916
@@ -353,8 +353,8 @@ int axis_layout(ecmc_ctx* h, int* used) {
   const int n_groups = (h->b.A_total + s.cpw - 1) / s.cpw;
   // candidate lists in shared memory, unless they leave room for fewer than
   // four warps per SM, or keep groups of a phase waiting that registers (16
-  // warps per SM) would admit: at N = 2^22, 484^2 cells, 8 lanes, 2610 us per
-  // sweep against 2715; with all groups resident the lists in L1 cost 3-15 %
+  // warps per SM) would admit: at N = 2^22, 484^2 cells, 8 lanes, 2586 us per
+  // sweep against 2668; with all groups resident the lists in L1 cost 3-15 %
   int fm = h->fmode_param;
   if (fm < 0) {
     const int w0 = (int)(kSmemLimit / axis_smem(s, 0));

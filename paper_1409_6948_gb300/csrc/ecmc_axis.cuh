@@ -48,13 +48,12 @@
 // fixed latencies, shared memory and instruction fetch); the FP64 pipe is 43 %
 // busy, HBM 1 %.  Measured on GB300, us per sweep, this kernel against the
 // one that searched strips of candidates at every event (ecmc_chain.cuh):
-//   N = 2^20, eta = 0.72,  240^2 cells, ell = 1.04, n_m = 2:   693 / 1140
-//   N = 2^22, eta = 0.716, 484^2 cells, ell = 1.05, n_m = 2:  2602 / 6135
-//   N = 2^16, eta = 0.708, 32^2 cells,  ell = 8,    n_m = 1:   318 / 1217
-//   N = 256,  eta = 0.70,  2^2 cells,   ell = 4,    n_m = 2:   328 / 642
-// (682, 2576, 309 and 324 before every exchange between the lanes of a cell was
-// ordered by a __syncwarp.)  It loses where few legs follow in a large cell: the
-// rule is axis_pays in ecmc_api.cu.
+//   N = 2^20, eta = 0.72,  240^2 cells, ell = 1.04, n_m = 2:   679 / 1140
+//   N = 2^22, eta = 0.716, 484^2 cells, ell = 1.05, n_m = 2:  2577 / 6135
+//   N = 2^16, eta = 0.708, 32^2 cells,  ell = 8,    n_m = 1:   319 / 1217
+//   N = 256,  eta = 0.70,  2^2 cells,   ell = 4,    n_m = 2:   302 / 642
+// It loses where few legs follow in a large cell: the rule is axis_pays in
+// ecmc_api.cu.
 #pragma once
 #include <climits>
 
